@@ -9,9 +9,9 @@
 // whose gradient at the logits is dZ = w_q (P - T) / sum w (zero for a >= nact).
 // Weights live in FP32 (master copy, Adam moments) and BF16 (what the
 // forward and backward products read); activations and gradients are FP32.
-// The products are one tiled SIMT kernel (64x64 tile, 16-deep k slices in
-// shared memory, 4x4 outputs per thread) with generic strides, so the same
-// code computes X W, dZ W^T and X^T dH.  Not in the paper: a service for
+// The products are one tiled SIMT kernel (64x64 tile, 8x8 outputs per thread,
+// k split over thread groups and CTAs) that reads either operand in either
+// direction, so the same code computes X W, dZ W^T and X^T dH.  Not in the paper: a service for
 // warm-starting the solver (Sec. 2's first-order methods start from a given
 // strategy).
 #include <cuda_bf16.h>
@@ -31,79 +31,215 @@ using namespace kps_abi;
 
 namespace {
 
-constexpr int kBM = 64, kBN = 64, kBK = 16;
+constexpr int kBM = 64, kBN = 64, kBK = 8;   // output tile of a CTA, k slice of a group
+constexpr int kPitch = kBM + 4;              // floats per k row of a staged operand
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// C(m,n) = sum_k A(m,k) B(k,n) [+ bias(n)] [relu] [* (gate(m,n) > 0)]
-// A(m,k) = A[m*sam + k*sak], B(k,n) = B[k*sbk + n*sbn], C row-major ldc.
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(256)
-gemm_kernel(int M, int N, int K, const TA *__restrict__ A, long long sam, long long sak, const TB *__restrict__ B,
-            long long sbk, long long sbn, float *__restrict__ C, long long ldc, const float *__restrict__ bias,
-            int relu, const float *__restrict__ gate, long long ldg) {
-    __shared__ float As[kBK][kBM + 4];
-    __shared__ float Bs[kBK][kBN + 4];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
-    const int tr = tid / 16, tc = tid % 16;   // 16 x 16 threads, 4 x 4 outputs each
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += kBK) {
-        // 64 x 16 elements of each operand, 4 per thread
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int e = tid + 256 * i;
-            // A tile: consecutive threads walk k when A is k-contiguous, else m
-            int am, ak;
-            if (sak == 1) { am = e / kBK; ak = e % kBK; } else { am = e % kBM; ak = e / kBM; }
-            const int gm = m0 + am, gk = k0 + ak;
-            As[ak][am] = (gm < M && gk < K) ? to_f<TA>(A[gm * sam + gk * sak]) : 0.f;
-            int bk, bn;
-            if (sbn == 1) { bk = e / kBN; bn = e % kBN; } else { bk = e % kBK; bn = e / kBK; }
-            const int gk2 = k0 + bk, gn = n0 + bn;
-            Bs[bk][bn] = (gk2 < K && gn < N) ? to_f<TB>(B[gk2 * sbk + gn * sbn]) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < kBK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][tr + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tc + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
+// 8 consecutive elements as floats (vector: 16-byte aligned).
+__device__ __forceinline__ void load8(const float *p, float *v) {
+    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void load8(const __nv_bfloat16 *p, float *v) {
+    const uint4 u = *reinterpret_cast<const uint4 *>(p);
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int m = m0 + tr + 16 * i;
+        v[2 * i] = __uint_as_float(w[i] << 16);
+        v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+
+// A thread's 8 elements of a group's [8 k][64 r] operand slice: with k
+// contiguous in memory row r = t and all 8 k, else k = t / 8 and the 8 rows
+// 8 (t % 8)...; zeros outside [0, R) x [k0, kend).
+template <bool KC, typename T>
+__device__ __forceinline__ void fetch(const T *__restrict__ A, long long ld, int r0, int R, int k0, int kend, bool vec,
+                                      int t, float *v) {
+    const int r = r0 + (KC ? t : 8 * (t & 7)), k = k0 + (KC ? 0 : t >> 3);
+    const T *p = KC ? A + (long long)r * ld + k : A + (long long)k * ld + r;
+    const bool full = KC ? (r < R && k + 8 <= kend) : (k < kend && r + 8 <= R);
+    if (full && vec) {
+        load8(p, v);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const bool in = KC ? (r < R && k + i < kend) : (k < kend && r + i < R);
+            v[i] = in ? to_f<T>(p[i]) : 0.f;
+        }
+    }
+}
+template <bool KC>
+__device__ __forceinline__ void stage(float *S, int t, const float *v) {
+    if (KC) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) S[i * kPitch + t] = v[i];
+    } else {
+        float *q = S + (t >> 3) * kPitch + 8 * (t & 7);
+        reinterpret_cast<float4 *>(q)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4 *>(q)[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+}
+
+// Where a product's value goes: bias, ReLU, gate ([gate > 0]), store.
+struct Epilogue {
+    float *C;
+    long long ldc;
+    const float *bias;
+    int relu;
+    const float *gate;
+    long long ldg;
+    __device__ __forceinline__ void put(int m, int n, float v) const {
+        if (bias) v += bias[n];
+        if (relu) v = fmaxf(v, 0.f);
+        if (gate && !(gate[(long long)m * ldg + n] > 0.f)) v = 0.f;
+        C[(long long)m * ldc + n] = v;
+    }
+};
+
+// C(m,n) = sum_k A(m,k) B(k,n), then the epilogue.  A(m,k) = A[m*lda + k] (AK)
+// or A[k*lda + m]; B(k,n) = B[n*ldb + k] (BK) or B[k*ldb + n].
+//
+// FP32 FMAs, because the operands are FP32 activations and gradients that are
+// not to be rounded: bound by the FMA pipe (4096 x 1232 x 256 is 2.6 GFLOP,
+// 35 us at 152 SMs x 128 lanes).  A thread owns 8 x 8 outputs, as packed
+// FP32x2 pairs along n: 4 shared loads of 16 bytes feed 32 packed FMAs, where
+// the 4 x 4 tile it replaces needed a load for every two FMAs.  The network's
+// products have few output tiles (256 for 4096 x 256, 80 for a 1232 x 256
+// weight gradient), so the k range is cut twice: each of KG groups of 64
+// threads takes every KG-th slice of 8 k (its own double-buffered staging and
+// named barrier; the groups' sums meet in shared memory), and blockIdx.z takes
+// a contiguous part of k when the tiles alone would leave SMs idle (partials
+// to `part`, added in order by reduce_kernel).  Both orders are fixed: results
+// are bit-reproducible.  KG = 1 without a z split adds k in ascending order.
+// Losses and gradients of a 4096-row minibatch: 1.53 ms before (64 x 64
+// tiles of 4 x 4 outputs per thread, no k split), 0.38 ms now.
+template <int KG, bool AK, bool BK, typename TA, typename TB>
+__global__ void __launch_bounds__(64 * KG, KG == 1 ? 8 : 2)
+gemm_kernel(int M, int N, int K, int kpart, const TA *__restrict__ A, long long lda, int avec,
+            const TB *__restrict__ B, long long ldb, int bvec, float *__restrict__ part, const Epilogue ep) {
+    constexpr int kBuf = kBK * kPitch;                       // one operand, one stage
+    constexpr int kRed = KG == 1 ? 0 : KG / 2 * kBM * kBN;   // sums handed over between groups
+    __shared__ __align__(16) float sh[KG * 4 * kBuf > kRed ? KG * 4 * kBuf : kRed];
+    const int t = threadIdx.x & 63, grp = threadIdx.x >> 6;
+    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
+    const int kb = blockIdx.z * kpart, kend = min(K, kb + kpart);
+    float *As = sh + grp * 4 * kBuf, *Bs = As + 2 * kBuf;
+    const int tr = t >> 3, tc = t & 7;
+    auto sync_group = [&]() {
+        if (KG == 1) __syncthreads();
+        else asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
+    };
+    float2 acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    float va[8], vb[8];
+    int k0 = kb + grp * kBK, st = 0;
+    if (k0 < kend) {
+        fetch<AK>(A, lda, m0, M, k0, kend, avec, t, va);
+        fetch<BK>(B, ldb, n0, N, k0, kend, bvec, t, vb);
+        stage<AK>(As, t, va);
+        stage<BK>(Bs, t, vb);
+    }
+    sync_group();
+    for (; k0 < kend; k0 += KG * kBK) {
+        const int kn = k0 + KG * kBK;
+        if (kn < kend) {
+            fetch<AK>(A, lda, m0, M, kn, kend, avec, t, va);
+            fetch<BK>(B, ldb, n0, N, kn, kend, bvec, t, vb);
+        }
+        const float *a = As + st * kBuf + 4 * tr, *b = Bs + st * kBuf + 4 * tc;
+#pragma unroll
+        for (int kk = 0; kk < kBK; ++kk) {
+            const float4 a0 = *reinterpret_cast<const float4 *>(a + kk * kPitch);
+            const float4 a1 = *reinterpret_cast<const float4 *>(a + kk * kPitch + 32);
+            const float4 b0 = *reinterpret_cast<const float4 *>(b + kk * kPitch);
+            const float4 b1 = *reinterpret_cast<const float4 *>(b + kk * kPitch + 32);
+            const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 br[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                                  make_float2(b1.z, b1.w)};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(make_float2(ar[i], ar[i]), br[j], acc[i][j]);
+        }
+        st ^= 1;
+        if (kn < kend) {
+            stage<AK>(As + st * kBuf, t, va);
+            stage<BK>(Bs + st * kBuf, t, vb);
+        }
+        sync_group();
+    }
+    // groups g and g + s meet pairwise, s halving: a fixed order
+#pragma unroll
+    for (int s = KG / 2; s >= 1; s >>= 1) {
+        __syncthreads();
+        if (grp >= s && grp < 2 * s) {
+            float2 *r = reinterpret_cast<float2 *>(sh) + (grp - s) * (kBM * kBN / 2) + t;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) r[64 * e] = acc[e >> 2][e & 3];
+        }
+        __syncthreads();
+        if (grp < s) {
+            const float2 *r = reinterpret_cast<const float2 *>(sh) + grp * (kBM * kBN / 2) + t;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) acc[e >> 2][e & 3] = __fadd2_rn(acc[e >> 2][e & 3], r[64 * e]);
+        }
+    }
+    if (grp != 0) return;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int m = m0 + 4 * tr + (i & 3) + 32 * (i >> 2);
         if (m >= M) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tc + 16 * j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (bias) v += bias[n];
-            if (relu) v = fmaxf(v, 0.f);
-            if (gate && !(gate[(long long)m * ldg + n] > 0.f)) v = 0.f;
-            C[(long long)m * ldc + n] = v;
+            const int n = n0 + 4 * tc + 2 * (j & 1) + 32 * (j >> 1);
+            if (part) {
+                float *q = part + ((long long)blockIdx.z * M + m) * N;
+                if (n < N) q[n] = acc[i][j].x;
+                if (n + 1 < N) q[n + 1] = acc[i][j].y;
+            } else {
+                if (n < N) ep.put(m, n, acc[i][j].x);
+                if (n + 1 < N) ep.put(m, n + 1, acc[i][j].y);
+            }
         }
     }
 }
 
-// Column sums of G [M x N] (bias gradients): out[n] = sum_m G[m, n].
-__global__ void colsum_kernel(int M, int N, const float *__restrict__ G, float *__restrict__ out) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+// The z parts of a split product added in order, then the epilogue.
+__global__ void __launch_bounds__(256) reduce_kernel(int M, int N, int nz, const float *__restrict__ part,
+                                                     const Epilogue ep) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x, mn = (long long)M * N;
+    if (i >= mn) return;
+    float v = part[i];
+    for (int z = 1; z < nz; ++z) v += part[z * mn + i];
+    ep.put((int)(i / N), (int)(i % N), v);
+}
+
+// Column sums of G [M x N] (bias gradients): the rows in gridDim.y parts, a
+// warp row of 32 columns per 8 rows of threads; the parts are added by
+// reduce_kernel (as an [1 x N] product of gridDim.y parts).
+__global__ void __launch_bounds__(256) colsum_kernel(int M, int N, int rows, const float *__restrict__ G,
+                                                     float *__restrict__ part) {
+    __shared__ float red[8][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5, n = blockIdx.x * 32 + x;
+    const int m0 = blockIdx.y * rows, m1 = min(M, m0 + rows);
     float s = 0.f;
-    for (int m = 0; m < M; ++m) s += G[(long long)m * N + n];
-    out[n] = s;
+    if (n < N)
+        for (int m = m0 + y; m < m1; m += 8) s += G[(long long)m * N + n];
+    red[y][x] = s;
+    __syncthreads();
+    if (y == 0 && n < N) {
+#pragma unroll
+        for (int i = 1; i < 8; ++i) s += red[i][x];
+        part[(long long)blockIdx.y * N + n] = s;
+    }
 }
 
 // Masked softmax of each row; with targets: per-row loss terms and dZ.
@@ -167,15 +303,31 @@ __global__ void to_bf16_kernel(long long n, const float *__restrict__ p, __nv_bf
     if (i < n) ph[i] = __float2bfloat16_rn(p[i]);
 }
 
-template <typename TA, typename TB>
-cudaError_t gemm(int M, int N, int K, const TA *A, long long sam, long long sak, const TB *B, long long sbk,
-                 long long sbn, float *C, long long ldc, const float *bias, bool relu, const float *gate,
-                 long long ldg, cudaStream_t st) {
+template <typename T>
+bool vec_ok(const T *p, long long ld) {
+    return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % (16 / (long long)sizeof(T)) == 0;
+}
+
+// Parts of k: enough CTAs for two per SM, each with at least kMinPart k.
+constexpr int kMinPart = 256, kMaxParts = 32;
+int gemm_parts(int M, int N, int K, int sms) {
+    const long long tiles = (long long)((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
+    return (int)std::max<long long>(1, std::min<long long>({2LL * sms / tiles, (long long)K / kMinPart, (long long)kMaxParts}));
+}
+
+// `part`: nz * M * N floats when nz > 1 (gemm_parts), else unused.
+template <int KG, bool AK, bool BK, typename TA, typename TB>
+cudaError_t gemm(int M, int N, int K, const TA *A, long long lda, const TB *B, long long ldb, const Epilogue &ep, int nz,
+                 float *part, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM);
+    const int slice = KG * kBK;
+    const int kpart = nz > 1 ? ((K + nz - 1) / nz + slice - 1) / slice * slice : K;
+    dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, nz);
     if (grid.y > 65535) return cudaErrorInvalidValue;
-    gemm_kernel<TA, TB><<<grid, 256, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, relu ? 1 : 0, gate,
-                                               ldg);
+    gemm_kernel<KG, AK, BK, TA, TB><<<grid, 64 * KG, 0, st>>>(M, N, K, kpart, A, lda, vec_ok(A, lda), B, ldb,
+                                                              vec_ok(B, ldb), nz > 1 ? part : nullptr, ep);
+    if (nz > 1)
+        reduce_kernel<<<(unsigned)(((long long)M * N + 255) / 256), 256, 0, st>>>(M, N, nz, part, ep);
     return cudaGetLastError();
 }
 
@@ -185,12 +337,22 @@ namespace kps_abi {
 
 cudaError_t mlp_gemm_xw(int M, int N, int K, const float *A, long long lda, const __nv_bfloat16 *W, long long ldw,
                         float *C, long long ldc, cudaStream_t st) {
-    return gemm<float, __nv_bfloat16>(M, N, K, A, lda, 1, W, ldw, 1, C, ldc, nullptr, false, nullptr, 0, st);
+    // k in ascending order: the predictor's activations are rounded to BF16
+    return gemm<1, true, false>(M, N, K, A, lda, W, ldw, Epilogue{C, ldc, nullptr, 0, nullptr, 0}, 1, nullptr, st);
 }
 
 }  // namespace kps_abi
 
 namespace {
+
+constexpr int kColParts = 64;   // row parts of a bias gradient
+
+// Floats of the largest set of split-k partial products: a product takes more than one part only while all its parts
+// are at most two tiles per SM, and a bias gradient kColParts rows.
+size_t part_floats(const kps_mlp *m) {
+    const size_t wide = std::max(m->width, m->dout);
+    return std::max((size_t)2 * m->sms * kBM * kBN, kColParts * wide);
+}
 
 kps_status ensure_cap(kps_mlp *m, int rows) {
     if (rows <= m->cap) return KPS_OK;
@@ -201,7 +363,8 @@ kps_status ensure_cap(kps_mlp *m, int rows) {
     cudaFree(m->dH1);
     cudaFree(m->dH2);
     cudaFree(m->row_loss);
-    m->H1 = m->H2 = m->Z = m->dZ = m->dH1 = m->dH2 = m->row_loss = nullptr;
+    cudaFree(m->part);
+    m->H1 = m->H2 = m->Z = m->dZ = m->dH1 = m->dH2 = m->row_loss = m->part = nullptr;
     m->cap = 0;
     const size_t r = (size_t)rows;
     cudaError_t e = cudaMalloc(&m->H1, r * m->width * 4);
@@ -211,6 +374,7 @@ kps_status ensure_cap(kps_mlp *m, int rows) {
     if (e == cudaSuccess) e = cudaMalloc(&m->dH1, r * m->width * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->dH2, r * m->width * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->row_loss, r * 4);
+    if (e == cudaSuccess) e = cudaMalloc(&m->part, part_floats(m) * 4);
     if (e != cudaSuccess) return fail(KPS_ENOMEM, "network activations");
     m->cap = rows;
     return KPS_OK;
@@ -219,14 +383,34 @@ kps_status ensure_cap(kps_mlp *m, int rows) {
 const __nv_bfloat16 *Wh(const kps_mlp *m, int l) { return m->ph + m->off[2 * l]; }
 const float *Bf(const kps_mlp *m, int l) { return m->p + m->off[2 * l + 1]; }
 
+// X W with W [K x N] as it is stored; split over k where the tiles are few.
+cudaError_t gemm_xw(kps_mlp *m, int M, int N, int K, const float *A, const __nv_bfloat16 *W, const Epilogue &ep,
+                    cudaStream_t st) {
+    return gemm<4, true, false>(M, N, K, A, K, W, N, ep, gemm_parts(M, N, K, m->sms), m->part, st);
+}
+// G W^T with W [N x K] as it is stored.
+cudaError_t gemm_gwt(kps_mlp *m, int M, int N, int K, const float *G, const __nv_bfloat16 *W, const Epilogue &ep,
+                     cudaStream_t st) {
+    return gemm<4, true, true>(M, N, K, G, K, W, K, ep, gemm_parts(M, N, K, m->sms), m->part, st);
+}
+// Weight and bias gradients of a layer: X^T G and the column sums of G.
+cudaError_t gemm_xtg(kps_mlp *m, int M, int N, int Q, const float *X, const float *G, float *dW, float *db,
+                     cudaStream_t st) {
+    cudaError_t e = gemm<4, false, false>(M, N, Q, X, M, G, N, Epilogue{dW, N, nullptr, 0, nullptr, 0},
+                                          gemm_parts(M, N, Q, m->sms), m->part, st);
+    if (e != cudaSuccess) return e;
+    const int rows = std::max(64, (Q + kColParts - 1) / kColParts), parts = (Q + rows - 1) / rows;
+    colsum_kernel<<<dim3((N + 31) / 32, parts), 256, 0, st>>>(Q, N, rows, G, m->part);
+    reduce_kernel<<<(N + 255) / 256, 256, 0, st>>>(1, N, parts, m->part, Epilogue{db, N, nullptr, 0, nullptr, 0});
+    return cudaGetLastError();
+}
+
 // Forward pass into H1, H2, Z (and P if given).
 kps_status forward(kps_mlp *m, const float *X, int Q, const int *nact, float *P, cudaStream_t st) {
     const int D = m->din, W = m->width, O = m->dout;
-    cudaError_t e = gemm<float, __nv_bfloat16>(Q, W, D, X, D, 1, Wh(m, 0), W, 1, m->H1, W, Bf(m, 0), true, nullptr, 0, st);
-    if (e == cudaSuccess)
-        e = gemm<float, __nv_bfloat16>(Q, W, W, m->H1, W, 1, Wh(m, 1), W, 1, m->H2, W, Bf(m, 1), true, nullptr, 0, st);
-    if (e == cudaSuccess)
-        e = gemm<float, __nv_bfloat16>(Q, O, W, m->H2, W, 1, Wh(m, 2), O, 1, m->Z, O, Bf(m, 2), false, nullptr, 0, st);
+    cudaError_t e = gemm_xw(m, Q, W, D, X, Wh(m, 0), Epilogue{m->H1, W, Bf(m, 0), 1, nullptr, 0}, st);
+    if (e == cudaSuccess) e = gemm_xw(m, Q, W, W, m->H1, Wh(m, 1), Epilogue{m->H2, W, Bf(m, 1), 1, nullptr, 0}, st);
+    if (e == cudaSuccess) e = gemm_xw(m, Q, O, W, m->H2, Wh(m, 2), Epilogue{m->Z, O, Bf(m, 2), 0, nullptr, 0}, st);
     if (e == cudaSuccess && P) {
         softmax_kernel<<<(Q + 127) / 128, 128, 0, st>>>(Q, O, m->Z, nact, P, nullptr, nullptr, 0.f, nullptr, nullptr);
         e = cudaGetLastError();
@@ -242,30 +426,13 @@ kps_status backward(kps_mlp *m, const float *X, int Q, const int *nact, const fl
     cudaError_t e = cudaGetLastError();
     float *g = m->g;
     // layer 3: dW3 = H2^T dZ, db3 = colsum dZ, dH2 = (dZ W3^T) * [H2 > 0]
-    if (e == cudaSuccess)
-        e = gemm<float, float>(W, O, Q, m->H2, 1, W, m->dZ, O, 1, g + m->off[4], O, nullptr, false, nullptr, 0, st);
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(O + 127) / 128, 128, 0, st>>>(Q, O, m->dZ, g + m->off[5]);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-        e = gemm<float, __nv_bfloat16>(Q, W, O, m->dZ, O, 1, Wh(m, 2), 1, O, m->dH2, W, nullptr, false, m->H2, W, st);
+    if (e == cudaSuccess) e = gemm_xtg(m, W, O, Q, m->H2, m->dZ, g + m->off[4], g + m->off[5], st);
+    if (e == cudaSuccess) e = gemm_gwt(m, Q, W, O, m->dZ, Wh(m, 2), Epilogue{m->dH2, W, nullptr, 0, m->H2, W}, st);
     // layer 2
-    if (e == cudaSuccess)
-        e = gemm<float, float>(W, W, Q, m->H1, 1, W, m->dH2, W, 1, g + m->off[2], W, nullptr, false, nullptr, 0, st);
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(W + 127) / 128, 128, 0, st>>>(Q, W, m->dH2, g + m->off[3]);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-        e = gemm<float, __nv_bfloat16>(Q, W, W, m->dH2, W, 1, Wh(m, 1), 1, W, m->dH1, W, nullptr, false, m->H1, W, st);
+    if (e == cudaSuccess) e = gemm_xtg(m, W, W, Q, m->H1, m->dH2, g + m->off[2], g + m->off[3], st);
+    if (e == cudaSuccess) e = gemm_gwt(m, Q, W, W, m->dH2, Wh(m, 1), Epilogue{m->dH1, W, nullptr, 0, m->H1, W}, st);
     // layer 1
-    if (e == cudaSuccess)
-        e = gemm<float, float>(D, W, Q, X, 1, D, m->dH1, W, 1, g + m->off[0], W, nullptr, false, nullptr, 0, st);
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(W + 127) / 128, 128, 0, st>>>(Q, W, m->dH1, g + m->off[1]);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = gemm_xtg(m, D, W, Q, X, m->dH1, g + m->off[0], g + m->off[1], st);
     if (e == cudaSuccess && loss) {
         sum_kernel<<<1, 256, 0, st>>>(Q, m->row_loss, loss);
         e = cudaGetLastError();
@@ -299,6 +466,10 @@ kps_status kps_mlp_create(int32_t din, int32_t width, int32_t dout, uint64_t see
                              dout};
     for (int i = 0; i < 6; ++i) m->off[i + 1] = m->off[i] + sz[i];
     const long long n = m->off[6];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        m->sms = 1;
     // He initialisation (normal, std sqrt(2 / fan_in)), zero biases
     std::vector<float> host(n, 0.f);
     std::mt19937_64 rng(seed);
@@ -337,7 +508,7 @@ kps_status kps_mlp_destroy(kps_mlp *m) {
     if (!m) return KPS_OK;
     for (void *q : {(void *)m->p, (void *)m->g, (void *)m->m, (void *)m->v, (void *)m->ph, (void *)m->wsum,
                     (void *)m->H1, (void *)m->H2, (void *)m->Z, (void *)m->dZ, (void *)m->dH1, (void *)m->dH2,
-                    (void *)m->row_loss})
+                    (void *)m->row_loss, (void *)m->part})
         if (q) cudaFree(q);
     delete m;
     return KPS_OK;

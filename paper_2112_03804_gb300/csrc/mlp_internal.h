@@ -15,6 +15,8 @@ struct kps_mlp {
     int cap = 0;
     float *H1 = nullptr, *H2 = nullptr, *Z = nullptr, *dZ = nullptr, *dH1 = nullptr, *dH2 = nullptr;
     float *row_loss = nullptr, *wsum = nullptr;
+    float *part = nullptr;          // partial sums of split products
+    int sms = 1;                    // of the device the network was created on
 };
 
 namespace kps_abi {
