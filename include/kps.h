@@ -180,7 +180,7 @@ kps_status kps_game_upload(kps_game *game, void *stream);
  * counts); the environment variable KPS_KERNEL = tma | tmem | vec | fast
  * forces one where it applies.  Diagnostics only: results agree within the
  * stated tolerances whichever kernel runs. */
-#define KPS_KERNEL_TMA 1      /* TMA-staged boxes, tensor-memory partials (FP32) */
+#define KPS_KERNEL_TMA 1      /* TMA-staged boxes, tensor-memory partials (all but FP64) */
 #define KPS_KERNEL_TMEM 2     /* register staging, tensor-memory partials */
 #define KPS_KERNEL_VEC 3      /* 16-byte asynchronous copies, partials through L2 */
 #define KPS_KERNEL_SCALAR 4   /* scalar staging, partials through L2 */

@@ -347,12 +347,12 @@ kps_status matvec_fast(kps_game *g, int dir, const kps::ScanParams &sp, int stor
     return KPS_OK;
 }
 
-// The TMA-staged FP32 path (kernels_tma.cu) when the game and the vectors
+// The TMA-staged path (kernels_tma.cu; FP32 and 16-bit storage) when the game and the vectors
 // allow it; *taken tells whether it ran.  KPS_KERNEL=tma|tmem|vec|fast
 // forces a path where it applies (any value other than tma disables this
 // one).
-kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t batch, cudaStream_t stream,
-                      bool *taken) {
+kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t batch, int storage,
+                      cudaStream_t stream, bool *taken) {
     *taken = false;
     const char *force = std::getenv("KPS_KERNEL");
     if (force && std::strcmp(force, "tma") != 0) return KPS_OK;
@@ -371,8 +371,7 @@ kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t
     if (g->tma_state[dir] != 1) return KPS_OK;
     *taken = true;
     g->last_kernel[dir] = KPS_KERNEL_TMA;
-    cudaError_t e = kps::launch_tma_scan(g->tma[dir].get(), static_cast<const float *>(vin),
-                                         static_cast<float *>(vout), batch, stream);
+    cudaError_t e = kps::launch_tma_scan(g->tma[dir].get(), storage, vin, vout, batch, stream);
     if (e != cudaSuccess) return cuda_fail(e, "launching the TMA-staged payoff scan");
     return KPS_OK;
 }
@@ -419,9 +418,9 @@ kps_status matvec(kps_game *g, int dir, const void *vin, void *vout, int32_t bat
     p.lam_out = dir == 0 ? l1 : l2;
     const int storage = dt == KPS_F32 ? kps::kStoreF32 : dt == KPS_F64 ? kps::kStoreF64
                         : dt == KPS_BF16 ? kps::kStoreBF16 : kps::kStoreF16;
-    if (storage == kps::kStoreF32) {
+    if (storage != kps::kStoreF64) {
         bool taken = false;
-        kps_status s2 = matvec_tma(g, dir, vin, vout, batch, stream, &taken);
+        kps_status s2 = matvec_tma(g, dir, vin, vout, batch, storage, stream, &taken);
         if (taken || s2 != KPS_OK) return s2;
     }
     if (h.max_tie <= kps::kTile) return matvec_fast(g, dir, p, storage, dt, stream);

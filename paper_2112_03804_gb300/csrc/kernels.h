@@ -169,8 +169,8 @@ int vec_multi_ctas_per_sm(int storage, int cards_per_hand, int nc, int nw);
 
 namespace kps {
 
-// TMA-staged single-game path (FP32 storage, kernels_tma.cu).  A CTA owns
-// one output sequence and 32 consecutive vectors of the batch (one per
+// TMA-staged single-game path (FP32, BF16 or FP16 storage, kernels_tma.cu).  A
+// CTA owns one output sequence, or two that share an input row, and 32 consecutive vectors of the batch (one per
 // lane); its warps scan chunks of the hand order, each a run of 16-hand
 // boxes that the tensor memory accelerator copies into shared memory.  The
 // parameter block is opaque here: built once per game and direction.
@@ -187,7 +187,7 @@ TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam
 void tma_destroy(TmaParams *p);
 // One product: out (device, [batch][n_out][hs]) from vin ([batch][n_in][hs]),
 // both 16-byte aligned.
-cudaError_t launch_tma_scan(TmaParams *p, const float *vin, float *vout, int batch, cudaStream_t stream);
+cudaError_t launch_tma_scan(TmaParams *p, int storage, const void *vin, void *vout, int batch, cudaStream_t stream);
 // Reads and clears the flag the TMA-staged kernel sets when a bounded wait
 // gives up (synchronises the device).
 cudaError_t tma_take_error(bool *set);

@@ -1,4 +1,5 @@
-// Kronecker-form payoff products, TMA-staged (sm_103a): single game, FP32.
+// Kronecker-form payoff products, TMA-staged (sm_103a): single game, FP32,
+// BF16 or FP16 storage, FP32 arithmetic.
 //
 // Mathematics (Prop. 1, Sec. 3; the fold block is the card-removal
 // compatibility of Sec. 4's eq. for C, the showdown block the strength sign
@@ -20,9 +21,10 @@
 // partners are at most 3 positions away, and the two corrections are made in
 // registers (the current 16-hand box and the previous one are held there).
 //
-// Organisation.  A CTA = one output sequence sigma and 32 consecutive
-// vectors (lane j = vector b0 + j): all its columns share their input rows,
-// payoffs and column kind (fold only, showdown only, both).  Four warps scan
+// Organisation.  A CTA = one item (an output sequence, or two that share one
+// input row, see below) and 32 consecutive vectors (lane j = vector b0 + j):
+// all its columns share their input rows, payoffs and column kind (fold only,
+// showdown only, both).  Four warps scan
 // four chunks of the hand order (chunk boundaries at 16-hand boxes that cut
 // no tie group).  For each box one lane issues cp.async.bulk.tensor copies
 // of the box's [32 vectors][16 hands] from each input row into a 64-byte
@@ -45,6 +47,23 @@
 // box and stored with one cp.async.bulk.tensor per box.  No atomics:
 // results are bit-reproducible.
 //
+// Pairs.  Where a player answers a bet by folding or calling, the two answers
+// are output sequences with the same input row y (the bet's): with b = lambda_in
+// y and one scan of b,
+//   out_call / lambda_out = S (2 Lo(b) + TieC(b) - K_F(b)),
+//   out_fold / lambda_out = F K_F(b),
+// so one item makes both: its finishing pass also gathers the totals P[c] (a
+// second table, in the idle half of warp 0's per-card table) and reads the
+// row's boxes once more (L2) for the b[h] of K_F.  A third of a game's items
+// go (43 sequences of the 1081-hand river game: 29 items), with their scans
+// and table traffic: 1024 FP32 vectors 134 -> 124 us, 250 vectors of the
+// 247-sequence tree 185 -> 168 us (single against paired items, same build).
+//
+// 16-bit storage (1000 BF16 vectors of the river game: 284 us on the
+// tensor-memory kernel, 119 us here) differs in the boxes alone.  Both storage
+// types are bound by the scan's and the finishing pass's short dependent
+// steps at eight resident warps per SM, not by memory (floor 55 / 27 us).
+//
 // Waits are bounded: a wait that gives up sets *err; the warp scans no
 // further box and finishes nothing, the CTA runs to its end without waiting
 // again (its results are not valid), waits (bounded) for its copies still in
@@ -54,6 +73,8 @@
 #include "scan_records.h"
 
 #include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -69,14 +90,17 @@
 namespace kps {
 
 constexpr int kTmaMaxExtra = 2;    // boxes of a chunk past the 256 tensor-memory columns
+constexpr int kMaxNw = 8;          // warps (chunks) of a CTA: 4, or 8 for few CTAs
 
 // Kernel arguments (__grid_constant__).
 struct alignas(128) TmaArgs {
-    CUtensorMap tin;               // input  [batch][n_in][H]  fp32, box 16 x 1 x 32, 64-byte swizzle
+    CUtensorMap tin;               // input  [batch][n_in][H], box 16 x 1 x 32, rows of a box swizzled (64 or 32 bytes)
     CUtensorMap tout;              // output [batch][n_out][hs] fp32, same box
     int H, hs, nc, k, n_out, n_in, batch, nbb, nbox, extra;
     int stall_test;                // test hook: warp 0's first box expects 16 bytes that never come
-    int bchunk[kTmaWarps + 1];     // warp k scans boxes [bchunk[k], bchunk[k+1])
+    int bchunk[kMaxNw + 1];        // warp k scans boxes [bchunk[k], bchunk[k+1])
+    int nitems;
+    const int2 *items;             // output sequence, and the fold-only sequence of its pair or -1
     const int *fcol, *scol;        // per output sequence: its fold / showdown input sequence or -1
     const float *fcoef, *scoef;    // and the payoffs
     const unsigned char *rscan;    // [nbox][kScanBlock]
@@ -88,34 +112,41 @@ struct alignas(128) TmaArgs {
 struct TmaParams {
     TmaArgs a;
     void *dev = nullptr;           // device copy of the records (scan blocks, then finishing records)
-    std::vector<unsigned char> host;
+    std::vector<unsigned char> host;   // records, the paired items, the single ones
+    size_t o_items = 0;
+    int npaired = 0, nsingle = 0;
+    int chunk4[5] = {}, chunk8[kMaxNw + 1] = {};
+    bool eight = false;            // the eight-warp shape fits
+    int extra4 = 0;                // overflow boxes of the four-warp shape
     int device = -1;
 };
 
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRingBytes = 12288;          // per warp: 3 slots of 4 KB or 6 of 2 KB
+constexpr int kRingBytes = 12288;          // per warp: 3 slots of 4 KB or 6 of 2 KB (half of it for 16-bit storage)
+constexpr int kPairMinCards = 48;          // per-card rows from which half a table holds three FP32 boxes
 constexpr int kRecRing = 6 * kScanBlock;   // per warp: one scan block per slot
-constexpr int kTmemCols = 256;             // per CTA (two CTAs per SM)
-constexpr int kHdrBytes = 1536;            // tensor-memory slot, barriers, per-warp sums
+constexpr int kTmemCols = 256;             // per four warps (two CTAs of four or one of eight per SM)
 constexpr unsigned long long kWaitNs = 2000000000ull;   // give up after 2 s
 
 enum Kind { kKindF = 1, kKindS = 2, kKindFS = 3 };
 
-// Shared memory (from a 1 KB aligned base): the four warps' rings, their
-// per-card tables (nc rows of 256 bytes), their overflow boxes of partial
+// Shared memory (from a 1 KB aligned base) with nw warps: the warps' rings,
+// their per-card tables (nc rows of 256 bytes), their overflow boxes of partial
 // results, their record rings, then the header (tensor-memory slot at +0,
-// 4 x 8 mbarriers at +16, per-warp sums [2][4][32] floats at +272).
+// nw x 8 mbarriers at +16, per-warp sums [2][nw][32] floats after them).
 __host__ __device__ inline size_t ring_off(int w) { return (size_t)w * kRingBytes; }
-__host__ __device__ inline size_t state_off(int w, int nc) { return (size_t)kTmaWarps * kRingBytes + (size_t)w * nc * 256; }
-__host__ __device__ inline size_t extra_off(int w, int nc, int extra) {
-    return state_off(kTmaWarps, nc) + (size_t)w * extra * kTmaBox * 32 * 4;
+__host__ __device__ inline size_t state_off(int nw, int w, int nc) { return (size_t)nw * kRingBytes + (size_t)w * nc * 256; }
+__host__ __device__ inline size_t extra_off(int nw, int w, int nc, int extra) {
+    return state_off(nw, nw, nc) + (size_t)w * extra * kTmaBox * 32 * 4;
 }
-__host__ __device__ inline size_t rec_off(int w, int nc, int extra) {
-    return extra_off(kTmaWarps, nc, extra) + (size_t)w * kRecRing;
+__host__ __device__ inline size_t rec_off(int nw, int w, int nc, int extra) {
+    return extra_off(nw, nw, nc, extra) + (size_t)w * kRecRing;
 }
-__host__ __device__ inline size_t hdr_off(int nc, int extra) { return rec_off(kTmaWarps, nc, extra); }
+__host__ __device__ inline size_t hdr_off(int nw, int nc, int extra) { return rec_off(nw, nw, nc, extra); }
+__host__ __device__ constexpr int sums_at(int nw) { return 16 + 64 * nw; }
+__host__ __device__ constexpr int hdr_bytes(int nw) { return sums_at(nw) + 256 * nw; }
 
 // ---- PTX wrappers ------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -240,45 +271,100 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// Byte offset of lane `row`'s 16-byte chunk q (hands 4q..4q+3) in a
-// [32][16] fp32 box written by the 64-byte swizzle: chunk bits 4-5 are
-// XORed with address bits 7-8 (the row pair).
-__device__ __forceinline__ uint32_t swz(int row, int q) {
-    return (uint32_t)(row * 64 + ((q ^ ((row >> 1) & 3)) << 4));
+// A box of [32 vectors][16 hands] in shared memory: rows of 64 (FP32) or 32
+// bytes, their 16-byte chunks swizzled by the copy (chunk bits XORed with the
+// row's: address bits 4-5 with 7-8, or bit 4 with bit 7), so that the lanes'
+// accesses of one chunk are conflict free.
+template <typename T> struct Box;
+template <> struct Box<float> {
+    static constexpr int kBytes = 2048;
+    __device__ static uint32_t at(int row, int q) { return (uint32_t)(row * 64 + ((q ^ ((row >> 1) & 3)) << 4)); }
+    // lane's 16 values as hand pairs (2i, 2i + 1)
+    __device__ static void load(const unsigned char *slot, int lane, float2 *y) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(slot + at(lane, q));
+            y[2 * q] = make_float2(v.x, v.y);
+            y[2 * q + 1] = make_float2(v.z, v.w);
+        }
+    }
+    __device__ static void store(unsigned char *slot, int lane, const float2 *o) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<float4 *>(slot + at(lane, q)) =
+                make_float4(o[2 * q].x, o[2 * q].y, o[2 * q + 1].x, o[2 * q + 1].y);
+    }
+};
+__device__ __forceinline__ float2 widen(uint32_t w, __nv_bfloat16) {
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
+__device__ __forceinline__ float2 widen(uint32_t w, __half) {
+    return __half22float2(*reinterpret_cast<const __half2 *>(&w));
+}
+__device__ __forceinline__ uint32_t narrow(float2 v, __nv_bfloat16) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+__device__ __forceinline__ uint32_t narrow(float2 v, __half) {
+    const __half2 h = __floats2half2_rn(v.x, v.y);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+template <typename T> struct Box {
+    static constexpr int kBytes = 1024;
+    __device__ static uint32_t at(int row, int q) { return (uint32_t)(row * 32 + ((q ^ ((row >> 2) & 1)) << 4)); }
+    __device__ static void load(const unsigned char *slot, int lane, float2 *y) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(slot + at(lane, q));
+            y[4 * q] = widen(v.x, T());
+            y[4 * q + 1] = widen(v.y, T());
+            y[4 * q + 2] = widen(v.z, T());
+            y[4 * q + 3] = widen(v.w, T());
+        }
+    }
+    __device__ static void store(unsigned char *slot, int lane, const float2 *o) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            *reinterpret_cast<uint4 *>(slot + at(lane, q)) =
+                make_uint4(narrow(o[4 * q], T()), narrow(o[4 * q + 1], T()), narrow(o[4 * q + 2], T()),
+                           narrow(o[4 * q + 3], T()));
+    }
+};
 
 // The CTA's column set, its warp's chunk and its shared-memory regions.
 struct Ctx {
     unsigned char *sm;
     int lane, warp;
     int bb, sigma, rf, rs;
-    float F, S;
+    int sigma2;                // fold-only sequence of a pair, or -1
+    float F, S;                // a pair's F: sigma2's
     int b0, nb;                // first box of the chunk, boxes in it
     uint32_t tmem;             // the warp's tensor-memory lanes, column 0
     bool ok;                   // no wait gave up
 };
 
-// Scan and combination of one column kind; returns this warp's C.
-template <int KIND, int K2>
+// Scan and combination of one column kind; returns this warp's C.  A
+// showdown-only column is scanned with S = 1 (finishing multiplies by S).
+template <typename T, int KIND, int K2, int NW>
 __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
     constexpr bool HF = (KIND & kKindF) != 0, HS = (KIND & kKindS) != 0, FS = KIND == kKindFS;
     constexpr int NS = FS ? 3 : 6;                    // ring slots
-    constexpr int SLOT = FS ? 4096 : 2048;            // bytes per slot
+    constexpr int BB = Box<T>::kBytes, SLOT = FS ? 2 * BB : BB;   // bytes per box, per slot
     const int lane = c.lane, warp = c.warp, nc = P.nc;
     unsigned char *ring = c.sm + ring_off(warp);
     const uint32_t ring_s = smem_u32(ring);
-    unsigned char *hdr = c.sm + hdr_off(nc, P.extra);
+    unsigned char *hdr = c.sm + hdr_off(NW, nc, P.extra);
     const uint32_t bar0 = smem_u32(hdr + 16) + 8u * 8u * (uint32_t)warp;
-    unsigned char *rring = c.sm + rec_off(warp, nc, P.extra);
+    unsigned char *rring = c.sm + rec_off(NW, warp, nc, P.extra);
     const uint32_t rring_s = smem_u32(rring);
     // per-card table of the chunk, [card][lane]: float2 {b mass, w total}
     // for columns of both kinds (rows of 256 bytes, row offset 2 * off),
     // one float otherwise (rows of 128 bytes, offset off)
-    unsigned char *stb = c.sm + state_off(warp, nc);
+    unsigned char *stb = c.sm + state_off(NW, warp, nc);
     unsigned char *lb = stb + (FS ? 8 : 4) * lane;
-    float *xpart = reinterpret_cast<float *>(c.sm + extra_off(warp, nc, P.extra));
-    float *sums = reinterpret_cast<float *>(hdr + 272);
-    const float F = c.F, S = c.S, S2 = 2.f * c.S;
+    float *xpart = reinterpret_cast<float *>(c.sm + extra_off(NW, warp, nc, P.extra));
+    float *sums = reinterpret_cast<float *>(hdr + sums_at(NW));
+    const float F = c.F, S = FS ? c.S : 1.f, S2 = 2.f * S;
     const int nb = c.nb;
     const int z0 = 32 * c.bb;
     auto row = [&](uint32_t off) -> unsigned char * { return lb + (FS ? 2 * off : off); };
@@ -292,7 +378,7 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
         const int x = kTmaBox * (c.b0 + m);
         mbar_expect_tx(bar, (uint32_t)(SLOT + kScanBlock) + (P.stall_test && m == 0 && warp == 0 ? 16u : 0u));
         if (HF) tma_load3(dst, &P.tin, x, c.rf, z0, bar);
-        if (HS) tma_load3(dst + (HF ? 2048u : 0u), &P.tin, x, c.rs, z0, bar);
+        if (HS) tma_load3(dst + (HF ? (uint32_t)BB : 0u), &P.tin, x, c.rs, z0, bar);
         bulk_load(rring_s + (uint32_t)(sl * kScanBlock), P.rscan + (size_t)(c.b0 + m) * kScanBlock, kScanBlock, bar);
     };
     if (lane == 0) {
@@ -338,23 +424,8 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
         const unsigned char *slot = ring + sl * SLOT;
         // the box's inputs as hand pairs (2i, 2i+1)
         float2 yf[8], ys[8];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (HF) {
-                const float4 v = *reinterpret_cast<const float4 *>(slot + swz(lane, q));
-                yf[2 * q] = make_float2(v.x, v.y);
-                yf[2 * q + 1] = make_float2(v.z, v.w);
-            } else {
-                yf[2 * q] = yf[2 * q + 1] = make_float2(0.f, 0.f);
-            }
-            if (HS) {
-                const float4 v = *reinterpret_cast<const float4 *>(slot + (HF ? 2048 : 0) + swz(lane, q));
-                ys[2 * q] = make_float2(v.x, v.y);
-                ys[2 * q + 1] = make_float2(v.z, v.w);
-            } else {
-                ys[2 * q] = ys[2 * q + 1] = make_float2(0.f, 0.f);
-            }
-        }
+        if (HF) Box<T>::load(slot, lane, yf);
+        if (HS) Box<T>::load(slot + (HF ? BB : 0), lane, ys);
         // the box's records: the next pair's are read before this pair's
         // per-card stores (program order keeps them ahead)
         const unsigned char *rs = rring + sl * kScanBlock;
@@ -424,8 +495,8 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
                 const float gA = G2, gB = fmaf(2.f, bb.x, G2);
                 G2 = fmaf(2.f, bb.y, gB);
                 const float2 t = fma2(make_float2(-2.f, -2.f), make_float2(cs1, cs2), make_float2(gA, gB));
-                p[k] = fma2(S2v, t, K2 == 2 ? ww : make_float2(0.f, 0.f));
-                if (!HF && K2 == 2) p[k] = fma2(nS2, bb, p[k]);   // showdown only: w = -S b
+                if (HF) p[k] = fma2(S2v, t, K2 == 2 ? ww : make_float2(0.f, 0.f));
+                else p[k] = K2 == 2 ? fma2(nS2, bb, t) : t;   // showdown only: S = 1, w = -b
             } else {
                 p[k] = K2 == 2 ? ww : make_float2(0.f, 0.f);
             }
@@ -497,18 +568,18 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
     } else {
         tot = -S * (0.5f * G2);
     }
-    sums[(0 * kTmaWarps + warp) * 32 + lane] = 0.5f * G2;
-    sums[(1 * kTmaWarps + warp) * 32 + lane] = tot;
+    sums[(0 * NW + warp) * 32 + lane] = 0.5f * G2;
+    sums[(1 * NW + warp) * 32 + lane] = tot;
     __syncthreads();
 
     // ---- combination: -Q_k[c] with Q_k[c] = Pall[c] + 2 S (mass of card c
     // in chunks < k), [card][lane] floats at the start of warp k's ring (free
     // now: every copy in has been consumed)
-    for (int q = warp; q < nc; q += kTmaWarps) {
-        float rr[kTmaWarps], pw[kTmaWarps];
+    for (int q = warp; q < nc; q += NW) {
+        float rr[NW], pw[NW];
 #pragma unroll
-        for (int k = 0; k < kTmaWarps; ++k) {
-            const unsigned char *sk = c.sm + state_off(k, nc);
+        for (int k = 0; k < NW; ++k) {
+            const unsigned char *sk = c.sm + state_off(NW, k, nc);
             if (FS) {
                 const float2 v = reinterpret_cast<const float2 *>(sk)[q * 32 + lane];
                 rr[k] = v.x;
@@ -519,46 +590,84 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
                 pw[k] = HS ? -S * v : v;
             }
         }
-        const float pall = (pw[0] + pw[1]) + (pw[2] + pw[3]);
+        const float pall = NW == 4 ? (pw[0] + pw[1]) + (pw[2] + pw[3])
+                                   : ((pw[0] + pw[1]) + (pw[2] + pw[3])) + ((pw[4 % NW] + pw[5 % NW]) + (pw[6 % NW] + pw[7 % NW]));
         float run = 0.f;
 #pragma unroll
-        for (int k = 0; k < kTmaWarps; ++k) {
+        for (int k = 0; k < NW; ++k) {
             reinterpret_cast<float *>(c.sm + ring_off(k))[q * 32 + lane] = -(pall + S2 * run);
             run += rr[k];
         }
+        // a pair's fold side: -P of b, past warp 0's per-card table
+        if (HS && !HF && c.sigma2 >= 0)
+            reinterpret_cast<float *>(c.sm + state_off(NW, 0, nc) + (size_t)nc * 128)[q * 32 + lane] = pall;
     }
     float Cw;
     {
-        float T = 0.f, gb = 0.f;
+        float tall = 0.f, gb = 0.f;
 #pragma unroll
-        for (int k = 0; k < kTmaWarps; ++k) {
-            T += sums[(1 * kTmaWarps + k) * 32 + lane];
-            if (k < warp) gb += sums[(0 * kTmaWarps + k) * 32 + lane];
+        for (int k = 0; k < NW; ++k) {
+            tall += sums[(1 * NW + k) * 32 + lane];
+            if (k < warp) gb += sums[(0 * NW + k) * 32 + lane];
         }
-        Cw = T + S2 * gb;
+        Cw = tall + S2 * gb;
     }
     __syncthreads();
 
     return Cw;
 }
 
-// Finishing pass (the same for every column kind): out = lambda_out
+// Finishing pass (the same for every column kind): out = scale lambda_out
 // ((partial + C) - (Q[c1] + Q[c2])), staged in swizzled boxes (the rest of the
-// ring, 2 KB each) and stored by TMA.  A box's finishing records (256 bytes)
-// are copied one box ahead by cp.async into two buffers in the warp's record
-// ring (idle after the scan).  A warp whose scan gave up finishes nothing: a
-// copy into its ring may still be in flight.
-template <int K2>
-__device__ __forceinline__ void tma_finish(const TmaArgs &P, const Ctx &c, float Cw) {
+// ring) and stored by TMA; scale is S for showdown-only columns, else 1.  A
+// box's finishing records (256 bytes) are copied one box ahead by cp.async
+// into two buffers in the warp's record ring (idle after the scan).  PAIR: the
+// fold side too, F lambda_out (Tot + b - (P[c1] + P[c2])), the row's boxes
+// copied one box ahead into two buffers in the warp's own (idle) per-card
+// table, whose rest is one more staging slot.  (Copied by the lanes, with
+// cp.async, a 1024-vector FP32 launch takes 6 % longer.)  A warp whose scan gave
+// up finishes nothing: a copy into its ring may still be in flight.
+template <typename T, int K2, int NW, bool PAIR>
+__device__ __forceinline__ void tma_finish(const TmaArgs &P, Ctx &c, float Cw, float scale) {
     if (!c.ok) return;
+    constexpr int BB = Box<T>::kBytes;
     const int lane = c.lane, nc = P.nc, nb = c.nb, z0 = 32 * c.bb;
     unsigned char *ring = c.sm + ring_off(c.warp);
-    const float *xpart = reinterpret_cast<const float *>(c.sm + extra_off(c.warp, nc, P.extra));
+    const float *xpart = reinterpret_cast<const float *>(c.sm + extra_off(NW, c.warp, nc, P.extra));
     const unsigned char *qb = ring + 4 * lane;
     const int qbytes = (nc * 128 + 1023) & ~1023;
-    const int nbuf = (kRingBytes - qbytes) / 2048;
-    unsigned char *frb = c.sm + rec_off(c.warp, nc, P.extra);
+    const int nring = min((kRingBytes - qbytes) / BB, 5), nbuf = nring + (PAIR ? 1 : 0);   // staging slots
+    unsigned char *frb = c.sm + rec_off(NW, c.warp, nc, P.extra);
     const uint32_t frb_s = smem_u32(frb);
+    // pairs: -P table, input boxes and a staging slot, their barriers (the
+    // ring's last two), Tot
+    const unsigned char *fb = c.sm + state_off(NW, 0, nc) + (size_t)nc * 128 + 4 * lane;
+    unsigned char *yb = c.sm + ((state_off(NW, c.warp, nc) + 1023) & ~(size_t)1023), *xst = yb + 2 * BB;
+    const uint32_t ybar = smem_u32(c.sm + hdr_off(NW, nc, P.extra) + 16) + 8u * (8u * (uint32_t)c.warp + 6u);
+    float Tb = 0.f;
+    if (PAIR) {
+        const float *sums = reinterpret_cast<const float *>(c.sm + hdr_off(NW, nc, P.extra) + sums_at(NW));
+#pragma unroll
+        for (int k = 0; k < NW; ++k) Tb += sums[(0 * NW + k) * 32 + lane];
+    }
+    const float2 F2 = make_float2(c.F, c.F), S2 = make_float2(scale, scale);
+    int ny = 0;                   // lane 0: boxes of the row copied
+    auto fetch_y = [&](int m) {   // lane 0: box m of the row
+        ny = m + 1;
+        const uint32_t bar = ybar + 8u * (uint32_t)(m & 1);
+        mbar_expect_tx(bar, BB);
+        tma_load3(smem_u32(yb) + (uint32_t)((m & 1) * BB), &P.tin, kTmaBox * (c.b0 + m), c.rs, z0, bar);
+    };
+    if (PAIR) {
+        if (lane == 0) {
+            mbar_init(ybar, 1);
+            mbar_init(ybar + 8u, 1);
+            fence_barrier_init();
+            fence_proxy_async();
+            if (nb > 0) fetch_y(0);
+        }
+        __syncwarp();
+    }
     auto fetch_fin = [&](int m) {
         if (m < nb && lane < 16)
             cp16(frb_s + (uint32_t)((m & 1) * 256 + 16 * lane),
@@ -575,12 +684,42 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, const Ctx &c, float
             for (int i = 0; i < 16; ++i) r[i] = xp[i * 32 + lane];
         }
     };
+    int nst = 0;   // boxes staged
+    auto put = [&](int m, int sigma, const float2 *o) {
+        const int sl = nst % nbuf;
+        unsigned char *buf = PAIR && sl == nring ? xst : ring + qbytes + sl * BB;
+        if (nst >= nbuf) {
+            if (lane == 0) bulk_wait_read_n(nbuf - 1);
+            __syncwarp();
+        }
+        ++nst;
+        Box<T>::store(buf, lane, o);
+        fence_proxy_async();
+        // every lane has staged its outputs
+        __syncwarp();
+        if (lane == 0) {
+            tma_store3(&P.tout, kTmaBox * (c.b0 + m), sigma, z0, smem_u32(buf));
+            bulk_commit();
+        }
+    };
     // box m of the chunk: its partials in pc, box m + 1's loaded into pn
     // (the two arrays alternate, so no copy between boxes)
     auto box = [&](int m, const float *pc, float *pn) {
         if (m + 1 < nb) load_box(m + 1, pn);
         fetch_fin(m + 1);
         cp_wait<1>();   // this lane's copy of box m's records
+        float2 y[8];
+        if (PAIR) {
+            if (lane == 0 && m + 1 < nb && c.ok) {
+                fence_proxy_async();   // box m - 1's values were read before its staging barrier
+                fetch_y(m + 1);
+            }
+            if (c.ok) {
+                const uint32_t bar = ybar + 8u * (uint32_t)(m & 1), par = (uint32_t)((m >> 1) & 1);
+                c.ok = __all_sync(kFull, mbar_try(bar, par) || mbar_wait(bar, par));
+            }
+            Box<T>::load(yb + (m & 1) * BB, lane, y);
+        }
         __syncwarp();
         const TmaFinRec *fr = reinterpret_cast<const TmaFinRec *>(frb + (m & 1) * 256);
         float2 o[8];
@@ -593,27 +732,22 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, const Ctx &c, float
             if (K2 == 2)
                 nq = add2(nq, make_float2(*reinterpret_cast<const float *>(qb + r.ob1),
                                           *reinterpret_cast<const float *>(qb + r.ob2)));
-            o[i / 2] = mul2(make_float2(r.lout1, r.lout2),
-                            add2(add2(make_float2(pc[i], pc[i + 1]), make_float2(Cw, Cw)), nq));
+            const float2 lo = make_float2(r.lout1, r.lout2);
+            o[i / 2] = mul2(mul2(S2, lo), add2(add2(make_float2(pc[i], pc[i + 1]), make_float2(Cw, Cw)), nq));
+            if (PAIR) {
+                float2 np = make_float2(*reinterpret_cast<const float *>(fb + r.oa1),
+                                        *reinterpret_cast<const float *>(fb + r.oa2));
+                float2 b = make_float2(Tb, Tb);
+                if (K2 == 2) {
+                    np = add2(np, make_float2(*reinterpret_cast<const float *>(fb + r.ob1),
+                                              *reinterpret_cast<const float *>(fb + r.ob2)));
+                    b = fma2(make_float2(r.lin1, r.lin2), y[i / 2], b);
+                }
+                y[i / 2] = mul2(mul2(F2, lo), add2(b, np));
+            }
         }
-        const int ob = m % nbuf;
-        unsigned char *buf = ring + qbytes + ob * 2048;
-        if (m >= nbuf) {
-            if (lane == 0) bulk_wait_read_n(nbuf - 1);
-            __syncwarp();
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<float4 *>(buf + swz(lane, q)) =
-                make_float4(o[2 * q].x, o[2 * q].y, o[2 * q + 1].x, o[2 * q + 1].y);
-        fence_proxy_async();
-        // every lane has read box m's records (their buffer is refilled
-        // with box m + 2 in the next box) and staged its outputs
-        __syncwarp();
-        if (lane == 0) {
-            tma_store3(&P.tout, kTmaBox * (c.b0 + m), c.sigma, z0, smem_u32(buf));
-            bulk_commit();
-        }
+        put(m, c.sigma, o);
+        if (PAIR) put(m, c.sigma2, y);
         if (m + 1 < nb) tm_wait_ld16(pn);
     };
     fetch_fin(0);
@@ -626,12 +760,18 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, const Ctx &c, float
         if (m + 1 < nb) box(m + 1, nxt, cur);
     }
     cp_wait<0>();
-    if (lane == 0) bulk_wait_read<0>();
+    if (lane == 0) {
+        bulk_wait_read<0>();
+        // a wait gave up: the row's last two copies may be in flight
+        if (PAIR && !c.ok)
+            for (int m = max(0, ny - 2); m < ny; ++m)
+                if (!mbar_wait(ybar + 8u * (uint32_t)(m & 1), (uint32_t)((m >> 1) & 1))) break;
+    }
     __syncwarp();
 }
 
-template <int K2>
-__global__ void __launch_bounds__(128, 2) tma_scan_kernel(const __grid_constant__ TmaArgs P) {
+template <typename T, int K2, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(const __grid_constant__ TmaArgs P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled boxes need 1 KB alignment (one KB of slack is allocated)
     unsigned char *sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -639,8 +779,10 @@ __global__ void __launch_bounds__(128, 2) tma_scan_kernel(const __grid_constant_
     c.sm = sm;
     c.lane = threadIdx.x & 31;
     c.warp = threadIdx.x >> 5;
-    c.bb = blockIdx.x / P.n_out;
-    c.sigma = blockIdx.x - c.bb * P.n_out;
+    c.bb = blockIdx.x / P.nitems;
+    const int2 item = P.items[blockIdx.x - c.bb * P.nitems];
+    c.sigma = item.x;
+    c.sigma2 = item.y;
     c.rf = P.fcol[c.sigma];
     c.rs = P.scol[c.sigma];
     c.F = c.rf >= 0 ? P.fcoef[c.sigma] : 0.f;
@@ -648,24 +790,29 @@ __global__ void __launch_bounds__(128, 2) tma_scan_kernel(const __grid_constant_
     c.b0 = P.bchunk[c.warp];
     c.nb = P.bchunk[c.warp + 1] - c.b0;
     c.ok = true;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + hdr_off(P.nc, P.extra));
-    if (c.warp == 0) tm_alloc(smem_u32(tslot), kTmemCols);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + hdr_off(NW, P.nc, P.extra));
+    if (c.warp == 0) tm_alloc(smem_u32(tslot), NW * 64);
     tm_fence_before();
     __syncthreads();
     tm_fence_after();
     const uint32_t tbase = *tslot;
-    c.tmem = tbase + ((uint32_t)(32 * c.warp) << 16);
+    c.tmem = tbase + ((uint32_t)(32 * (c.warp & 3)) << 16) + (uint32_t)(kTmemCols * (c.warp >> 2));
     const int kind = (c.rf >= 0 ? kKindF : 0) | (c.rs >= 0 ? kKindS : 0);
     float Cw;
-    if (kind == kKindFS) Cw = tma_scan<kKindFS, K2>(P, c);
-    else if (kind == kKindF) Cw = tma_scan<kKindF, K2>(P, c);
-    else Cw = tma_scan<kKindS, K2>(P, c);
-    tma_finish<K2>(P, c, Cw);
+    if (kind == kKindFS) Cw = tma_scan<T, kKindFS, K2, NW>(P, c);
+    else if (kind == kKindF) Cw = tma_scan<T, kKindF, K2, NW>(P, c);
+    else Cw = tma_scan<T, kKindS, K2, NW>(P, c);
+    if (NW == 4 && c.sigma2 >= 0) {   // eight warps: items are not paired
+        c.F = P.fcoef[c.sigma2];
+        tma_finish<T, K2, NW, true>(P, c, Cw, c.S);
+    } else {
+        tma_finish<T, K2, NW, false>(P, c, Cw, kind == kKindS ? c.S : 1.f);
+    }
     if (!c.ok && c.lane == 0) atomicExch(P.err, 1u);
     tm_fence_before();
     __syncthreads();
     tm_fence_after();
-    if (c.warp == 0) tm_dealloc(tbase, kTmemCols);
+    if (c.warp == 0) tm_dealloc(tbase, NW * 64);
 }
 
 // ---- host ------------------------------------------------------------------
@@ -688,25 +835,36 @@ EncodeFn encode_fn(cudaError_t *err) {
     return fn;
 }
 
-cudaError_t encode3(CUtensorMap *map, const void *base, int x, int y, int z, int pitch) {
+cudaError_t encode3(CUtensorMap *map, int storage, const void *base, int x, int y, int z, int pitch) {
     cudaError_t e;
     EncodeFn fn = encode_fn(&e);
     if (!fn) return e;
+    const bool f32 = storage == kStoreF32;
+    const cuuint64_t es = f32 ? 4 : 2;
     const cuuint64_t dims[3] = {(cuuint64_t)x, (cuuint64_t)y, (cuuint64_t)z};
-    const cuuint64_t strides[2] = {(cuuint64_t)pitch * 4, (cuuint64_t)pitch * 4 * (cuuint64_t)y};
+    const cuuint64_t strides[2] = {(cuuint64_t)pitch * es, (cuuint64_t)pitch * es * (cuuint64_t)y};
     const cuuint32_t box[3] = {(cuuint32_t)kTmaBox, 1, 32};
     const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = fn(map,
+                          f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                          : storage == kStoreBF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+                          3, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          f32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 __device__ unsigned int g_tma_err;
 
+template <typename T>
+auto pick(bool one, int nw) {
+    return one ? (nw == 4 ? tma_scan_kernel<T, 1, 4> : tma_scan_kernel<T, 1, 8>)
+               : (nw == 4 ? tma_scan_kernel<T, 2, 4> : tma_scan_kernel<T, 2, 8>);
+}
+
 }  // namespace
 
-static size_t tma_smem_bytes(int nc, int extra) { return hdr_off(nc, extra) + kHdrBytes + 1024; }
+static size_t tma_smem_bytes(int nw, int nc, int extra) { return hdr_off(nw, nc, extra) + hdr_bytes(nw) + 1024; }
 
 // Chunks, records and eligibility of one direction; fills p.a (but the
 // tensor maps, pointers and batch) and p.host.  Empty string on success.
@@ -720,8 +878,25 @@ static std::string tma_prepare(const HostGame &h, const double *lam_in, const do
     A.nc = r.nc;
     A.k = r.k;
     A.nbox = r.nbox;
-    A.extra = r.extra;
-    for (int k = 0; k <= kTmaWarps; ++k) A.bchunk[k] = r.bchunk[k];
+    for (int k = 0; k <= kTmaWarps; ++k) p.chunk4[k] = r.bchunk[k];
+    // eight chunks: each cut in two at the box boundary nearest its middle that
+    // cuts no tie group
+    auto clean = [&](int bx) { return bx <= 0 || bx >= r.nbox || 16 * bx >= r.H || h.group_lo[16 * bx] == 16 * bx; };
+    p.eight = true;
+    for (int k = 0; k < kTmaWarps; ++k) {
+        const int lo = r.bchunk[k], hi = r.bchunk[k + 1], mid = (lo + hi) / 2;
+        int cut = -1;
+        for (int d = 0; d <= hi - lo && cut < 0; ++d) {
+            if (mid - d >= lo && clean(mid - d)) cut = mid - d;
+            else if (mid + d <= hi && clean(mid + d)) cut = mid + d;
+        }
+        p.chunk8[2 * k] = lo;
+        p.chunk8[2 * k + 1] = cut;
+        p.eight = p.eight && cut >= 0 && cut - lo <= 16 && hi - cut <= 16;
+    }
+    p.chunk8[2 * kTmaWarps] = r.nbox;
+    p.eight = p.eight && tma_smem_bytes(kMaxNw, r.nc, 0) <= (size_t)max_dyn_smem();
+    p.extra4 = r.extra;
     p.host = std::move(r.bytes);
     return "";
 }
@@ -744,9 +919,27 @@ TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam
     } catch (const std::bad_alloc &) {
         w = "host allocation";
     }
-    for (int r = 0; r < n_out && w.empty(); ++r)
+    // items: a fold-only sequence goes with the showdown-only one of its input row
+    std::vector<int2> items;
+    std::vector<int> mate(n_out, -1);
+    std::vector<char> taken(n_out, 0);
+    for (int r = 0; r < n_out && w.empty(); ++r) {
         if (hfcol[r] < 0 && hscol[r] < 0) w = "an output sequence without terminals";
-    if (w.empty() && std::max<size_t>(tma_smem_bytes(p->a.nc, p->a.extra), 80 * 1024) > (size_t)max_dyn_smem())
+        for (int q = 0; q < n_out && hfcol[r] < 0 && mate[r] < 0 && p->a.nc >= kPairMinCards; ++q)
+            if (hscol[q] < 0 && hfcol[q] == hscol[r] && !taken[q]) {
+                mate[r] = q;
+                taken[q] = 1;
+            }
+    }
+    for (int r = 0; r < n_out; ++r)
+        if (!taken[r]) items.push_back(make_int2(r, mate[r]));
+    p->npaired = (int)items.size();
+    p->nsingle = n_out;
+    for (int r = 0; r < n_out; ++r) items.push_back(make_int2(r, -1));
+    p->o_items = (p->host.size() + 15) / 16 * 16;
+    p->host.resize(p->o_items + sizeof(int2) * items.size());
+    if (!items.empty()) std::memcpy(p->host.data() + p->o_items, items.data(), sizeof(int2) * items.size());
+    if (w.empty() && std::max<size_t>(tma_smem_bytes(kTmaWarps, p->a.nc, p->extra4), 80 * 1024) > (size_t)max_dyn_smem())
         w = "shared memory";
     if (!w.empty()) {
         delete p;
@@ -777,7 +970,7 @@ void tma_destroy(TmaParams *p) {
     delete p;
 }
 
-cudaError_t launch_tma_scan(TmaParams *pp, const float *vin, float *vout, int batch, cudaStream_t stream) {
+cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *vout, int batch, cudaStream_t stream) {
     TmaParams &p = *pp;
     TmaArgs &A = p.a;
     cudaError_t e;
@@ -805,19 +998,44 @@ cudaError_t launch_tma_scan(TmaParams *pp, const float *vin, float *vout, int ba
     // so that its bounded wait gives up and sets the error flag
     const char *st = std::getenv("KPS_TEST_STALL_WAIT");
     A.stall_test = st && std::atoi(st) > 0 ? 1 : 0;
-    e = encode3(&A.tin, vin, A.H, A.n_in, batch, A.hs);
-    if (e == cudaSuccess) e = encode3(&A.tout, vout, A.hs, A.n_out, batch, A.hs);
+    e = encode3(&A.tin, storage, vin, A.H, A.n_in, batch, A.hs);
+    if (e == cudaSuccess) e = encode3(&A.tout, storage, vout, A.hs, A.n_out, batch, A.hs);
     if (e != cudaSuccess) return e;
+    int dev = 0, sms = 1;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // Shape.  Eight warps (half as long a scan per warp) while every single item
+    // has an SM to itself: 1 FP32 vector 26.6 -> 20.5 us, 96 vectors 28.8 ->
+    // 22.6 us.  Else four warps, and pairs where they save a wave of two CTAs
+    // per SM, since a paired item alone takes longer (41 against 35 us a wave):
+    // 192 vectors (0.85 / 0.57 waves) single 34.9, paired 41.0 us; 256 (1.13 /
+    // 0.76) 54.0, 41.2; 384 (1.70 / 1.14) 60.4, 67.6; 512 (2.26 / 1.53) 80.6, 72.0.
+    const long long single = (long long)p.nsingle * A.nbb, paired = (long long)p.npaired * A.nbb, slots = 2 * sms;
+    const int nw = p.eight && single <= sms ? 8 : 4;
+    const bool pair = nw == 4 && (paired + slots - 1) / slots < (single + slots - 1) / slots;
+    const unsigned char *items = static_cast<const unsigned char *>(p.dev) + p.o_items;
+    A.items = reinterpret_cast<const int2 *>(items) + (pair ? 0 : p.npaired);
+    A.nitems = pair ? p.npaired : p.nsingle;
+    A.extra = nw == 4 ? p.extra4 : 0;
+    for (int k = 0; k <= nw; ++k) A.bchunk[k] = nw == 4 ? p.chunk4[k] : p.chunk8[k];
     // at least 80 KB: never more than two CTAs per SM, so that their tensor
     // memory (256 columns each) always fits
-    const size_t smem = std::max<size_t>(tma_smem_bytes(A.nc, A.extra), 80 * 1024);
-    const long long blocks = (long long)A.n_out * A.nbb;
+    const size_t smem = std::max<size_t>(tma_smem_bytes(nw, A.nc, A.extra), nw == 4 ? 80 * 1024 : 120 * 1024);
+    const long long blocks = pair ? paired : single;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    auto fn = A.k == 1 ? tma_scan_kernel<1> : tma_scan_kernel<2>;
+    void (*fn)(TmaArgs) = nullptr;
+    const bool one = A.k == 1;
+    switch (storage) {
+        case kStoreF32: fn = pick<float>(one, nw); break;
+        case kStoreBF16: fn = pick<__nv_bfloat16>(one, nw); break;
+        case kStoreF16: fn = pick<__half>(one, nw); break;
+        default: return cudaErrorInvalidValue;
+    }
     e = ensure_dyn_smem(reinterpret_cast<const void *>(fn), smem);
     if (e != cudaSuccess) return e;
-    fn<<<(unsigned)blocks, 32 * kTmaWarps, smem, stream>>>(A);
+    fn<<<(unsigned)blocks, 32 * nw, smem, stream>>>(A);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,8 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
             f.ob2 = r.ob2;
             f.lout1 = i < H ? (float)lam_out[i] : 0.f;
             f.lout2 = i + 1 < H ? (float)lam_out[i + 1] : 0.f;
+            f.lin1 = r.lin1;
+            f.lin2 = r.lin2;
             fin[k] = f;
             uint32_t bits = 0;
             for (int e = 0; e < 2; ++e) {

@@ -12,7 +12,7 @@
 //   lin*      input weights lambda_in (0 for padding hands),
 //   ma, mb    1 when the first / second card of hand 2i+1 is a card of hand
 //             2i, else 0,
-//   lout*     output weights lambda_out.
+//   lout*     output weights lambda_out; the finishing records repeat lin*.
 // A box's scan block is its 8 pair records followed by two tie words: byte
 // 8j + (k - 4j) of word j (pair k) has
 //   bits 2-4  hand 2k has a compatible tied hand 1, 2, 3 positions before it
@@ -39,7 +39,7 @@ struct alignas(16) TmaScanRec {
 constexpr int kScanBlock = 8 * 32 + 16;   // bytes per box
 struct alignas(16) TmaFinRec {
     uint32_t oa1, ob1, oa2, ob2;
-    float lout1, lout2, pad0, pad1;
+    float lout1, lout2, lin1, lin2;
 };
 
 // Records of one game and direction.  bytes = nbox scan blocks, then
