@@ -228,9 +228,9 @@ typedef struct kps_batch kps_batch;
  *   KPS_BATCH_STAGED  FP32, BF16 or FP16 storage (FP32 arithmetic): 4 warps
  *                     per CTA scan chunks of a game's hand order in 16-hand
  *                     boxes staged by cp.async, with per-box hand records
- *                     (games whose tie groups have at most 4 hands and whose
- *                     chunks fit 24 boxes; the others run on the
- *                     tensor-memory kernel in a second launch). */
+ *                     (games whose chunks fit 24 boxes and that have few
+ *                     hands in tie groups of more than 4; the others run
+ *                     on the tensor-memory kernel in a second launch). */
 #define KPS_BATCH_TMEM 0
 #define KPS_BATCH_STAGED 1
 

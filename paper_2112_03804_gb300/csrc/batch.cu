@@ -74,6 +74,8 @@ bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
             x.scol = g->dev.scol[dir];
             x.fcoef = g->dev.fcoef_f[dir];
             x.scoef = g->dev.scoef_f[dir];
+            x.hfcol = g->fcol[dir].data();
+            x.hscol = g->scol[dir].data();
             x.in_off = b->off[dir == 0 ? 1 : 0][i];
             x.out_off = b->off[dir == 0 ? 0 : 1][i];
         }

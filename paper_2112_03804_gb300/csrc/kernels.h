@@ -203,6 +203,7 @@ struct AmGameDesc {
     int n_out;
     const int *fcol, *scol;           // device tables of the direction
     const float *fcoef, *scoef;
+    const int *hfcol, *hscol;         // host copies
     long long in_off, out_off;        // element offsets in the batch vectors
 };
 struct AmPlan;

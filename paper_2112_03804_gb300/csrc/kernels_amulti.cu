@@ -7,10 +7,11 @@
 //   a = lambda_in * y_f,  b = lambda_in * y_s,  w = F a - S b,
 // K_F(w)[h] = Tot - P[c1] - P[c2] + w[h] (one-card hands: Tot - P[c1]).
 //
-// Organisation.  A work item is one game and up to 32 of its output
-// sequences: lane j owns sequence sigma0 + j, with its own fold and
-// showdown input rows and payoffs (a sequence without a fold or a
-// showdown terminal reads a zero row and has a zero payoff for it).  The
+// Organisation.  A work item is one game and up to 32 of its rows: lane j owns
+// row row0 + j, an output sequence with its own fold and showdown input rows
+// and payoffs (a sequence without a fold or a showdown terminal reads a zero
+// row and has a zero payoff for it), or the pair of a call and a fold that
+// share an input row: one scan of b (S = 1) gives both, as in kernels_tma.cu.  The
 // four warps of a CTA scan four chunks of the game's hand order in boxes
 // of 16 hands (the chunks and per-box hand records of scan_records.h,
 // built once per game and direction).  For each box every lane copies its
@@ -26,7 +27,9 @@
 // chunks are combined in shared memory exactly as in the single-game
 // kernel; the finishing pass reads each box's finishing records from the
 // record ring (copied one box ahead with cp.async, 256 bytes per half-warp),
-// and each lane writes its finished row segments with 16-byte stores.  CTAs are persistent: they take work items from an atomic ticket
+// and each lane writes its finished row segments with 16-byte stores.  Ties:
+// groups of up to 4 hands in registers, longer ones pair by pair from the
+// entry lists of scan_records.h.  CTAs are persistent: they take work items from an atomic ticket
 // or a static stride.  No spin-waits (cp.async groups complete in
 // hardware), no atomics on results: bit-reproducible.
 #include "kernels.h"
@@ -38,6 +41,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <cstring>
 #include <new>
@@ -58,22 +62,24 @@ constexpr int kMaxExtra = 8;               // chunk boxes past tensor memory (sc
 
 // One game in one direction (device).
 struct alignas(16) AmGame {
-    int H, hs, nc, n_out;
+    int H, hs, nc, n_rows;
     int nbox, pad0, pad1, pad2;
     int bchunk[kTmaWarps + 1];
     int pad3[3];
     int bchunk8[2 * kTmaWarps + 1];   // split items: each chunk cut in two at a tie-free box boundary
     int pad4[3];
     long long in_off, out_off;     // element offsets of the game's input / output vectors
+    const int2 *rows;              // [n_rows] output sequence, the fold-only sequence of its pair or -1
     const int *fcol, *scol;        // per output sequence: its fold / showdown input sequence or -1
     const float *fcoef, *scoef;    // and the payoffs
     const unsigned char *rscan;    // [nbox][kScanBlock]
     const TmaFinRec *rfin;         // [nbox * 8]
+    const TieEntry *ent;           // pairs of long tie groups
 };
 
 struct AmArgs {
     const AmGame *games;
-    const int4 *items;             // (game, first output sequence, split, 0)
+    const int4 *items;             // (game, first row, split, last row + 1)
     int nitems, nc, schedule;
     const void *vin;               // element type: the kernel's storage type
     void *vout;
@@ -195,8 +201,8 @@ template <> struct Store<__half> {
 // with fewer boxes runs zero-filled boxes to the other's count, so that the
 // warp's tensor-memory operations stay uniform.
 template <typename T, int K2>
-__device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int sigma0, int split, unsigned char *sm,
-                                        uint32_t tmem, float *xs) {
+__device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int row0, int row1, int split,
+                                        unsigned char *sm, uint32_t tmem, float *xs) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nc = P.nc, hs = G.hs;
     const int half = split ? lane >> 4 : 0, col = split ? lane & 15 : lane;
@@ -206,11 +212,17 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
     const int b0h0 = __shfl_sync(kFull, b0, 0), b0h1 = __shfl_sync(kFull, b0, 16);
     const int nbh0 = __shfl_sync(kFull, nbl, 0), nbh1 = __shfl_sync(kFull, nbl, 16);
     const int nb = split ? max(nbh0, nbh1) : nbl;   // the warp's box count
-    const int sigma = sigma0 + col;
-    const bool act = sigma < G.n_out;
+    const bool act = row0 + col < row1;
+    const int2 sq = act ? G.rows[row0 + col] : make_int2(0, -1);
+    const int sigma = sq.x;
     const int rf = act ? G.fcol[sigma] : -1, rs = act ? G.scol[sigma] : -1;
     const float F = rf >= 0 ? G.fcoef[sigma] : 0.f;
-    const float S = rs >= 0 ? G.scoef[sigma] : 0.f;
+    // a showdown-only row is scanned with S = 1 and finished with its payoff;
+    // Fm: the payoff of its fold-only mate
+    const bool unit = rf < 0 && rs >= 0;
+    const float S = unit ? 1.f : rs >= 0 ? G.scoef[sigma] : 0.f;
+    const float So = unit ? G.scoef[sigma] : 1.f, Fm = sq.y >= 0 ? G.fcoef[sq.y] : 0.f;
+    const bool pairs = __any_sync(kFull, sq.y >= 0);
     const float S2 = 2.f * S;
     constexpr int NQ = 16 / Store<T>::kPer;   // 16-byte chunks per 16-hand row segment
     const T *vin = static_cast<const T *>(P.vin) + G.in_off;
@@ -352,6 +364,21 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
                 }
             }
         }
+        // tie groups of more than 4 hands, pair by pair (rare: 1 in 270 of the
+        // 1081-hand games).  The game stays on this kernel: in a launch of its own
+        // on the tensor-memory kernel it cost a 256-game product 51 us more.
+        const uint32_t nent = reinterpret_cast<const uint32_t *>(rsb + 256)[3];
+        if (nent && rs >= 0) {
+            const TieEntry *te = G.ent + reinterpret_cast<const uint32_t *>(rsb + 256)[2];
+#pragma unroll 1
+            for (uint32_t e = 0; e < nent; ++e) {
+                const TieEntry t = te[e];
+                const float x = S * (t.lin * float(pb[t.q]));
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (i == t.i) p[i] += x;
+            }
+        }
         // every lane has read the slot's records: refill it
         __syncwarp();
         issue(m + kNS);
@@ -394,6 +421,11 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
                 reinterpret_cast<float *>(sm + am_ring_off(k))[q * 32 + lane] = pall + S2 * run;
                 run += rr[k];
             }
+            // pairs: P in place of every warp's sums (this lane alone read them)
+            if (pairs)
+#pragma unroll
+                for (int k = 0; k < kTmaWarps; ++k)
+                    reinterpret_cast<float2 *>(sm + am_state_off(k, nc))[q * 32 + lane].x = pall;
         }
     } else if (lane < 16) {
         for (int q = warp; q < nc; q += kTmaWarps) {
@@ -412,11 +444,15 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
                 reinterpret_cast<float *>(sm + am_ring_off(k >> 1))[q * 32 + lane + 16 * (k & 1)] = pall + S2 * run;
                 run += rr[k];
             }
+            if (pairs)
+#pragma unroll
+                for (int k = 0; k < 2 * kTmaWarps; ++k)
+                    reinterpret_cast<float2 *>(sm + am_state_off(k >> 1, nc))[q * 32 + lane + 16 * (k & 1)].x = pall;
         }
     }
-    float Cw;
+    float Cw, tall = 0.f;
     {
-        float tall = 0.f, gb = 0.f;
+        float gb = 0.f;
         if (!split) {
 #pragma unroll
             for (int k = 0; k < kTmaWarps; ++k) {
@@ -435,8 +471,13 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
     }
     __syncthreads();
 
-    // finishing: out = lambda_out (partial + C - Q[c1] - Q[c2])
+    // finishing: out = So lambda_out (partial + C - Q[c1] - Q[c2]), and a pair's
+    // fold side Fm lambda_out (b - Tot + P[c1] + P[c2]) (P and Tot of w = -b),
+    // its row read once more, box by box, into the rest of the ring
     const unsigned char *qb = ring + 4 * lane;
+    const unsigned char *pq = stb + 8 * lane;
+    const uint32_t yb = (uint32_t)kRing - 4096u + 16u * (uint32_t)lane;
+    T *orow2 = static_cast<T *>(P.vout) + G.out_off + (size_t)(sq.y >= 0 ? sq.y : 0) * hs;
     T *orow = static_cast<T *>(P.vout) + G.out_off + (size_t)(act ? sigma : 0) * hs;
     float cur[16], nxt[16];
     auto load_box = [&](int m, float *r) {
@@ -454,9 +495,18 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
     const uint32_t frb_s = smem_u32(rring);
     auto fetch_fin = [&](int m) {
         if (m < nb && (split || lane < 16)) {
-            const int bm = b0 + (m < nbl ? m : 0);   // a zero-filled box reads its half's first records
+            // a zero-filled box reads the game's first records: its half may be empty
+            // at the very end of the order
+            const int bm = m < nbl ? b0 + m : 0;
             cp16(frb_s + (uint32_t)((((m & 1) * 2 + half) * 256) + 16 * (lane & 15)),
                  reinterpret_cast<const unsigned char *>(G.rfin + (size_t)kTmaBox / 2 * bm) + 16 * (lane & 15), 16u);
+        }
+        if (pairs && sq.y >= 0 && m < nbl) {
+            const int x = kTmaBox * (b0 + m);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (x + Store<T>::kPer * q < hs)
+                    cp16(ring_s + yb + (uint32_t)((m & 1) * 2048) + 512u * q, pb + x + Store<T>::kPer * q, 16u);
         }
         cp_commit();
     };
@@ -470,18 +520,32 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
         cp_wait<1>();   // this lane's copy of box m's records
         __syncwarp();
         const TmaFinRec *fr = reinterpret_cast<const TmaFinRec *>(rring + ((m & 1) * 2 + half) * 256);
-        float o[16];
+        float o[16], y[16];
+        if (pairs) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) Store<T>::load(ring + yb + (m & 1) * 2048 + 512 * q, y + Store<T>::kPer * q);
+        }
 #pragma unroll
         for (int i = 0; i < 16; i += 2) {
             const TmaFinRec r = fr[i / 2];
+            if (pairs) {
+                float p1 = *reinterpret_cast<const float *>(pq + 2 * r.oa1);
+                float p2 = *reinterpret_cast<const float *>(pq + 2 * r.oa2);
+                if (K2 == 2) {
+                    p1 += *reinterpret_cast<const float *>(pq + 2 * r.ob1);
+                    p2 += *reinterpret_cast<const float *>(pq + 2 * r.ob2);
+                }
+                y[i] = (r.lout1 * Fm) * ((K2 == 2 ? fmaf(r.lin1, y[i], -tall) : -tall) + p1);
+                y[i + 1] = (r.lout2 * Fm) * ((K2 == 2 ? fmaf(r.lin2, y[i + 1], -tall) : -tall) + p2);
+            }
             float q1 = *reinterpret_cast<const float *>(qb + r.oa1);
             float q2 = *reinterpret_cast<const float *>(qb + r.oa2);
             if (K2 == 2) {
                 q1 += *reinterpret_cast<const float *>(qb + r.ob1);
                 q2 += *reinterpret_cast<const float *>(qb + r.ob2);
             }
-            o[i] = r.lout1 * ((pc[i] + Cw) - q1);
-            o[i + 1] = r.lout2 * ((pc[i + 1] + Cw) - q2);
+            o[i] = (r.lout1 * So) * ((pc[i] + Cw) - q1);
+            o[i + 1] = (r.lout2 * So) * ((pc[i + 1] + Cw) - q2);
         }
         if (act && real) {
             const int x = kTmaBox * (b0 + m);
@@ -489,6 +553,13 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int si
             for (int q = 0; q < NQ; ++q)
                 if (x + Store<T>::kPer * q < hs)
                     *reinterpret_cast<uint4 *>(orow + x + Store<T>::kPer * q) = Store<T>::pack(o + Store<T>::kPer * q);
+            if (pairs && sq.y >= 0) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q)
+                    if (x + Store<T>::kPer * q < hs)
+                        *reinterpret_cast<uint4 *>(orow2 + x + Store<T>::kPer * q) =
+                            Store<T>::pack(y + Store<T>::kPer * q);
+            }
         }
         if (m + 1 < nb) tm_wait_ld16(pn);
     };
@@ -532,7 +603,7 @@ __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_consta
         }
         if (item >= P.nitems) break;
         const int4 it = P.items[item];
-        am_item<T, K2>(P, P.games[it.x], it.y, it.z, sm, tmem, xs);
+        am_item<T, K2>(P, P.games[it.x], it.y, it.w, it.z, sm, tmem, xs);
         // the next ticket is written only after every thread has read this one
         // (am_item ends its combination with a CTA barrier)
     }
@@ -543,6 +614,11 @@ __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_consta
 }
 
 }  // namespace
+
+// Time (us) of an item [single rows, pairs][full, split] of a 1081-hand game,
+// {alone on its SM, two per SM}, measured on 8 to 512 river games: what
+// am_create's choice of rows and items goes by.
+constexpr double kItemTime[2][2][2] = {{{35, 52}, {25, 31}}, {{42, 66}, {31, 41}}};
 
 struct AmPlan {
     AmArgs a{};
@@ -574,7 +650,7 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
         }
         std::string w;
         try {
-            w = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, &rec[i]);
+            w = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, true, &rec[i]);
         } catch (const std::bad_alloc &) {
             *why = "host allocation";
             return nullptr;
@@ -590,9 +666,103 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
         ++ntaken;
         nc = std::max(nc, rec[i].nc);
         rbytes += (rec[i].bytes.size() + 255) / 256 * 256;
-        nitems += (d.n_out + 31) / 32;
     }
     if (ntaken == 0) return nullptr;
+    // Rows and items of every game: pairs or single sequences, items of 32 rows
+    // (a tail of at most 16 as a split item) or split items alone.  Pairs leave
+    // fewer items, split items half as long a scan: one A product of 512 river
+    // games takes 128 us with pairs in full items, 148 without pairs, of 100 games
+    // 33 us with single rows in split items, 52 in full ones, 43 with pairs; of
+    // the 241 games of a turn endgame (19 sequences, 13 rows) 37 us with pairs, 44
+    // without.
+    std::vector<char> can_split(ng, 0);
+    std::vector<std::array<int, 2 * kTmaWarps + 1>> sub(ng);
+    std::vector<std::vector<int2>> paired(ng), single(ng);
+    for (int i = 0; i < ng; ++i) {
+        if (!(*taken)[i]) continue;
+        const AmGameDesc &d = games[i];
+        const ScanRecords &r = rec[i];
+        // sub-chunks of split items: each chunk cut at the tie-free box
+        // boundary nearest its middle (an empty second half if there is none)
+        const HostGame &h = *d.h;
+        auto clean = [&](int bx) {
+            return bx <= 0 || bx >= r.nbox || 16 * bx >= r.H || h.group_lo[16 * bx] == 16 * bx;
+        };
+        can_split[i] = 1;
+        for (int w = 0; w < kTmaWarps; ++w) {
+            const int lo = r.bchunk[w], hi = r.bchunk[w + 1], ideal = (lo + hi) / 2;
+            int mid = hi;
+            for (int dd = 0; dd <= hi - lo && mid == hi; ++dd) {
+                if (ideal - dd >= lo && clean(ideal - dd)) mid = ideal - dd;
+                else if (ideal + dd <= hi && clean(ideal + dd)) mid = ideal + dd;
+            }
+            sub[i][2 * w] = lo;
+            sub[i][2 * w + 1] = mid;
+            can_split[i] = can_split[i] && mid - lo <= 16 && hi - mid <= 16;
+        }
+        sub[i][2 * kTmaWarps] = r.nbox;
+        // fold_of[c]: the fold-only sequence that reads input row c
+        std::vector<char> mated(d.n_out, 0);
+        std::vector<int> fold_of;
+        for (int s = 0; s < d.n_out; ++s) {
+            const int c = std::max(d.hfcol[s], d.hscol[s]);
+            if (c >= (int)fold_of.size()) fold_of.resize(c + 1, -1);
+            if (d.hfcol[s] >= 0 && d.hscol[s] < 0) fold_of[d.hfcol[s]] = s;
+        }
+        single[i].reserve(d.n_out);
+        paired[i].reserve(d.n_out);
+        for (int s = 0; s < d.n_out; ++s) {
+            single[i].push_back(make_int2(s, -1));
+            if (d.hfcol[s] >= 0) continue;
+            int2 row = make_int2(s, -1);
+            if (d.hscol[s] >= 0) {
+                row.y = fold_of[d.hscol[s]];
+                if (row.y >= 0 && mated[row.y]) row.y = -1;
+                if (row.y >= 0) mated[row.y] = 1;
+            }
+            paired[i].push_back(row);
+        }
+        for (int s = 0; s < d.n_out; ++s)
+            if (d.hfcol[s] >= 0 && !mated[s]) paired[i].push_back(make_int2(s, -1));
+    }
+    // estimated time of a layout (see kItemTime), its items in *out
+    auto layout = [&](const std::vector<std::vector<int2>> &rows, bool halves, std::vector<int4> *out) {
+        double sum = 0.0, alone = 0.0, longest = 0.0;
+        long long n_items = 0;
+        for (int i = 0; i < ng; ++i) {
+            const int n = (int)rows[i].size();
+            for (int r0 = 0; r0 < n;) {
+                const bool half = can_split[i] && (halves || n - r0 <= 16);
+                const int r1 = std::min(n, r0 + (half ? 16 : 32));
+                if (out) out->push_back(make_int4(i, r0, half ? 1 : 0, r1));
+                const double *c = kItemTime[&rows == &paired ? 1 : 0][half ? 1 : 0];
+                sum += c[1];
+                alone = std::max(alone, c[0]);
+                longest = std::max(longest, c[1]);
+                ++n_items;
+                r0 = r1;
+            }
+        }
+        if (2 * n_items <= grid_cap) return alone;
+        return n_items <= grid_cap ? longest : sum / grid_cap + 0.45 * longest;
+    };
+    double best = 0.0;
+    const std::vector<std::vector<int2>> *rows = nullptr;
+    bool halves = false;
+    for (int v = 0; v < 4; ++v) {
+        const auto &rv = v & 1 ? single : paired;
+        const double t = layout(rv, (v & 2) != 0, nullptr);
+        if (!rows || t < best) {
+            best = t;
+            rows = &rv;
+            halves = (v & 2) != 0;
+        }
+    }
+    std::vector<int4> items;
+    layout(*rows, halves, &items);
+    nitems = (long long)items.size();
+    size_t nrows = 0;
+    for (int i = 0; i < ng; ++i) nrows += (*rows)[i].size();
     if (nitems > 0x7fffffffLL) {
         *why = "too many work items";
         return nullptr;
@@ -602,7 +772,8 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
         return nullptr;
     }
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-    const size_t o_games = 0, o_items = al(sizeof(AmGame) * ng), o_rec = o_items + al(sizeof(int4) * (size_t)nitems);
+    const size_t o_games = 0, o_items = al(sizeof(AmGame) * ng), o_rows = o_items + al(sizeof(int4) * (size_t)nitems),
+                 o_rec = o_rows + al(sizeof(int2) * nrows);
     const size_t total = o_rec + rbytes;
     AmPlan *p = new (std::nothrow) AmPlan();
     if (!p) {
@@ -622,9 +793,7 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
     unsigned char *dev = static_cast<unsigned char *>(p->blob);
     std::vector<unsigned char> host(total, 0);
     std::vector<AmGame> g(ng);
-    std::vector<int4> items;
-    items.reserve((size_t)nitems);
-    size_t ro = o_rec;
+    size_t ro = o_rec, rowo = o_rows;
     for (int i = 0; i < ng; ++i) {
         const AmGameDesc &d = games[i];
         const ScanRecords &r = rec[i];
@@ -634,7 +803,11 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
         x.H = r.H;
         x.hs = r.hs;
         x.nc = r.nc;
-        x.n_out = d.n_out;
+        x.n_rows = (int)(*rows)[i].size();
+        std::memcpy(host.data() + rowo, (*rows)[i].data(), sizeof(int2) * (*rows)[i].size());
+        x.rows = reinterpret_cast<const int2 *>(dev + rowo);
+        rowo += sizeof(int2) * (*rows)[i].size();
+        for (int w = 0; w <= 2 * kTmaWarps; ++w) x.bchunk8[w] = sub[i][w];
         x.nbox = r.nbox;
         for (int w = 0; w <= kTmaWarps; ++w) x.bchunk[w] = r.bchunk[w];
         x.in_off = d.in_off;
@@ -646,30 +819,8 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
         std::memcpy(host.data() + ro, r.bytes.data(), r.bytes.size());
         x.rscan = dev + ro;
         x.rfin = reinterpret_cast<const TmaFinRec *>(dev + ro + (size_t)r.nbox * kScanBlock);
+        x.ent = reinterpret_cast<const TieEntry *>(dev + ro + r.entries_at);
         ro += al(r.bytes.size());
-        // sub-chunks of split items: each chunk cut at the tie-free box
-        // boundary nearest its middle (an empty second half if there is none)
-        const HostGame &h = *d.h;
-        auto clean = [&](int bx) {
-            return bx <= 0 || bx >= r.nbox || 16 * bx >= r.H || h.group_lo[16 * bx] == 16 * bx;
-        };
-        bool split_ok = true;
-        for (int w = 0; w < kTmaWarps; ++w) {
-            const int lo = r.bchunk[w], hi = r.bchunk[w + 1], ideal = (lo + hi) / 2;
-            int mid = hi;
-            for (int dd = 0; dd <= hi - lo && mid == hi; ++dd) {
-                if (ideal - dd >= lo && clean(ideal - dd)) mid = ideal - dd;
-                else if (ideal + dd <= hi && clean(ideal + dd)) mid = ideal + dd;
-            }
-            x.bchunk8[2 * w] = lo;
-            x.bchunk8[2 * w + 1] = mid;
-            split_ok = split_ok && mid - lo <= 16 && hi - mid <= 16;
-        }
-        x.bchunk8[2 * kTmaWarps] = r.nbox;
-        // full items of 32 sequences; a tail of at most 16 as a split item
-        const int nfull = d.n_out / 32, tail = d.n_out - 32 * nfull;
-        for (int t = 0; t < nfull; ++t) items.push_back(make_int4(i, 32 * t, 0, 0));
-        if (tail > 0) items.push_back(make_int4(i, 32 * nfull, tail <= 16 && split_ok ? 1 : 0, 0));
     }
     std::memcpy(host.data() + o_games, g.data(), sizeof(AmGame) * ng);
     if (!items.empty()) std::memcpy(host.data() + o_items, items.data(), sizeof(int4) * items.size());

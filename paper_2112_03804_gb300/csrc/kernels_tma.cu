@@ -870,7 +870,7 @@ static size_t tma_smem_bytes(int nw, int nc, int extra) { return hdr_off(nw, nc,
 // tensor maps, pointers and batch) and p.host.  Empty string on success.
 static std::string tma_prepare(const HostGame &h, const double *lam_in, const double *lam_out, TmaParams &p) {
     ScanRecords r;
-    const std::string why = build_scan_records(h, lam_in, lam_out, kTmaMaxExtra, &r);
+    const std::string why = build_scan_records(h, lam_in, lam_out, kTmaMaxExtra, false, &r);
     if (!why.empty()) return why;
     TmaArgs &A = p.a;
     A.H = r.H;

@@ -8,7 +8,7 @@
 namespace kps {
 
 std::string build_scan_records(const HostGame &h, const double *lam_in, const double *lam_out, int max_extra,
-                               ScanRecords *out) {
+                               bool long_ties, ScanRecords *out) {
     ScanRecords &R = *out;
     if (h.k != 1 && h.k != 2) return "cards per hand";
     const int nc = h.ncards + 1;
@@ -16,11 +16,14 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
     const int H = h.H, hs = h.hs;
     const int nbox = (hs + kTmaBox - 1) / kTmaBox;
     // tie groups: at most 4 hands (partners within 3 positions)
+    auto is_long = [&](int i) { return h.group_hi[i] - h.group_lo[i] > 3; };
     for (int i = 0; i < H; ++i)
-        if (h.group_hi[i] - h.group_lo[i] > 3) return "tie group longer than 4 hands";
+        if (is_long(i) && !long_ties) return "tie group longer than 4 hands";
     // chunk boundaries at box boundaries that cut no tie group, as close to
     // an even split as possible
-    auto clean = [&](int bx) { return bx <= 0 || bx >= nbox || 16 * bx >= H || h.group_lo[16 * bx] == 16 * bx; };
+    auto clean = [&](int bx) {
+        return bx <= 0 || bx >= nbox || 16 * bx >= H || h.group_lo[16 * bx] == 16 * bx || is_long(16 * bx);
+    };
     R.bchunk[0] = 0;
     R.bchunk[kTmaWarps] = nbox;
     for (int k = 1; k < kTmaWarps; ++k) {
@@ -61,6 +64,8 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
                 if (card(x, j) == card(y, l)) return true;
         return false;
     };
+    std::vector<TieEntry> entries;
+    size_t chunk_first = 0;
     for (int bx = 0; bx < nbox; ++bx) {
         unsigned char *blk = R.bytes.data() + (size_t)bx * kScanBlock;
         TmaFinRec *fin = reinterpret_cast<TmaFinRec *>(R.bytes.data() + scan_bytes) + 8 * bx;
@@ -93,7 +98,7 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
             uint32_t bits = 0;
             for (int e = 0; e < 2; ++e) {
                 const int hi = i + e;
-                if (hi >= H) continue;
+                if (hi >= H || is_long(hi)) continue;
                 for (int d = 1; d <= 3; ++d) {
                     const int q = hi - d;
                     if (q < h.group_lo[hi]) break;
@@ -104,7 +109,22 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
             tw[k / 4] |= bits << (8 * (k & 3));
         }
         std::memcpy(blk + 256, tw, sizeof(tw));
+        for (int k = 0; k <= kTmaWarps; ++k)
+            if (R.bchunk[k] == bx) chunk_first = entries.size();
+        const uint32_t first = (uint32_t)entries.size();
+        for (int i = 16 * bx; i < std::min(H, 16 * bx + 16); ++i) {
+            if (!is_long(i)) continue;
+            for (int q = h.group_lo[i]; q <= h.group_hi[i]; ++q)
+                if (q != i && !share(i, q))
+                    entries.push_back(TieEntry{i - 16 * bx, q, (float)(q > i ? lam_in[q] : -lam_in[q]), 0});
+        }
+        if (entries.size() - chunk_first > (size_t)kMaxTieEntries) return "many hands in long tie groups";
+        const uint32_t ref[2] = {first, (uint32_t)entries.size() - first};
+        std::memcpy(blk + 264, ref, sizeof(ref));
     }
+    R.entries_at = R.bytes.size();
+    R.bytes.resize(R.entries_at + entries.size() * sizeof(TieEntry));
+    if (!entries.empty()) std::memcpy(R.bytes.data() + R.entries_at, entries.data(), entries.size() * sizeof(TieEntry));
     return "";
 }
 

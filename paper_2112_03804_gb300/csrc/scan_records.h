@@ -17,8 +17,12 @@
 // 8j + (k - 4j) of word j (pair k) has
 //   bits 2-4  hand 2k has a compatible tied hand 1, 2, 3 positions before it
 //   bits 5-7  the same for hand 2k+1.
-// Tie groups of at most 4 hands are accepted, and chunk boundaries fall on
-// box boundaries that cut no tie group.
+// Chunk boundaries fall on box boundaries that cut no tie group of up to 4
+// hands.  Longer groups are refused, or (long_ties) listed: the last 8 bytes of
+// a box's scan block are {first, count} into the TieEntry list, one entry per
+// ordered pair of compatible hands of such a group; those hands have no tie
+// bits, and chunk boundaries may cut the group (the scan counts every earlier
+// hand as weaker, whichever chunk it is in, and an entry undoes that).
 #pragma once
 
 #include <cstdint>
@@ -37,24 +41,31 @@ struct alignas(16) TmaScanRec {
     float lin1, lin2, ma, mb;
 };
 constexpr int kScanBlock = 8 * 32 + 16;   // bytes per box
+struct alignas(16) TieEntry {
+    int i, q;                      // hand 16 box + i, its tied partner q
+    float lin;                     // lambda_in[q] when q comes later, - lambda_in[q] when earlier
+    int pad;
+};
+constexpr int kMaxTieEntries = 256;       // per chunk of a box row
 struct alignas(16) TmaFinRec {
     uint32_t oa1, ob1, oa2, ob2;
     float lout1, lout2, lin1, lin2;
 };
 
-// Records of one game and direction.  bytes = nbox scan blocks, then
-// nbox * 8 finishing records.
+// Records of one game and direction.  bytes = nbox scan blocks, nbox * 8
+// finishing records, the tie entries.
 struct ScanRecords {
     int H = 0, hs = 0, nc = 0, k = 0, nbox = 0;
     int extra = 0;                 // boxes of the longest chunk past 16
     int bchunk[kTmaWarps + 1] = {0, 0, 0, 0, 0};
+    size_t entries_at = 0;         // byte offset of the tie entries
     std::vector<unsigned char> bytes;
 };
 
 // Empty string on success, else why the game does not fit these kernels
-// (tie group over 4 hands, more than 64 card rows, a chunk longer than
-// 16 + max_extra boxes).
+// (tie group over 4 hands or, with long_ties, more than kMaxTieEntries pairs in a
+// chunk; more than 64 card rows; a chunk longer than 16 + max_extra boxes).
 std::string build_scan_records(const HostGame &h, const double *lam_in, const double *lam_out, int max_extra,
-                               ScanRecords *out);
+                               bool long_ties, ScanRecords *out);
 
 }  // namespace kps
