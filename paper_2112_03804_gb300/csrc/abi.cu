@@ -376,6 +376,56 @@ kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t
     return KPS_OK;
 }
 
+kps::F64GameDesc f64_desc(const kps_game *g, int dir) {
+    const kps::HostGame &h = g->host;
+    kps::F64GameDesc d{};
+    d.h = &h;
+    d.lam_in = dir == 0 ? h.lam2.data() : h.lam1.data();
+    d.lam_out = dir == 0 ? h.lam1.data() : h.lam2.data();
+    d.n_out = dir == 0 ? h.n[0] : h.n[1];
+    d.n_in = dir == 0 ? h.n[1] : h.n[0];
+    d.fcol = g->dev.fcol[dir];
+    d.scol = g->dev.scol[dir];
+    d.fcoef = g->dev.fcoef_d[dir];
+    d.scoef = g->dev.scoef_d[dir];
+    d.hfcol = g->fcol[dir].data();
+    d.hscol = g->scol[dir].data();
+    return d;
+}
+
+// The FP64 path (kernels_f64.cu) when the game and the vectors allow it;
+// *taken tells whether it ran.  KPS_KERNEL = f64 or unset.
+kps_status matvec_f64(kps_game *g, int dir, const void *vin, void *vout, int32_t batch, cudaStream_t stream,
+                      bool *taken) {
+    *taken = false;
+    const char *force = std::getenv("KPS_KERNEL");
+    if (force && std::strcmp(force, "f64") != 0) return KPS_OK;
+    if (((reinterpret_cast<uintptr_t>(vin) | reinterpret_cast<uintptr_t>(vout)) & 15) != 0) return KPS_OK;
+    if (g->f64_state[dir] == 0) {
+        // the plan is uploaded with a synchronisation, which a capturing stream
+        // cannot do: the other FP64 kernel's tables may be there already
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return KPS_OK;
+        std::string why;
+        kps::F64Plan *p = nullptr;
+        try {
+            p = kps::f64_create({f64_desc(g, dir)}, false, stream, &why);
+        } catch (const std::bad_alloc &) {
+        }
+        g->f64[dir].reset(p);
+        g->f64_state[dir] = p ? 1 : -1;
+    }
+    if (g->f64_state[dir] != 1) return KPS_OK;
+    *taken = true;
+    g->last_kernel[dir] = KPS_KERNEL_F64;
+    cudaError_t e = kps::launch_f64_scan(g->f64[dir].get(), static_cast<const double *>(vin),
+                                         static_cast<double *>(vout), batch, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "launching the FP64 payoff scan");
+    return KPS_OK;
+}
+
 kps_status matvec(kps_game *g, int dir, const void *vin, void *vout, int32_t batch, kps_dtype dt,
                   void *stream_ptr) {
     if (!g) return fail(KPS_EINVAL, "game is NULL");
@@ -421,6 +471,11 @@ kps_status matvec(kps_game *g, int dir, const void *vin, void *vout, int32_t bat
     if (storage != kps::kStoreF64) {
         bool taken = false;
         kps_status s2 = matvec_tma(g, dir, vin, vout, batch, storage, stream, &taken);
+        if (taken || s2 != KPS_OK) return s2;
+    }
+    if (storage == kps::kStoreF64) {
+        bool taken = false;
+        kps_status s2 = matvec_f64(g, dir, vin, vout, batch, stream, &taken);
         if (taken || s2 != KPS_OK) return s2;
     }
     if (h.max_tie <= kps::kTile) return matvec_fast(g, dir, p, storage, dt, stream);

@@ -75,6 +75,12 @@ struct kps_game {
     };
     std::unique_ptr<kps::TmaParams, TmaDel> tma[2];
     int tma_state[2] = {0, 0};
+    // plans of the FP64 path per direction, as above
+    struct F64Del {
+        void operator()(kps::F64Plan *p) const { kps::f64_destroy(p); }
+    };
+    std::unique_ptr<kps::F64Plan, F64Del> f64[2];
+    int f64_state[2] = {0, 0};
     // kernel of the last product per direction (KPS_KERNEL_* of kps.h)
     int last_kernel[2] = {0, 0};
 };
@@ -83,6 +89,9 @@ namespace kps_abi {
 
 // kps_sparsify with internal build options (NULL = none).
 kps_status create_game(const kps_game_spec *spec, const kps::BuildOptions *opt, kps_game **out);
+
+// The FP64 plan's view of a game (uploaded) in a direction.
+kps::F64GameDesc f64_desc(const kps_game *g, int dir);
 
 // Uploads the game's tables to the current device on first use.
 kps_status upload(kps_game *g, cudaStream_t stream);

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <new>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <string>
@@ -291,6 +293,37 @@ kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, 
     return KPS_OK;
 }
 
+bool batch_f64_ready(kps_batch *b, cudaStream_t stream) {
+    if (b->f64_state != 0) return b->f64_state == 1;
+    if (const char *force = std::getenv("KPS_KERNEL"))
+        if (std::strcmp(force, "f64") != 0) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) cudaGetLastError();
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    b->f64_state = -1;
+    for (int dir = 0; dir < 2; ++dir) {
+        std::string why;
+        try {
+            std::vector<kps::F64GameDesc> d;
+            for (size_t i = 0; i < b->games.size(); ++i) {
+                d.push_back(f64_desc(b->games[i], dir));
+                d.back().in_off = b->off[dir == 0 ? 1 : 0][i];
+                d.back().out_off = b->off[dir == 0 ? 0 : 1][i];
+            }
+            b->f64[dir] = kps::f64_create(d, true, stream, &why);
+        } catch (const std::bad_alloc &) {
+        }
+        if (!b->f64[dir]) {
+            kps::f64_destroy(b->f64[0]);
+            b->f64[0] = nullptr;
+            return false;
+        }
+    }
+    b->f64_state = 1;
+    return true;
+}
+
 kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream) {
     if (!b) return fail(KPS_EINVAL, "batch is NULL");
     if (dtype_size(dt) == 0) return fail(KPS_EINVAL, "unknown dtype");
@@ -305,6 +338,12 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
     if (ci < co + out_bytes && co < ci + in_bytes) return fail(KPS_EINVAL, "input and output overlap");
     if (((reinterpret_cast<uintptr_t>(vin) | reinterpret_cast<uintptr_t>(vout)) & 15) != 0)
         return fail(KPS_EINVAL, "batch vectors must be 16-byte aligned");
+    if (dt == KPS_F64 && batch_f64_ready(b, stream)) {
+        const cudaError_t e =
+            kps::launch_f64_scan(b->f64[dir], static_cast<const double *>(vin), static_cast<double *>(vout), 1, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "launching the FP64 batched payoff scan");
+        return KPS_OK;
+    }
     BatchShape s;
     kps_status st = batch_default_shape(b, dt, stream, &s);
     if (st != KPS_OK) return st;
@@ -384,6 +423,7 @@ kps_status kps_batch_destroy(kps_batch *b) {
     for (auto &kv : b->tables) cudaFree(kv.second.blob);
     for (auto &kv : b->rest_tables) cudaFree(kv.second.blob);
     for (int k = 0; k < 2; ++k) kps::am_destroy(b->am[k]);
+    for (int k = 0; k < 2; ++k) kps::f64_destroy(b->f64[k]);
     warm_free(b);
     if (b->ticket) cudaFree(b->ticket);
     delete b;

@@ -45,6 +45,8 @@ struct kps_batch {
     int am_nrest = 0;
     int rest_nw = 0;                 // warps of the tensor-memory launch over those games
     std::map<int, kps_abi::BatchTable> rest_tables;   // per direction
+    kps::F64Plan *f64[2] = {nullptr, nullptr};        // FP64 kernel, per direction
+    int f64_state = 0;               // 0 not tried, 1 built, -1 a game does not fit
 };
 
 namespace kps_abi {
@@ -59,6 +61,9 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
 // Builds the staged kernel's plans on first use (host work, synchronises
 // `stream`); true when every game fits that kernel.
 bool batch_staged_ready(kps_batch *b, cudaStream_t stream);
+// Builds the FP64 kernel's plans on first use (not on a capturing stream);
+// true when every game fits that kernel.
+bool batch_f64_ready(kps_batch *b, cudaStream_t stream);
 // Reads and clears the flag the warm-start predictor sets when a bounded
 // wait gives up (warm.cu; synchronises the device).
 cudaError_t predict_take_error(bool *set);

@@ -192,6 +192,24 @@ cudaError_t launch_tma_scan(TmaParams *p, int storage, const void *vin, void *vo
 // gives up (synchronises the device).
 cudaError_t tma_take_error(bool *set);
 
+// FP64 path (kernels_f64.cu) for two-card games with few ties: one game and
+// many vectors, or (multi) many games with one vector each.  Builds and uploads
+// the plan (synchronises `stream`); nullptr with *why set when a game does not
+// fit.  batch: vectors of a single game, 1 for many games.
+struct F64GameDesc {
+    const HostGame *h;
+    const double *lam_in, *lam_out;   // host, library order
+    int n_out, n_in;
+    const int *fcol, *scol;           // device tables of the direction
+    const double *fcoef, *scoef;
+    const int *hfcol, *hscol;         // host copies
+    long long in_off, out_off;        // element offsets in the batch vectors
+};
+struct F64Plan;
+F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why);
+void f64_destroy(F64Plan *p);
+cudaError_t launch_f64_scan(F64Plan *p, const double *vin, double *vout, int batch, cudaStream_t stream);
+
 // Staged multi-game path (FP32, BF16 or FP16 storage, kStore*; FP32
 // arithmetic; kernels_amulti.cu): one persistent
 // launch over (game, 32 output sequences) work items of a batch, one vector

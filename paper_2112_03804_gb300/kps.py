@@ -413,7 +413,7 @@ class TechniqueB:
 
 STATIC_SCRATCH_FLOATS = 4194304
 BATCH_TMEM, BATCH_STAGED = 0, 1
-KERNEL_NAMES = {1: "tma", 2: "tmem", 3: "vec", 4: "fast", 5: "general"}
+KERNEL_NAMES = {1: "tma", 2: "tmem", 3: "vec", 4: "fast", 5: "general", 6: "f64"}
 
 
 def matvec_A_static_scratch(game: Game, y, out, batch: int, dtype=None, stream=None):
