@@ -14,15 +14,16 @@
 // and the pipe must never wait: six warps per SM, each with its own per-card
 // table.  The kernel it replaces (kernels_vec.cu, still taken where this one
 // does not apply) had three warps per SM and several times the instructions:
-// MEASURED.
+// 100 vectors of the 1081-hand river game 436 -> 215 us, one product of 64 such
+// games 514 -> 132 us.
 //
 // Organisation.  A CTA = one item: up to 32 columns (row, vector) of one game
-// and one kind, lane = column, or up to 16 columns with lanes 16-31 on the same
-// columns over the second half of every warp's chunk (split items: where 32
-// columns are not there, or too few items for the SMs).  The NW warps scan NW
+// and one kind, lane = column; or up to 16 (8) columns, their two (four) groups
+// of lanes on two (four) parts of every warp's chunk: where 32 columns are not
+// there, or where shorter items fill the SMs better.  The NW warps scan NW
 // chunks of the hand order in boxes of 8 hands.  Every lane copies its own
 // 64-byte row segments with cp.async one box ahead ([16 bytes][lane]: conflict
-// free), the first 17 lanes of a half the box's records.  Partial results go to
+// free), a group's lanes together its box's records.  Partial results go to
 // the output row and come back in the finishing pass (the lane's own, L2), so
 // that shared memory holds the tables only.  Combination: Q_k[c] = P[c] + 2 S
 // (mass of card c in earlier chunks) takes the place of chunk k's sums in its
@@ -49,6 +50,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBox = 8;                    // hands per box
 constexpr int kNW = 6;                     // warps per CTA
 constexpr int kNS = 2;                     // ring slots
+constexpr int kParts = 4;                  // most parts of a chunk
 constexpr int kRow = 2048;                 // bytes of one row's box (32 lanes x 64)
 constexpr int kSlot = 2 * kRow;
 
@@ -58,15 +60,17 @@ struct alignas(16) Rec {                   // hands 2i, 2i + 1 of a box
     uint32_t ma, mb;                       // the second hand's first / second card is one of the first hand's
     uint32_t pad[2];
 };
-struct alignas(16) RecBox {
-    Rec r[kBox / 2];
-    uint32_t first, count, pad[2];         // tie entries
-};
-static_assert(sizeof(Rec) == 64 && sizeof(RecBox) == 272, "record layout");
 struct alignas(16) Tie {
     int i, q;                              // hand i of the box, its tied partner q
     double lin;                            // lambda_in[q], negative when q is earlier
 };
+constexpr int kInline = 2;                 // tie entries in the record itself (a tied pair inside a box makes two)
+struct alignas(16) RecBox {
+    Rec r[kBox / 2];
+    Tie t[kInline];
+    uint32_t first, count, pad[2];         // the others in the game's list; count of all
+};
+static_assert(sizeof(Rec) == 64 && sizeof(RecBox) == 304, "record layout");
 
 // One game in one direction (device).
 struct alignas(16) Game {
@@ -82,15 +86,15 @@ struct alignas(16) Game {
 
 struct Args {
     const Game *games;
-    const int4 *items;                     // (game, first column, end, split | unit << 1), or null: one game
+    const int4 *items;                     // (game, first column, end, parts | unit << 3), or null: one game
     const double *vin;
     double *vout;
-    int batch, nc, split, nother;          // one game: vectors, and its items: nother of the other rows first
+    int batch, nc, parts, nother;          // one game: vectors, and its items: nother of the other rows first
 };
 
 // Shared memory of a warp: table [card][lane] {b mass, w total}, ring, records.
 __host__ __device__ inline size_t table_bytes(int nc) { return (size_t)nc * 512; }
-__host__ __device__ inline size_t warp_bytes(int nc) { return table_bytes(nc) + kNS * kSlot + kNS * 2 * sizeof(RecBox); }
+__host__ __device__ inline size_t warp_bytes(int nc) { return table_bytes(nc) + kNS * kSlot + kNS * kParts * sizeof(RecBox); }
 inline size_t smem_bytes(int nc) { return kNW * warp_bytes(nc) + 2 * kNW * 32 * 8; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -107,10 +111,10 @@ __device__ __forceinline__ void cp_wait() {
 // UNIT: every column is showdown-only (S = 1, w = -b; a table's second
 // components unused), its fold-only mate finished with it.
 template <bool UNIT>
-__device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0, int col1, bool split,
+__device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0, int col1, int parts,
                                          unsigned char *smem) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nc = P.nc, hs = G.hs;
-    const int half = split ? lane >> 4 : 0, col = col0 + (split ? lane & 15 : lane);
+    const int width = 32 / parts, part = lane / width, slot = lane & (width - 1), col = col0 + slot;
     const bool act = col < col1;
     const int row = (UNIT ? 0 : G.nunit) + (act ? col / P.batch : 0), vec = act ? col % P.batch : 0;
     const int2 sq = act ? G.rows[row] : make_int2(0, -1);
@@ -124,13 +128,10 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
     const double *pa = vin + (long long)(rf >= 0 ? rf : 0) * hs, *pb = vin + (long long)(rs >= 0 ? rs : 0) * hs;
     double *vout = P.vout + G.out_off + (long long)vec * G.n_out * hs;
     double *po = vout + (long long)sigma * hs, *po2 = vout + (long long)(sq.y >= 0 ? sq.y : 0) * hs;
-    // this lane's boxes, and both halves' for the records
-    auto bound = [&](int k) { return (int)((long long)G.nbox * k / (kNW * (split ? 2 : 1))); };
-    const int sub = split ? 2 * warp + half : warp;
-    const int b0 = bound(sub), nbl = bound(sub + 1) - b0;
-    const int h0 = split ? bound(2 * warp) : b0, n0 = split ? bound(2 * warp + 1) - h0 : nbl;
-    const int h1 = split ? bound(2 * warp + 1) : b0, n1 = split ? bound(2 * warp + 2) - h1 : 0;
-    const int nb = max(n0, n1);
+    // this lane's boxes, and the warp's longest part
+    const int nk = kNW * parts, sub = parts * warp + part;
+    auto bound = [&](int k) { return (int)((long long)G.nbox * k / nk); };
+    const int b0 = bound(sub), nbl = bound(sub + 1) - b0, nb = __reduce_max_sync(kFull, nbl);
 
     unsigned char *mine = smem + (size_t)warp * warp_bytes(nc);
     double2 *tab = reinterpret_cast<double2 *>(mine) + lane;   // [card * 32]; a record offset is card * 16
@@ -154,16 +155,11 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
                     cp16(ring_s + (uint32_t)(sl * kSlot + kRow + 512 * q), pb + x + 2 * q, real && rs >= 0 ? 16u : 0u);
                 }
             }
-            // records of each half's box (zeros past its last)
-            if (lane < (int)sizeof(RecBox) / 16) {
-                const bool r0 = m < n0, r1 = m < n1;
-                cp16(recs_s + (uint32_t)(2 * sl * sizeof(RecBox)) + 16u * (uint32_t)lane,
-                     reinterpret_cast<const unsigned char *>(r0 ? G.rec + h0 + m : G.rec) + 16 * lane, r0 ? 16u : 0u);
-                if (split)
-                    cp16(recs_s + (uint32_t)((2 * sl + 1) * sizeof(RecBox)) + 16u * (uint32_t)lane,
-                         reinterpret_cast<const unsigned char *>(r1 ? G.rec + h1 + m : G.rec) + 16 * lane,
-                         r1 ? 16u : 0u);
-            }
+            // records of each part's box (zeros past its last)
+            const bool rec = m < nbl;
+            for (int j = slot; j < (int)sizeof(RecBox) / 16; j += width)
+                cp16(recs_s + (uint32_t)((kParts * sl + part) * sizeof(RecBox)) + 16u * (uint32_t)j,
+                     reinterpret_cast<const unsigned char *>(rec ? G.rec + b0 + m : G.rec) + 16 * j, rec ? 16u : 0u);
         }
         cp_commit();
     };
@@ -184,7 +180,7 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
         cp_wait<1>();
         __syncwarp();
         const int sl = m & 1, x = kBox * (b0 + m);
-        const RecBox *rb = reinterpret_cast<const RecBox *>(recs) + 2 * sl + half;
+        const RecBox *rb = reinterpret_cast<const RecBox *>(recs) + kParts * sl + part;
         double ys[kBox], yf[kBox], p[kBox];
         if (!UNIT) values(ring + sl * kSlot + 16 * lane, x, yf);
         values(ring + sl * kSlot + kRow + 16 * lane, x, ys);
@@ -230,10 +226,17 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
             }
         }
         if (rb->count && rs >= 0) {
-            const Tie *te = G.ties + rb->first;
             for (uint32_t e = 0; e < rb->count; ++e) {
-                const Tie t = te[e];
-                const double d = S * (t.lin * pb[t.q]);
+                const Tie t = e < kInline ? rb->t[e] : G.ties[rb->first + e - kInline];
+                double y = 0.0;
+                if ((unsigned)(t.q - x) < (unsigned)kBox) {   // most partners are in the box itself
+#pragma unroll
+                    for (int i = 0; i < kBox; ++i)
+                        if (i == t.q - x) y = ys[i];
+                } else {
+                    y = pb[t.q];
+                }
+                const double d = S * (t.lin * y);
 #pragma unroll
                 for (int i = 0; i < kBox; ++i)
                     if (i == t.i) p[i] += d;
@@ -255,13 +258,13 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
     sums[warp * 32 + lane] = Gm;
     sums[(kNW + warp) * 32 + lane] = UNIT ? -Gm : 0.5 * tot;   // every hand is in two card rows
     __syncthreads();
-    const int nk = split ? 2 * kNW : kNW;
-    if (!split || lane < 16) {
-        for (int c = warp; c < nc; c += kNW) {
+    {
+        // a row of the tables by the lanes of one part, for its columns
+        for (int c = sub; c < nc; c += nk) {
             double pall = 0.0, run = 0.0;
             auto cell = [&](int k) {
-                return reinterpret_cast<double2 *>(smem + (size_t)(split ? k >> 1 : k) * warp_bytes(nc)) + c * 32 + lane +
-                       (split ? 16 * (k & 1) : 0);
+                return reinterpret_cast<double2 *>(smem + (size_t)(k / parts) * warp_bytes(nc)) + c * 32 + slot +
+                       width * (k % parts);
             };
             for (int k = 0; k < nk; ++k) pall += UNIT ? -cell(k)->x : cell(k)->y;
             for (int k = 0; k < nk; ++k) {
@@ -274,7 +277,7 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
     }
     double C, tall = 0.0, gb = 0.0;
     for (int k = 0; k < nk; ++k) {
-        const int i = split ? (k >> 1) * 32 + (lane & 15) + 16 * (k & 1) : k * 32 + lane;
+        const int i = k / parts * 32 + slot + width * (k % parts);
         tall += sums[kNW * 32 + i];
         if (k < sub) gb += sums[i];
     }
@@ -302,7 +305,7 @@ __device__ __forceinline__ void f64_item(const Args &P, const Game &G, int col0,
         load(m + 1, nxt, yn);
         cp_wait<1>();
         __syncwarp();
-        const RecBox *rb = reinterpret_cast<const RecBox *>(recs) + 2 * (m & 1) + half;
+        const RecBox *rb = reinterpret_cast<const RecBox *>(recs) + kParts * (m & 1) + part;
         const int x = kBox * (b0 + m);
         if (act && m < nbl) {
 #pragma unroll
@@ -339,14 +342,14 @@ __global__ void __launch_bounds__(32 * kNW, 1) f64_scan_kernel(const __grid_cons
     } else {
         // one game: the items of the other rows (the longer ones), then the showdown-only ones
         const Game &G = P.games[0];
-        const int w = P.split ? 16 : 32, b = (int)blockIdx.x;
+        const int w = 32 / P.parts, b = (int)blockIdx.x;
         const bool unit = b >= P.nother;
         const int c0 = w * (unit ? b - P.nother : b), n = (unit ? G.nunit : G.nrows - G.nunit) * P.batch;
-        it = make_int4(0, c0, min(n, c0 + w), (P.split ? 1 : 0) | (unit ? 2 : 0));
+        it = make_int4(0, c0, min(n, c0 + w), P.parts | (unit ? 8 : 0));
     }
     const Game &G = P.games[it.x];
-    if (it.w & 2) f64_item<true>(P, G, it.y, it.z, (it.w & 1) != 0, smem);
-    else f64_item<false>(P, G, it.y, it.z, (it.w & 1) != 0, smem);
+    if (it.w & 8) f64_item<true>(P, G, it.y, it.z, it.w & 7, smem);
+    else f64_item<false>(P, G, it.y, it.z, it.w & 7, smem);
 }
 
 }  // namespace
@@ -403,10 +406,16 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
                 }
             }
             rb[b].first = (uint32_t)ties.size();
+            uint32_t n = 0;
             for (int x = kBox * b; x < std::min(h.H, kBox * b + kBox); ++x)
                 for (int q = h.group_lo[x]; q <= h.group_hi[x]; ++q)
-                    if (q != x && !share(x, q)) ties.push_back(Tie{x - kBox * b, q, q > x ? d.lam_in[q] : -d.lam_in[q]});
-            rb[b].count = (uint32_t)ties.size() - rb[b].first;
+                    if (q != x && !share(x, q)) {
+                        const Tie t{x - kBox * b, q, q > x ? d.lam_in[q] : -d.lam_in[q]};
+                        if (n < kInline) rb[b].t[n] = t;
+                        else ties.push_back(t);
+                        ++n;
+                    }
+            rb[b].count = n;
         }
         // on average at most two corrections a hand
         if (ties.size() > 2 * (size_t)h.H) { *why = "many tied hands"; return nullptr; }
@@ -439,21 +448,30 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
     }
     if (smem_bytes(nc) > (size_t)max_dyn_smem()) { *why = "shared memory"; return nullptr; }
     if (multi) {
-        // items of 32 columns, a tail of at most 16 split; all split when they
-        // still have an SM each (half as long)
-        auto count = [&](int n, int w) { return (n + w - 1) / w; };
-        long long n16 = 0;
-        for (int i = 0; i < ng; ++i) n16 += count(g[i].nunit, 16) + count(g[i].nrows - g[i].nunit, 16);
-        for (int unit = 0; unit < 2; ++unit)     // the longer items first
-            for (int i = 0; i < ng; ++i) {
-                const int n = unit ? g[i].nunit : g[i].nrows - g[i].nunit;
-                for (int c = 0; c < n;) {
-                    const bool half = n16 <= sms || n - c <= 16;
-                    const int e = std::min(n, c + (half ? 16 : 32));
-                    items.push_back(make_int4(i, c, e, (half ? 1 : 0) | (unit ? 2 : 0)));
-                    c = e;
+        // items of at least `least` parts, more where the columns left fill
+        // only one of the groups; returns their time in units of a whole item's
+        auto build = [&](int least, std::vector<int4> *out) {
+            double sum = 0.0;
+            long long n_items = 0;
+            for (int unit = 0; unit < 2; ++unit)     // the longer items first
+                for (int i = 0; i < ng; ++i) {
+                    const int n = unit ? g[i].nunit : g[i].nrows - g[i].nunit;
+                    for (int c = 0; c < n;) {
+                        int parts = least;
+                        while (parts < kParts && n - c <= 16 / parts) parts *= 2;
+                        const int e = std::min(n, c + 32 / parts);
+                        if (out) out->push_back(make_int4(i, c, e, parts | (unit ? 8 : 0)));
+                        sum += 1.0 / parts;
+                        ++n_items;
+                        c = e;
+                    }
                 }
-            }
+            return n_items <= sms ? 1.0 / least : sum / sms + 0.5 / least;
+        };
+        int least = 1;
+        for (int j = 2; j <= kParts; j *= 2)
+            if (build(j, nullptr) < build(least, nullptr)) least = j;
+        build(least, &items);
     }
     F64Plan *p = new (std::nothrow) F64Plan();
     if (!p) { *why = "host allocation"; return nullptr; }
@@ -529,9 +547,14 @@ cudaError_t launch_f64_scan(F64Plan *p, const double *vin, double *vout, int bat
         if (e != cudaSuccess) return e;
         const long long cu = (long long)p->nunit * batch, co = (long long)p->nother * batch;
         if (std::max(cu, co) > 0x7fffffe0LL) return cudaErrorInvalidValue;
-        // split items (half as long) while they have an SM each
-        a.split = (cu + 15) / 16 + (co + 15) / 16 <= sms ? 1 : 0;
-        const int w = a.split ? 16 : 32;
+        // the parts whose waves of items are shortest: 100 vectors of the river
+        // game make 91 items of 32 columns (218 us) or 364 of 8 (215 us)
+        auto items = [&](int j) { return (co + 32 / j - 1) / (32 / j) + (cu + 32 / j - 1) / (32 / j); };
+        auto time = [&](int j) { return (double)((items(j) + sms - 1) / sms) * (1.0 / j + 0.05); };
+        a.parts = 1;
+        for (int j = 2; j <= kParts; j *= 2)
+            if (time(j) < time(a.parts)) a.parts = j;
+        const int w = 32 / a.parts;
         a.nother = (int)((co + w - 1) / w);
         n = a.nother + (cu + w - 1) / w;
     }

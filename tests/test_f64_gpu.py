@@ -1,5 +1,5 @@
 """The FP64 product kernel at the sizes where it can go wrong: bit-exact on
-dyadic games (tie groups, items of 16 and of 32 columns), boards of 3 to 5
+dyadic games (tie groups, items of 8 to 32 columns), boards of 3 to 5
 cards, games it does not take, padding entries that hold NaN, and many games in
 one launch, against the oracle (1e-12 normwise, as every FP64 product).
 """
@@ -31,7 +31,7 @@ def _product(g, v, order, transpose):
 
 
 @pytest.mark.parametrize("ties", [False, True], ids=["river", "river_ties4"])
-@pytest.mark.parametrize("batch", [1, 5, 90])
+@pytest.mark.parametrize("batch", [1, 5, 90, 300])
 def test_river_bit_exact(ties, batch):
     spec = dyadic_river(seed=2, ties=ties)
     og, g = OracleGame(spec), kps.Game(spec)
