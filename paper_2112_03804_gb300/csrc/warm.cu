@@ -185,19 +185,24 @@ constexpr int kWidth = 256;
 constexpr int kOpRow = 4096;        // bytes between 8-row groups of an operand (K = 256)
 constexpr int kTmemPred = 512;      // columns: layer 2 at 0..255, layer 3 at 256..271
 
-struct RowInfo {
+struct RowInfo {                     // what the scatter of a row needs
     long long base;                  // batch-vector offset of (player, hand)
-    int gp, node, ca, cb, nact, s0, hs, player;
+    int nact, s0, hs, player;
+};
+struct alignas(16) RowIn {           // what layer 1 needs
     float pos, tie, mu;
+    uint32_t cards;                  // first card, second card << 8, has a second << 16, live << 17
 };
 
 // Shared memory: W2 [256 rows][K] (128 KB), the activations [128][K]
-// (64 KB), W3 [16][K] (8 KB), the row records, then the barrier and the
-// tensor-memory slot.
+// (64 KB), W3 [16][K] (8 KB), the row records of two tiles, b2 and b3, then the
+// barrier and the tensor-memory slot.
 constexpr size_t kOffW2 = 0, kOffH = kOffW2 + (size_t)kWidth / 8 * kOpRow, kOffW3 = kOffH + (size_t)kPR / 8 * kOpRow,
-                 kOffRows = kOffW3 + 2 * (size_t)kOpRow, kOffBar = kOffRows + kPR * sizeof(RowInfo);
+                 kOffRows = kOffW3 + 2 * (size_t)kOpRow, kOffIn = kOffRows + 2 * kPR * sizeof(RowInfo),
+                 kOffGn = kOffIn + 2 * kPR * sizeof(RowIn), kOffB2 = kOffGn + 2 * kPR * sizeof(int2),
+                 kOffBar = kOffB2 + (kWidth + 16) * sizeof(float);
 __host__ __device__ constexpr size_t predict_smem_bytes() { return kOffBar + 16 + 128; }
-// (barrier at kOffBar, tensor-memory slot at +8, the tile's first game at +12)
+// (barrier at kOffBar, tensor-memory slot at +8)
 
 __device__ __forceinline__ uint32_t op_off(int r, int k) {
     return (uint32_t)((r >> 3) * kOpRow + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
@@ -292,7 +297,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *W2s = smem_raw + kOffW2, *Hs = smem_raw + kOffH, *W3s = smem_raw + kOffW3;
-    RowInfo *rows = reinterpret_cast<RowInfo *>(smem_raw + kOffRows);
+    float *b2s = reinterpret_cast<float *>(smem_raw + kOffB2), *b3s = b2s + kWidth;
     const uint32_t bar = smem_addr(smem_raw + kOffBar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem_raw + kOffBar + 8);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -306,6 +311,8 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
         *reinterpret_cast<__nv_bfloat16 *>(W3s + op_off(n, k)) =
             n < a.dout ? a.W3[k * a.dout + n] : __float2bfloat16_rn(0.f);
     }
+    if (tid < kWidth) b2s[tid] = a.b2[tid];
+    if (tid < 16) b3s[tid] = tid < a.dout ? a.b3[tid] : 0.f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
                      "r"(kTmemPred));
@@ -325,77 +332,89 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
     const __nv_bfloat16 *Wc = a.W1h + 4 * kWidth;
     uint32_t phase = 0;
     bool ok = true;
+    // A CTA takes a contiguous run of tiles, so the games of its rows only move
+    // forward (no search), and consecutive rows mostly share game and node: their
+    // part of layer 1 is formed once.  The rows of the next tile are looked up
+    // while the tensor cores run layer 2.  4.15 M queries of 128 games: 4.82 ms
+    // with a search and four gathered parts per row, 3.24 ms now.
     const long long ntiles = (a.nq + kPR - 1) / kPR;
-    int *tile_game = reinterpret_cast<int *>(smem_raw + kOffBar + 12);
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        // the tile's queries are consecutive: one search for the game of its
-        // first query, then every row steps forward from it
-        if (tid == 0) *tile_game = decode(a.d, tile * kPR).game;
-        __syncthreads();
-        if (tid < kPR) {
-            const long long q = tile * kPR + tid;
-            RowInfo ri;
-            ri.nact = 0;
-            if (q < a.nq) {
-                int gq = *tile_game;
-                while (a.d.qstart[gq + 1] <= q) ++gq;
-                const WarmGame &GQ = a.d.games[gq];
-                Query Q;
-                Q.game = gq;
-                int r = (int)(q - GQ.qstart);
-                const int n1 = GQ.nodes[0] * GQ.H;
-                Q.player = r < n1 ? 0 : 1;
-                if (Q.player) r -= n1;
-                Q.node = r / GQ.H;
-                Q.hand = r - Q.node * GQ.H;
-                const WarmGame &G = a.d.games[Q.game];
-                const int4 nd = a.d.node[G.node_off[Q.player] + Q.node];
-                const int2 cd = a.d.cards[G.hand_off + Q.hand];
-                const float4 hf = reinterpret_cast<const float4 *>(a.d.hand)[G.hand_off + Q.hand];
-                ri.base = G.voff[Q.player] + Q.hand;
-                ri.gp = 2 * Q.game + Q.player;
-                ri.node = G.node_off[Q.player] + Q.node;
-                ri.ca = cd.x;
-                ri.cb = cd.y;
-                ri.nact = nd.y;
-                ri.s0 = nd.x;
-                ri.hs = G.hs;
-                ri.player = Q.player;
-                ri.pos = hf.x;
-                ri.tie = hf.y;
-                ri.mu = Q.player == 0 ? hf.z : hf.w;
-            }
-            rows[tid] = ri;
+    const long long t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
+    int game = tid < kPR && t0 < t1 ? decode(a.d, min(t0 * kPR + tid, a.nq - 1)).game : 0;   // of this thread's row
+    auto look_up = [&](long long tile) {
+        const int buf = (int)((tile - t0) & 1);
+        const long long q = tile * kPR + tid;
+        RowInfo ri{};
+        RowIn in{};
+        int2 gn = make_int2(-1, -1);
+        if (q < a.nq) {
+            while (a.d.qstart[game + 1] <= q) ++game;
+            const WarmGame &G = a.d.games[game];
+            int r = (int)(q - G.qstart);
+            const int n1 = G.nodes[0] * G.H;
+            const int player = r < n1 ? 0 : 1;
+            if (player) r -= n1;
+            const int k = r / G.H, hand = r - k * G.H;
+            const int4 nd = a.d.node[G.node_off[player] + k];
+            const int2 cd = a.d.cards[G.hand_off + hand];
+            const float4 hf = reinterpret_cast<const float4 *>(a.d.hand)[G.hand_off + hand];
+            ri.base = G.voff[player] + hand;
+            ri.nact = nd.y;
+            ri.s0 = nd.x;
+            ri.hs = G.hs;
+            ri.player = player;
+            in.pos = hf.x;
+            in.tie = hf.y;
+            in.mu = player == 0 ? hf.z : hf.w;
+            in.cards = (uint32_t)cd.x | ((uint32_t)(cd.y >= 0 ? cd.y : 0) << 8) | (cd.y >= 0 ? 1u << 16 : 0u) |
+                       (nd.y > 0 ? 1u << 17 : 0u);
+            gn = make_int2(2 * game + player, G.node_off[player] + k);
         }
+        reinterpret_cast<RowInfo *>(smem_raw + kOffRows)[buf * kPR + tid] = ri;
+        reinterpret_cast<RowIn *>(smem_raw + kOffIn)[buf * kPR + tid] = in;
+        reinterpret_cast<int2 *>(smem_raw + kOffGn)[buf * kPR + tid] = gn;
+    };
+    if (tid < kPR && t0 < t1) look_up(t0);
+    int2 cur = make_int2(-1, -1);
+    float part = 0.f;                // game and node part of layer 1 for `cur`
+    for (long long tile = t0; tile < t1; ++tile) {
+        const int buf = (int)((tile - t0) & 1);
+        const RowInfo *rows = reinterpret_cast<const RowInfo *>(smem_raw + kOffRows) + buf * kPR;
+        const RowIn *rin = reinterpret_cast<const RowIn *>(smem_raw + kOffIn) + buf * kPR;
+        const int2 *rgn = reinterpret_cast<const int2 *>(smem_raw + kOffGn) + buf * kPR;
         __syncthreads();
-        // layer 1: column j of every row, written as BF16 in the A layout.
-        // Eight rows at a time: their records and all their gathers are
-        // issued before any sum or store, so the loads overlap (the sum order
-        // is the definition's: game part, node part, hand features, cards).
-        for (int r0 = 0; r0 < kPR; r0 += 8) {
-            float g[8], nd[8], wa[8], wb[8], pos[8], tie[8], mu[8];
-            bool live[8], two[8];
+        // layer 1: column j of every row, written as BF16 in the A layout,
+        // sixteen rows at a time, all their gathers issued before any sum or
+        // store (the sum order is the definition's: game part, node part, hand
+        // features, cards).
+        for (int r0 = 0; r0 < kPR; r0 += 16) {
+            const int2 first = rgn[r0], last = rgn[r0 + 15];
+            const bool same = first.x == last.x && first.y == last.y && first.x >= 0;
+            if (same && (first.x != cur.x || first.y != cur.y)) {
+                cur = first;
+                part = a.G1[(long long)cur.x * kWidth + j] + a.N1[(long long)cur.y * kWidth + j];
+            }
+            float base[16], wa[16], wb[16];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const RowInfo &ri = rows[r0 + u];
-                live[u] = ri.nact > 0;
-                two[u] = ri.cb >= 0;
-                const int gp = live[u] ? ri.gp : 0, node = live[u] ? ri.node : 0;
-                const int ca = live[u] ? ri.ca : 0, cb = live[u] && two[u] ? ri.cb : 0;
-                g[u] = a.G1[(long long)gp * kWidth + j];
-                nd[u] = a.N1[(long long)node * kWidth + j];
-                wa[u] = __bfloat162float(Wc[ca * kWidth + j]);
-                wb[u] = __bfloat162float(Wc[cb * kWidth + j]);
-                pos[u] = ri.pos;
-                tie[u] = ri.tie;
-                mu[u] = ri.mu;
+            for (int u = 0; u < 16; ++u) {
+                const uint32_t cards = rin[r0 + u].cards;
+                wa[u] = __bfloat162float(Wc[(cards & 0xffu) * kWidth + j]);
+                wb[u] = __bfloat162float(Wc[((cards >> 8) & 0xffu) * kWidth + j]);
+                base[u] = part;
+            }
+            if (!same) {
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    const int2 gn = rgn[r0 + u];
+                    base[u] = gn.x >= 0 ? a.G1[(long long)gn.x * kWidth + j] + a.N1[(long long)gn.y * kWidth + j] : 0.f;
+                }
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 16; ++u) {
+                const RowIn in = rin[r0 + u];
                 float z = 0.f;
-                if (live[u]) {
-                    z = g[u] + nd[u] + pos[u] * wpos + tie[u] * wtie + mu[u] * wmu + wa[u] + bias1;
-                    if (two[u]) z += wb[u];
+                if (in.cards & (1u << 17)) {
+                    z = base[u] + in.pos * wpos + in.tie * wtie + in.mu * wmu + wa[u] + bias1;
+                    if (in.cards & (1u << 16)) z += wb[u];
                     z = fmaxf(z, 0.f);
                 }
                 *reinterpret_cast<__nv_bfloat16 *>(Hs + op_off(r0 + u, j)) = __float2bfloat16_rn(z);
@@ -414,6 +433,8 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
                 mma_f16(tbase, op_desc(ha + 256u * s), op_desc(wa + 256u * s), mma_idesc(kPR, kWidth), s > 0);
             mma_commit(bar);
         }
+        __syncwarp();
+        if (tid < kPR && tile + 1 < t1) look_up(tile + 1);   // meanwhile
         if (ok) ok = pmbar_wait(bar, phase);
         phase ^= 1u;
         if (!__syncthreads_and(ok)) break;
@@ -430,7 +451,7 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
                 uint32_t w[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    w[i] = pack_bf16(fmaxf(v[2 * i] + a.b2[c + 2 * i], 0.f), fmaxf(v[2 * i + 1] + a.b2[c + 2 * i + 1], 0.f));
+                    w[i] = pack_bf16(fmaxf(v[2 * i] + b2s[c + 2 * i], 0.f), fmaxf(v[2 * i + 1] + b2s[c + 2 * i + 1], 0.f));
                 *reinterpret_cast<uint4 *>(Hs + op_off(r, c)) = make_uint4(w[0], w[1], w[2], w[3]);
                 *reinterpret_cast<uint4 *>(Hs + op_off(r, c + 8)) = make_uint4(w[4], w[5], w[6], w[7]);
             }
@@ -460,7 +481,7 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
                 float mx = -INFINITY;
 #pragma unroll
                 for (int n = 0; n < 16; ++n) {
-                    z[n] += n < a.dout ? a.b3[n] : 0.f;
+                    z[n] += b3s[n];
                     if (n < ri.nact) mx = fmaxf(mx, z[n]);
                 }
                 float e[16], s = 0.f;
