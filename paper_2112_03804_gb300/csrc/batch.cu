@@ -58,32 +58,41 @@ int tmem_min_warps(kps_batch *b) {
 
 }  // namespace
 
+namespace {
+// The staged kernel's view of the batch's games in a direction.
+std::vector<kps::AmGameDesc> am_descs(const kps_batch *b, int dir) {
+    const int ng = (int)b->games.size();
+    std::vector<kps::AmGameDesc> d(ng);
+    for (int i = 0; i < ng; ++i) {
+        const kps_game *g = b->games[i];
+        const kps::HostGame &h = g->host;
+        kps::AmGameDesc &x = d[i];
+        x.h = &h;
+        x.lam_in = dir == 0 ? h.lam2.data() : h.lam1.data();
+        x.lam_out = dir == 0 ? h.lam1.data() : h.lam2.data();
+        x.n_out = dir == 0 ? h.n[0] : h.n[1];
+        x.fcol = g->dev.fcol[dir];
+        x.scol = g->dev.scol[dir];
+        x.fcoef = g->dev.fcoef_f[dir];
+        x.scoef = g->dev.scoef_f[dir];
+        x.hfcol = g->fcol[dir].data();
+        x.hscol = g->scol[dir].data();
+        x.in_off = b->off[dir == 0 ? 1 : 0][i];
+        x.out_off = b->off[dir == 0 ? 0 : 1][i];
+    }
+    return d;
+}
+}  // namespace
+
 bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
     if (b->am_state != 0) return b->am_state == 1;
     b->am_state = -1;
     const int ng = (int)b->games.size();
     for (int dir = 0; dir < 2; ++dir) {
-        std::vector<kps::AmGameDesc> d(ng);
-        for (int i = 0; i < ng; ++i) {
-            const kps_game *g = b->games[i];
-            const kps::HostGame &h = g->host;
-            kps::AmGameDesc &x = d[i];
-            x.h = &h;
-            x.lam_in = dir == 0 ? h.lam2.data() : h.lam1.data();
-            x.lam_out = dir == 0 ? h.lam1.data() : h.lam2.data();
-            x.n_out = dir == 0 ? h.n[0] : h.n[1];
-            x.fcol = g->dev.fcol[dir];
-            x.scol = g->dev.scol[dir];
-            x.fcoef = g->dev.fcoef_f[dir];
-            x.scoef = g->dev.scoef_f[dir];
-            x.hfcol = g->fcol[dir].data();
-            x.hscol = g->scol[dir].data();
-            x.in_off = b->off[dir == 0 ? 1 : 0][i];
-            x.out_off = b->off[dir == 0 ? 0 : 1][i];
-        }
+        const std::vector<kps::AmGameDesc> d = am_descs(b, dir);
         std::string why;
         std::vector<char> taken;
-        b->am[dir] = kps::am_create(d, 2 * sm_count(), stream, &taken, &why);
+        b->am[dir] = kps::am_create(d, 2 * sm_count(), false, stream, &taken, &why);
         bool ok = b->am[dir] != nullptr && kps::am_ctas_per_sm(b->am[dir]) >= 1;
         if (ok && dir == 1) ok = b->am_rest.size() == taken.size();
         for (int i = 0; ok && i < ng; ++i) {
@@ -125,6 +134,17 @@ bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
     }
     b->am_state = 1;
     return true;
+}
+
+bool batch_plain_ready(kps_batch *b, cudaStream_t stream) {
+    if (!batch_staged_ready(b, stream)) return false;
+    for (int dir = 0; dir < 2 && (!b->am_plain[0] || !b->am_plain[1]); ++dir) {
+        std::string why;
+        std::vector<char> taken;
+        kps::am_destroy(b->am_plain[dir]);
+        b->am_plain[dir] = kps::am_create(am_descs(b, dir), 2 * sm_count(), true, stream, &taken, &why);
+    }
+    return b->am_plain[0] && b->am_plain[1];
 }
 
 namespace {
@@ -324,7 +344,8 @@ bool batch_f64_ready(kps_batch *b, cudaStream_t stream) {
     return true;
 }
 
-kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream) {
+kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream,
+                        bool plain) {
     if (!b) return fail(KPS_EINVAL, "batch is NULL");
     if (dtype_size(dt) == 0) return fail(KPS_EINVAL, "unknown dtype");
     if (!vin || !vout) return fail(KPS_EINVAL, "vector pointer is NULL");
@@ -351,7 +372,8 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
         cudaError_t e = cudaSuccess;
         if (s.schedule == 0) e = cudaMemsetAsync(b->ticket, 0, sizeof(int), stream);
         if (e != cudaSuccess) return cuda_fail(e, "clearing the work-item ticket");
-        e = kps::launch_async_multi(b->am[dir], storage_of(dt), vin, vout, b->ticket, s.schedule, s.grid, stream);
+        kps::AmPlan *am = plain && b->am_plain[0] && b->am_plain[1] ? b->am_plain[dir] : b->am[dir];
+        e = kps::launch_async_multi(am, storage_of(dt), vin, vout, b->ticket, s.schedule, s.grid, stream);
         if (e != cudaSuccess) return cuda_fail(e, "launching the staged batched payoff scan");
         if (b->am_nrest > 0) {
             // the games the staged kernel leaves: tensor-memory kernel, static stride
@@ -423,6 +445,7 @@ kps_status kps_batch_destroy(kps_batch *b) {
     for (auto &kv : b->tables) cudaFree(kv.second.blob);
     for (auto &kv : b->rest_tables) cudaFree(kv.second.blob);
     for (int k = 0; k < 2; ++k) kps::am_destroy(b->am[k]);
+    for (int k = 0; k < 2; ++k) kps::am_destroy(b->am_plain[k]);
     for (int k = 0; k < 2; ++k) kps::f64_destroy(b->f64[k]);
     warm_free(b);
     if (b->ticket) cudaFree(b->ticket);

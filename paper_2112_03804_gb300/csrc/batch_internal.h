@@ -40,6 +40,7 @@ struct kps_batch {
     std::map<int, kps_abi::BatchShape> shape;   // per dtype
     void *warm = nullptr;            // warm-start feature tables (warm.cu)
     kps::AmPlan *am[2] = {nullptr, nullptr};   // staged FP32 kernel, per direction
+    kps::AmPlan *am_plain[2] = {nullptr, nullptr};   // the same with plain rows (the solver's)
     int am_state = 0;                // 0 not tried, 1 built, -1 it takes no game
     std::vector<char> am_rest;       // per game: 1 when the staged kernel leaves it to the tensor-memory one
     int am_nrest = 0;
@@ -57,7 +58,12 @@ kps_status batch_table(kps_batch *b, int dir, bool f64, int nw, cudaStream_t str
 kps_status batch_rest_table(kps_batch *b, int dir, cudaStream_t stream, const BatchTable **out);
 kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, BatchShape *out);
 // dir 0: out = A y per game (y player-2 layout, out player-1 layout); dir 1: A^T.
-kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream);
+// plain: the staged kernel's plain rows where batch_plain_ready built them.
+kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream,
+                        bool plain = false);
+// Builds the plans of plain rows (host work, synchronises `stream`); false
+// when the staged kernel does not serve this batch.
+bool batch_plain_ready(kps_batch *b, cudaStream_t stream);
 // Builds the staged kernel's plans on first use (host work, synchronises
 // `stream`); true when every game fits that kernel.
 bool batch_staged_ready(kps_batch *b, cudaStream_t stream);

@@ -228,9 +228,12 @@ struct AmPlan;
 // Builds and uploads the plan (synchronises `stream`) for the games this
 // path takes ((*taken)[i] = 1; the others, e.g. with a tie group longer than
 // 4 hands, get no work items); nullptr when it takes none or on a failure,
-// *why set.  Scratch for `grid_cap` CTAs.
-AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream_t stream, std::vector<char> *taken,
-                  std::string *why);
+// *why set.  Scratch for `grid_cap` CTAs.  plain: one sequence per row, items of
+// 32 rows, every row scanned with its own payoffs (the solver's products, whose
+// roundings must not depend on how rows are grouped: a regret within rounding
+// of the matching floor decides a strategy entry).
+AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
+                  std::vector<char> *taken, std::string *why);
 void am_destroy(AmPlan *p);
 int am_ctas_per_sm(const AmPlan *p);
 int am_grid_cap(const AmPlan *p);

@@ -81,6 +81,7 @@ struct AmArgs {
     const AmGame *games;
     const int4 *items;             // (game, first row, split, last row + 1)
     int nitems, nc, schedule;
+    int unit;                      // showdown-only rows are scanned with S = 1
     const void *vin;               // element type: the kernel's storage type
     void *vout;
     float *scratch;                // [grid][4 warps][kMaxExtra][16][32]
@@ -219,7 +220,7 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
     const float F = rf >= 0 ? G.fcoef[sigma] : 0.f;
     // a showdown-only row is scanned with S = 1 and finished with its payoff;
     // Fm: the payoff of its fold-only mate
-    const bool unit = rf < 0 && rs >= 0;
+    const bool unit = P.unit && rf < 0 && rs >= 0;
     const float S = unit ? 1.f : rs >= 0 ? G.scoef[sigma] : 0.f;
     const float So = unit ? G.scoef[sigma] : 1.f, Fm = sq.y >= 0 ? G.fcoef[sq.y] : 0.f;
     const bool pairs = __any_sync(kFull, sq.y >= 0);
@@ -629,8 +630,8 @@ struct AmPlan {
     int device = -1;
 };
 
-AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream_t stream, std::vector<char> *taken,
-                  std::string *why) {
+AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
+                  std::vector<char> *taken, std::string *why) {
     if (games.empty() || grid_cap < 1) {
         *why = "no games";
         return nullptr;
@@ -749,7 +750,7 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
     double best = 0.0;
     const std::vector<std::vector<int2>> *rows = nullptr;
     bool halves = false;
-    for (int v = 0; v < 4; ++v) {
+    for (int v = plain ? 1 : 0; v < (plain ? 2 : 4); ++v) {
         const auto &rv = v & 1 ? single : paired;
         const double t = layout(rv, (v & 2) != 0, nullptr);
         if (!rows || t < best) {
@@ -835,6 +836,7 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream
     }
     p->a.games = reinterpret_cast<const AmGame *>(dev + o_games);
     p->a.items = reinterpret_cast<const int4 *>(dev + o_items);
+    p->a.unit = plain ? 0 : 1;
     p->a.nitems = (int)nitems;
     p->a.nc = nc;
     p->k = k;

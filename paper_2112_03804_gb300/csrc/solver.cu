@@ -43,6 +43,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "abi_internal.h"
@@ -141,10 +142,11 @@ struct UpdateArgs {
 
 // One node of the bottom-up walk with NA actions (exactly unrolled; NA = 0:
 // the node's own count na, up to kMaxActions, predicated): regrets updated
-// from the action values, the node's value added into its parent's slot.
+// from the action values (sign times the slots), the node's value added into
+// its parent's slot.
 template <int NA, typename C, int BW>
 __device__ __forceinline__ void up_node(C *qv, C *rg, int s0, int na, int par, bool init, const float *beh0,
-                                        long long hs, C theta, int method, C dpos, C dneg) {
+                                        long long hs, C theta, int method, C dpos, C dneg, C sign) {
     constexpr int M = NA > 0 ? NA : kMaxActions;
     if (NA > 0) na = NA;
     C r[M], b[M], q[M];
@@ -152,7 +154,7 @@ __device__ __forceinline__ void up_node(C *qv, C *rg, int s0, int na, int par, b
     for (int a = 0; a < M; ++a)
         if (a < na) {
             r[a] = rg[(s0 + a) * BW];
-            q[a] = qv[(s0 + a) * BW];
+            q[a] = sign * qv[(s0 + a) * BW];
         }
     if (init) {
 #pragma unroll
@@ -177,7 +179,7 @@ __device__ __forceinline__ void up_node(C *qv, C *rg, int s0, int na, int par, b
             const C rn = r[a] + q[a] - v;
             rg[(s0 + a) * BW] = method == 0 ? (rn > C(0) ? rn : C(0)) : rn * (rn > C(0) ? dpos : dneg);
         }
-    if (par >= 0) qv[par * BW] += v;
+    if (par >= 0) qv[par * BW] += sign * v;
 }
 
 // One node of the top-down walk: the next behavioural strategy by regret
@@ -211,6 +213,8 @@ __device__ __forceinline__ void down_node(C *qv, const C *rg, int s0, int na, in
 // the new sequence form), and regrets and strategy are written back last.
 // At least 10 resident 64-thread blocks per SM for 16- and 32-bit
 // accumulators (the kernel is latency bound); FP64 keeps its registers.
+// (Values and regrets by asynchronous copies, all in flight at once, took 144
+// instead of 133 us on 256 river games: the loads are not what it waits for.)
 template <typename S, typename C, int BW>
 __global__ void __launch_bounds__(BW, sizeof(C) == 8 ? 1 : 640 / BW) rm_update_kernel(const UpdateArgs<S, C> u) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(BW, sizeof(C) == 8 ? 1 : 640 / BW) rm_update_k
 #pragma unroll 4
     for (int s = 0; s < n; ++s) {
         const long long i = (long long)s * hs;
-        qv[s * BW] = u.sign * C(Cv<S>::ld(gp + i));
+        qv[s * BW] = C(Cv<S>::ld(gp + i));
         rg[s * BW] = Rp[i];
         xsp[i] += wt * C(Cv<S>::ld(xp + i));
     }
@@ -249,20 +253,23 @@ __global__ void __launch_bounds__(BW, sizeof(C) == 8 ? 1 : 640 / BW) rm_update_k
     // action count picks an exactly unrolled step; the branch is uniform
     // over the block, whose threads are hands of one game)
     const float *beh0 = u.beh0 ? u.beh0 + base : nullptr;
+    int4 next = nn > 0 ? nodes[nn - 1] : make_int4(0, 0, 0, 0);   // the next node's record, one node ahead
     for (int k = nn - 1; k >= 0; --k) {
-        const int4 nd = nodes[k];
+        const int4 nd = next;
+        next = nodes[k > 0 ? k - 1 : 0];
         const int s0 = nd.x, na = nd.y, par = nd.z;
         switch (na) {
-            case 2: up_node<2, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
-            case 3: up_node<3, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
-            case 4: up_node<4, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
-            case 5: up_node<5, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
-            case 6: up_node<6, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
-            default: up_node<0, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg); break;
+            case 2: up_node<2, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
+            case 3: up_node<3, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
+            case 4: up_node<4, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
+            case 5: up_node<5, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
+            case 6: up_node<6, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
+            default: up_node<0, C, BW>(qv, rg, s0, na, par, init, beh0, hs, theta, u.method, dpos, dneg, u.sign); break;
         }
     }
     for (int k = 0; k < nn; ++k) {
-        const int4 nd = nodes[k];
+        const int4 nd = next;
+        next = nodes[k + 1 < nn ? k + 1 : k];
         const int s0 = nd.x, na = nd.y, par = nd.z;
         switch (na) {
             case 2: down_node<2, C, BW>(qv, rg, s0, na, par, theta); break;
@@ -328,9 +335,19 @@ __global__ void __launch_bounds__(BW) average_kernel(const UpdateArgs<S, C> u, O
     const int p = u.player, hs = G.hs;
     const long long base = G.off[p] + w.h;
     const double wsum = *u.wsum;
+    // FP32 sums: the quotient by wsum as a product with its rounded reciprocal
+    // and one correction by the remainder, which rounds as the division does
+    // (Markstein 1990); three FP64 instructions on a pipe that starts one per SM
+    // about every 16 cycles, where the division took most of the kernel's time
+    // (256 river games: 205 -> 109 us).  The quotient cannot be subnormal.
+    const double rw = wsum > 0.0 ? 1.0 / wsum : 0.0;
     auto avg = [&](int s) -> double {
         const long long i = base + (long long)s * hs;
-        return wsum > 0.0 ? (double)u.xsum[i] / wsum : (double)Cv<S>::ld(u.x + i);
+        if (!(wsum > 0.0)) return (double)Cv<S>::ld(u.x + i);
+        const C xs = u.xsum[i];
+        if (sizeof(C) == 8 || !isfinite(xs)) return (double)xs / wsum;
+        const double x = (double)xs, q = x * rw;
+        return fma(fma(-q, wsum, x), rw, q);
     };
     const int4 *nodes = u.nodes + G.node_off[p];
     for (int k = 0; k < G.nnodes[p]; ++k) {
@@ -532,11 +549,11 @@ cudaError_t average32_t(kps_solver *s, int p, float *out, cudaStream_t st) {
                         : F<__half, float>(__VA_ARGS__))
 
 kps_status one_iteration(kps_solver *s, cudaStream_t st) {
-    kps_status r = batch_matvec(s->batch, 0, s->x[1], s->g[0], s->dt, st);
+    kps_status r = batch_matvec(s->batch, 0, s->x[1], s->g[0], s->dt, st, true);
     if (r != KPS_OK) return r;
     cudaError_t e = KPS_DISPATCH(s->dt, update_t, s, 0, st);
     if (e != cudaSuccess) return cuda_fail(e, "player-1 update");
-    r = batch_matvec(s->batch, 1, s->x[0], s->g[1], s->dt, st);
+    r = batch_matvec(s->batch, 1, s->x[0], s->g[1], s->dt, st, true);
     if (r != KPS_OK) return r;
     e = KPS_DISPATCH(s->dt, update_t, s, 1, st);
     if (e != cudaSuccess) return cuda_fail(e, "player-2 update");
@@ -551,18 +568,39 @@ kps_status one_iteration(kps_solver *s, cudaStream_t st) {
 // has gone wrong, and the averages and exploitability carry it from then on
 // (RM+'s max(0, .) turns a NaN regret into 0, so the regrets alone can look
 // clean while the averages are not).
+// Reads 16 bytes at a time (all three arrays are allocations of a multiple of
+// 8 entries) and looks at the exponent bits alone: 256 river games, FP32, 121 ->
+// 28 us (one entry per step, through FP64 tests, before).
+__device__ __forceinline__ bool bad16(uint4 v, uint32_t exp32) {
+    return (v.x & exp32) == exp32 || (v.y & exp32) == exp32 || (v.z & exp32) == exp32 || (v.w & exp32) == exp32;
+}
+template <typename T>
+__device__ __forceinline__ bool bad_values(const T *p, long long n) {
+    constexpr int per = 16 / (int)sizeof(T);
+    constexpr uint32_t lo = std::is_same<T, __half>::value ? 0x7c00u : std::is_same<T, __nv_bfloat16>::value ? 0x7f80u : 0u;
+    const uint4 *q = reinterpret_cast<const uint4 *>(p);
+    const long long step = (long long)gridDim.x * blockDim.x, m = n / per;
+    bool bad = false;
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += step) {
+        const uint4 v = q[i];
+        if (sizeof(T) == 8) bad = bad || (v.y & 0x7ff00000u) == 0x7ff00000u || (v.w & 0x7ff00000u) == 0x7ff00000u;
+        else if (sizeof(T) == 4) bad = bad || bad16(v, 0x7f800000u);
+        else bad = bad || bad16(v, lo) || bad16(v, lo << 16);
+    }
+    return bad;
+}
 template <typename S, typename C>
-__global__ void nonfinite_kernel(const C *regret, const C *xsum, const S *x, long long n, unsigned int *bad) {
-    bool ok = true;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        ok = ok && isfinite((double)regret[i]) && isfinite((double)xsum[i]) && isfinite((double)Cv<S>::ld(x + i));
-    if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicOr(bad, 1u);
+__global__ void __launch_bounds__(256) nonfinite_kernel(const C *regret, const C *xsum, const S *x, long long n,
+                                                        unsigned int *bad) {
+    const bool b1 = bad_values(regret, n), b2 = bad_values(xsum, n), b3 = bad_values(x, n);
+    if (__syncthreads_or(b1 || b2 || b3) && threadIdx.x == 0) atomicOr(bad, 1u);
 }
 
 template <typename S, typename C>
 cudaError_t nonfinite_t(kps_solver *s, int p, cudaStream_t st) {
     const long long n = s->batch->off[p].back();
-    const int blocks = (int)std::min<long long>(1024, (n + 255) / 256);
+    const int blocks = (int)std::min<long long>(1024, (n + 2047) / 2048);
     if (blocks <= 0) return cudaSuccess;
     nonfinite_kernel<S, C><<<blocks, 256, 0, st>>>(static_cast<const C *>(s->regret[p]),
                                                     static_cast<const C *>(s->xsum[p]),
@@ -785,6 +823,7 @@ kps_status kps_solver_create(kps_batch *b, kps_dtype dt, kps_solver **out) {
         }
         if (st != KPS_OK) { free_solver(s); return st; }
     }
+    if (dt != KPS_F64) batch_plain_ready(b, nullptr);
     // one iteration outside any capture sets every kernel attribute; then start over
     kps_status st = kps_solver_reset(s, nullptr, nullptr, nullptr);
     if (st == KPS_OK) st = one_iteration(s, nullptr);
