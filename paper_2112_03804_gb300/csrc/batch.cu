@@ -370,9 +370,11 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
     if (st != KPS_OK) return st;
     if (s.kernel == KPS_BATCH_STAGED) {
         cudaError_t e = cudaSuccess;
+        kps::AmPlan *am = plain && b->am_plain[0] && b->am_plain[1] ? b->am_plain[dir] : b->am[dir];
+        // no ticket to clear where every CTA has at most one item
+        if (kps::am_items(am) <= s.grid) s.schedule = 1;
         if (s.schedule == 0) e = cudaMemsetAsync(b->ticket, 0, sizeof(int), stream);
         if (e != cudaSuccess) return cuda_fail(e, "clearing the work-item ticket");
-        kps::AmPlan *am = plain && b->am_plain[0] && b->am_plain[1] ? b->am_plain[dir] : b->am[dir];
         e = kps::launch_async_multi(am, storage_of(dt), vin, vout, b->ticket, s.schedule, s.grid, stream);
         if (e != cudaSuccess) return cuda_fail(e, "launching the staged batched payoff scan");
         if (b->am_nrest > 0) {

@@ -237,6 +237,7 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain
 void am_destroy(AmPlan *p);
 int am_ctas_per_sm(const AmPlan *p);
 int am_grid_cap(const AmPlan *p);
+int am_items(const AmPlan *p);        // work items of a launch
 // One product over every game; ticket: a device counter cleared before the
 // launch when schedule == 0 (ticket), unused when 1 (static stride).
 cudaError_t launch_async_multi(AmPlan *p, int storage, const void *vin, void *vout, int *ticket, int schedule,

@@ -857,6 +857,8 @@ static size_t am_launch_smem(int nc) { return std::max<size_t>(am_smem_bytes(nc)
 
 int am_grid_cap(const AmPlan *p) { return p->grid_cap; }
 
+int am_items(const AmPlan *p) { return p->a.nitems; }
+
 int am_ctas_per_sm(const AmPlan *p) {
     const size_t smem = am_launch_smem(p->a.nc);
     int dev = 0, per_sm = 0, reserved = 0;

@@ -99,17 +99,36 @@ __device__ __forceinline__ Where locate(const SolverGame *games, const int *bloc
 }
 
 // Regret matching of one node: b[a] = R+[a] / sum, uniform if the sum is
-// at most the noise floor theta.
-template <typename C>
+// at most the noise floor theta.  The quotients share the rounded reciprocal of
+// the sum; one correction by the remainder rounds each as the division does
+// (Markstein 1990; away from the ends of the exponent range, where the division
+// itself is taken), in three instructions an action.
+template <int M, typename C>
 __device__ __forceinline__ void regret_match(const C *r, int na, C *b, C theta) {
     // positive parts (RM+ regrets are never negative; DCFR's may be)
     C sum = C(0);
 #pragma unroll
-    for (int a = 0; a < kMaxActions; ++a)
+    for (int a = 0; a < M; ++a)
         if (a < na) sum += r[a] > C(0) ? r[a] : C(0);
+    const C one = C(1) / (sum > theta ? sum : C(na));   // 1 / na when uniform
+    if (!(sum > theta)) {
 #pragma unroll
-    for (int a = 0; a < kMaxActions; ++a)
-        if (a < na) b[a] = sum > theta ? (r[a] > C(0) ? r[a] : C(0)) / sum : C(1) / C(na);
+        for (int a = 0; a < M; ++a)
+            if (a < na) b[a] = one;
+    } else if (sum > C(1e-30) && sum < C(1e30)) {
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+            if (a < na) {
+                const C p = r[a] > C(0) ? r[a] : C(0), q = p * one;
+                b[a] = fma(fma(-q, sum, p), one, q);
+            }
+    } else {
+#pragma unroll 1
+        for (int a = 0; a < M; ++a)
+#pragma unroll
+            for (int k = 0; k < M; ++k)
+                if (k == a && a < na) b[k] = (r[k] > C(0) ? r[k] : C(0)) / sum;
+    }
 }
 
 // Weight of iteration t in the average: t (RM+) or t^gamma (DCFR, from the
@@ -161,13 +180,7 @@ __device__ __forceinline__ void up_node(C *qv, C *rg, int s0, int na, int par, b
         for (int a = 0; a < M; ++a)
             if (a < na) b[a] = C(beh0[(long long)(s0 + a) * hs]);
     } else {
-        C sum = C(0);
-#pragma unroll
-        for (int a = 0; a < M; ++a)
-            if (a < na) sum += r[a] > C(0) ? r[a] : C(0);
-#pragma unroll
-        for (int a = 0; a < M; ++a)
-            if (a < na) b[a] = sum > theta ? (r[a] > C(0) ? r[a] : C(0)) / sum : C(1) / C(na);
+        regret_match<M>(r, na, b, theta);
     }
     C v = C(0);
 #pragma unroll
@@ -192,13 +205,7 @@ __device__ __forceinline__ void down_node(C *qv, const C *rg, int s0, int na, in
 #pragma unroll
     for (int a = 0; a < M; ++a)
         if (a < na) r[a] = rg[(s0 + a) * BW];
-    C sum = C(0);
-#pragma unroll
-    for (int a = 0; a < M; ++a)
-        if (a < na) sum += r[a] > C(0) ? r[a] : C(0);
-#pragma unroll
-    for (int a = 0; a < M; ++a)
-        if (a < na) b[a] = sum > theta ? (r[a] > C(0) ? r[a] : C(0)) / sum : C(1) / C(na);
+    regret_match<M>(r, na, b, theta);
     const C xpar = par >= 0 ? qv[par * BW] : C(1);
 #pragma unroll
     for (int a = 0; a < M; ++a)
