@@ -172,16 +172,13 @@ kps_status tiles_for(kps_game *g, int nw, cudaStream_t stream, const kps_game::T
             std::memcpy(blob.data() + n * sizeof(int2), w2.data(), n * sizeof(int2));
         }
         if (!trip.empty()) std::memcpy(blob.data() + 2 * n * sizeof(int2), trip.data(), trip.size() * sizeof(uint32_t));
-        cudaError_t e = cudaMalloc(&t.dev, bytes);
-        if (e != cudaSuccess) return fail(KPS_ENOMEM, "tile table");
+        void *dev = nullptr;
+        const cudaError_t e = kps::upload_table(&dev, blob.data(), bytes, stream);
+        if (e == cudaErrorMemoryAllocation) return fail(KPS_ENOMEM, "tile table");
+        if (e != cudaSuccess) return cuda_fail(e, "uploading the tile table");
+        t.dev = static_cast<int2 *>(dev);
         t.tie_work = t.dev + n;
         t.tie_trip = reinterpret_cast<uint32_t *>(t.dev + 2 * n);
-        e = cudaMemcpyAsync(t.dev, blob.data(), bytes, cudaMemcpyHostToDevice, stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-        if (e != cudaSuccess) {
-            cudaFree(t.dev);
-            return cuda_fail(e, "uploading the tile table");
-        }
         it = g->tiles.emplace(nw, std::move(t)).first;
     }
     *out = &it->second;

@@ -457,6 +457,30 @@ cudaError_t ensure_dyn_smem(const void *fn, size_t smem) {
     return cudaSuccess;
 }
 
+cudaError_t upload_table(void **dev, const void *src, size_t bytes, cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) return e;
+    const bool own = cap != cudaStreamCaptureStatusNone;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (own) {
+        e = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) return e;
+        e = cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
+    }
+    void *p = nullptr;
+    if (e == cudaSuccess) {
+        e = cudaMalloc(&p, bytes);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (own) cudaStreamDestroy(stream);
+    }
+    if (e != cudaSuccess && p) cudaFree(p);
+    if (own) cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) *dev = p;
+    return e;
+}
+
 int max_dyn_smem() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;

@@ -43,6 +43,12 @@ int max_dyn_smem();
 // on the current device (set once per kernel, device and size; thread safe).
 cudaError_t ensure_dyn_smem(const void *fn, size_t smem);
 
+// New device memory in *dev with a copy of the host bytes, there when the call
+// returns.  On a capturing stream the copy goes through a stream of its own (a
+// table is not a part of the graph, and a captured product may be the first
+// one to need it).  On an error nothing is allocated.
+cudaError_t upload_table(void **dev, const void *src, size_t bytes, cudaStream_t stream);
+
 cudaError_t launch_pair_scan(const ScanParams &p, int storage, int cards_per_hand,
                              bool partial_in_smem, cudaStream_t stream);
 

@@ -630,8 +630,9 @@ struct AmPlan {
     int device = -1;
 };
 
-AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                  std::vector<char> *taken, std::string *why) {
+namespace {
+AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
+                   std::vector<char> *taken, std::string *why) {
     if (games.empty() || grid_cap < 1) {
         *why = "no games";
         return nullptr;
@@ -776,6 +777,8 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain
     const size_t o_games = 0, o_items = al(sizeof(AmGame) * ng), o_rows = o_items + al(sizeof(int4) * (size_t)nitems),
                  o_rec = o_rows + al(sizeof(int2) * nrows);
     const size_t total = o_rec + rbytes;
+    std::vector<unsigned char> host(total, 0);
+    std::vector<AmGame> g(ng);
     AmPlan *p = new (std::nothrow) AmPlan();
     if (!p) {
         *why = "host allocation";
@@ -792,8 +795,6 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain
     }
     p->grid_cap = grid_cap;
     unsigned char *dev = static_cast<unsigned char *>(p->blob);
-    std::vector<unsigned char> host(total, 0);
-    std::vector<AmGame> g(ng);
     size_t ro = o_rec, rowo = o_rows;
     for (int i = 0; i < ng; ++i) {
         const AmGameDesc &d = games[i];
@@ -842,6 +843,17 @@ AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain
     p->k = k;
     cudaGetDevice(&p->device);
     return p;
+}
+}  // namespace
+
+AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
+                  std::vector<char> *taken, std::string *why) {
+    try {
+        return build_plan(games, grid_cap, plain, stream, taken, why);
+    } catch (const std::bad_alloc &) {
+        *why = "host allocation";
+        return nullptr;
+    }
 }
 
 void am_destroy(AmPlan *p) {

@@ -901,6 +901,37 @@ static std::string tma_prepare(const HostGame &h, const double *lam_in, const do
     return "";
 }
 
+// Items after the records: first the pairs (a fold-only sequence goes with the
+// first showdown-only one of its input row) and what is left alone, then every
+// sequence alone.
+std::string tma_items(int n_out, const int *hfcol, const int *hscol, TmaParams &p) {
+    std::vector<int2> items;
+    std::vector<int> fold_of;   // by input row: its first fold-only sequence, -1 once taken
+    std::vector<int> mate(n_out, -1);
+    std::vector<char> taken(n_out, 0);
+    for (int r = 0; r < n_out; ++r) {
+        if (hfcol[r] < 0 && hscol[r] < 0) return "an output sequence without terminals";
+        if (hscol[r] >= 0 || p.a.nc < kPairMinCards) continue;
+        if (hfcol[r] >= (int)fold_of.size()) fold_of.resize(hfcol[r] + 1, -1);
+        if (fold_of[hfcol[r]] < 0) fold_of[hfcol[r]] = r;
+    }
+    for (int r = 0; r < n_out; ++r) {
+        if (hfcol[r] >= 0 || hscol[r] >= (int)fold_of.size()) continue;
+        mate[r] = fold_of[hscol[r]];
+        fold_of[hscol[r]] = -1;
+        if (mate[r] >= 0) taken[mate[r]] = 1;
+    }
+    for (int r = 0; r < n_out; ++r)
+        if (!taken[r]) items.push_back(make_int2(r, mate[r]));
+    p.npaired = (int)items.size();
+    p.nsingle = n_out;
+    for (int r = 0; r < n_out; ++r) items.push_back(make_int2(r, -1));
+    p.o_items = (p.host.size() + 15) / 16 * 16;
+    p.host.resize(p.o_items + sizeof(int2) * items.size());
+    if (!items.empty()) std::memcpy(p.host.data() + p.o_items, items.data(), sizeof(int2) * items.size());
+    return "";
+}
+
 }  // namespace kps
 
 namespace kps {
@@ -916,29 +947,10 @@ TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam
     std::string w;
     try {
         w = tma_prepare(h, lam_in, lam_out, *p);
+        if (w.empty()) w = tma_items(n_out, hfcol, hscol, *p);
     } catch (const std::bad_alloc &) {
         w = "host allocation";
     }
-    // items: a fold-only sequence goes with the showdown-only one of its input row
-    std::vector<int2> items;
-    std::vector<int> mate(n_out, -1);
-    std::vector<char> taken(n_out, 0);
-    for (int r = 0; r < n_out && w.empty(); ++r) {
-        if (hfcol[r] < 0 && hscol[r] < 0) w = "an output sequence without terminals";
-        for (int q = 0; q < n_out && hfcol[r] < 0 && mate[r] < 0 && p->a.nc >= kPairMinCards; ++q)
-            if (hscol[q] < 0 && hfcol[q] == hscol[r] && !taken[q]) {
-                mate[r] = q;
-                taken[q] = 1;
-            }
-    }
-    for (int r = 0; r < n_out; ++r)
-        if (!taken[r]) items.push_back(make_int2(r, mate[r]));
-    p->npaired = (int)items.size();
-    p->nsingle = n_out;
-    for (int r = 0; r < n_out; ++r) items.push_back(make_int2(r, -1));
-    p->o_items = (p->host.size() + 15) / 16 * 16;
-    p->host.resize(p->o_items + sizeof(int2) * items.size());
-    if (!items.empty()) std::memcpy(p->host.data() + p->o_items, items.data(), sizeof(int2) * items.size());
     if (w.empty() && std::max<size_t>(tma_smem_bytes(kTmaWarps, p->a.nc, p->extra4), 80 * 1024) > (size_t)max_dyn_smem())
         w = "shared memory";
     if (!w.empty()) {
@@ -972,26 +984,19 @@ void tma_destroy(TmaParams *p) {
 
 cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *vout, int batch, cudaStream_t stream) {
     TmaParams &p = *pp;
-    TmaArgs &A = p.a;
     cudaError_t e;
     if (!p.dev) {
         // the record tables go to the device on the first product
-        e = cudaMalloc(&p.dev, p.host.size());
+        e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p.a.err), g_tma_err);
         if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(p.dev, p.host.data(), p.host.size(), cudaMemcpyHostToDevice, stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-        if (e != cudaSuccess) {
-            cudaFree(p.dev);
-            p.dev = nullptr;
-            return e;
-        }
-        A.rscan = static_cast<const unsigned char *>(p.dev);
-        A.rfin = reinterpret_cast<const TmaFinRec *>(static_cast<const unsigned char *>(p.dev) +
-                                                     (size_t)A.nbox * kScanBlock);
+        e = upload_table(&p.dev, p.host.data(), p.host.size(), stream);
+        if (e != cudaSuccess) return e;
+        p.a.rscan = static_cast<const unsigned char *>(p.dev);
+        p.a.rfin = reinterpret_cast<const TmaFinRec *>(static_cast<const unsigned char *>(p.dev) +
+                                                       (size_t)p.a.nbox * kScanBlock);
         cudaGetDevice(&p.device);
-        e = cudaGetSymbolAddress(reinterpret_cast<void **>(&A.err), g_tma_err);
-        if (e != cudaSuccess) return e;
     }
+    TmaArgs A = p.a;   // a copy: other threads may launch the same game's products
     A.batch = batch;
     A.nbb = (batch + 31) / 32;
     // test hook (KPS_TEST_STALL_WAIT=1): one barrier per CTA never completes,
