@@ -99,6 +99,34 @@ struct Epilogue {
         if (gate && !(gate[(long long)m * ldg + n] > 0.f)) v = 0.f;
         C[(long long)m * ldc + n] = v;
     }
+    // 16-byte loads and stores of its rows are aligned
+    bool vec_ok() const {
+        auto a = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+        return a(C) && ldc % 4 == 0 && a(bias) && a(gate) && (!gate || ldg % 4 == 0);
+    }
+    // Columns n .. n + 3, the last ones maybe past N
+    __device__ __forceinline__ void put4(int m, int n, int N, float4 v, bool vec) const {
+        if (vec && n + 4 <= N) {
+            if (bias) {
+                const float4 b = *reinterpret_cast<const float4 *>(bias + n);
+                v.x += b.x; v.y += b.y; v.z += b.z; v.w += b.w;
+            }
+            if (relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+            if (gate) {
+                const float4 g = *reinterpret_cast<const float4 *>(gate + (long long)m * ldg + n);
+                if (!(g.x > 0.f)) v.x = 0.f;
+                if (!(g.y > 0.f)) v.y = 0.f;
+                if (!(g.z > 0.f)) v.z = 0.f;
+                if (!(g.w > 0.f)) v.w = 0.f;
+            }
+            *reinterpret_cast<float4 *>(C + (long long)m * ldc + n) = v;
+        } else {
+            if (n < N) put(m, n, v.x);
+            if (n + 1 < N) put(m, n + 1, v.y);
+            if (n + 2 < N) put(m, n + 2, v.z);
+            if (n + 3 < N) put(m, n + 3, v.w);
+        }
+    }
 };
 
 // C(m,n) = sum_k A(m,k) B(k,n), then the epilogue.  A(m,k) = A[m*lda + k] (AK)
@@ -117,11 +145,17 @@ struct Epilogue {
 // to `part`, added in order by reduce_kernel).  Both orders are fixed: results
 // are bit-reproducible.  KG = 1 without a z split adds k in ascending order.
 // Losses and gradients of a 4096-row minibatch: 1.53 ms before (64 x 64
-// tiles of 4 x 4 outputs per thread, no k split), 0.38 ms now.
+// tiles of 4 x 4 outputs per thread, no k split), 0.31 ms now; of 0.38 -> 0.31
+// half by unrolling two k instead of eight (which spilled registers) and half
+// by the tile's way out through shared memory (one group stored it 4 bytes at a
+// time, each behind its gate's load).  The first layer's product takes 75 us: 57 %
+// of the FMA pipe on 256 of 304 resident CTAs, short of its global loads; the
+// shared loads take two thirds of the pipe's time, so A staged with every value
+// twice (no register pairs to build, half as many loads again) is 1.15x slower.
 template <int KG, bool AK, bool BK, typename TA, typename TB>
 __global__ void __launch_bounds__(64 * KG, KG == 1 ? 8 : 2)
 gemm_kernel(int M, int N, int K, int kpart, const TA *__restrict__ A, long long lda, int avec,
-            const TB *__restrict__ B, long long ldb, int bvec, float *__restrict__ part, const Epilogue ep) {
+            const TB *__restrict__ B, long long ldb, int bvec, float *__restrict__ part, const Epilogue ep, int evec) {
     constexpr int kBuf = kBK * kPitch;                       // one operand, one stage
     constexpr int kRed = KG == 1 ? 0 : KG / 2 * kBM * kBN;   // sums handed over between groups
     __shared__ __align__(16) float sh[KG * 4 * kBuf > kRed ? KG * 4 * kBuf : kRed];
@@ -155,7 +189,7 @@ gemm_kernel(int M, int N, int K, int kpart, const TA *__restrict__ A, long long 
             fetch<BK>(B, ldb, n0, N, kn, kend, bvec, t, vb);
         }
         const float *a = As + st * kBuf + 4 * tr, *b = Bs + st * kBuf + 4 * tc;
-#pragma unroll
+#pragma unroll 2
         for (int kk = 0; kk < kBK; ++kk) {
             const float4 a0 = *reinterpret_cast<const float4 *>(a + kk * kPitch);
             const float4 a1 = *reinterpret_cast<const float4 *>(a + kk * kPitch + 32);
@@ -192,23 +226,36 @@ gemm_kernel(int M, int N, int K, int kpart, const TA *__restrict__ A, long long 
             for (int e = 0; e < 32; ++e) acc[e >> 2][e & 3] = __fadd2_rn(acc[e >> 2][e & 3], r[64 * e]);
         }
     }
-    if (grp != 0) return;
+    // the tile goes through shared memory, so that every thread of the CTA
+    // stores (and reads bias and gate) 16 bytes at a time, rows contiguous
+    Epilogue out = ep;
+    if (part) out = Epilogue{part + (long long)blockIdx.z * M * N, N, nullptr, 0, nullptr, 0};
+    const bool vec = part ? N % 4 == 0 : evec != 0;
+    if (KG == 1) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int m = m0 + 4 * tr + (i & 3) + 32 * (i >> 2);
-        if (m >= M) continue;
+        for (int i = 0; i < 8; ++i) {
+            const int m = m0 + 4 * tr + (i & 3) + 32 * (i >> 2);
+            if (m >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + 4 * tc + 2 * (j & 1) + 32 * (j >> 1);
-            if (part) {
-                float *q = part + ((long long)blockIdx.z * M + m) * N;
-                if (n < N) q[n] = acc[i][j].x;
-                if (n + 1 < N) q[n + 1] = acc[i][j].y;
-            } else {
-                if (n < N) ep.put(m, n, acc[i][j].x);
-                if (n + 1 < N) ep.put(m, n + 1, acc[i][j].y);
-            }
+            for (int j = 0; j < 2; ++j)
+                out.put4(m, n0 + 4 * tc + 32 * j, N,
+                         make_float4(acc[i][2 * j].x, acc[i][2 * j].y, acc[i][2 * j + 1].x, acc[i][2 * j + 1].y), vec);
         }
+        return;
+    }
+    __syncthreads();
+    if (grp == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                *reinterpret_cast<float4 *>(sh + (4 * tr + (i & 3) + 32 * (i >> 2)) * kPitch + 4 * tc + 32 * j) =
+                    make_float4(acc[i][2 * j].x, acc[i][2 * j].y, acc[i][2 * j + 1].x, acc[i][2 * j + 1].y);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kBM * kBN / 4; e += 64 * KG) {
+        const int r = e >> 4, c = 4 * (e & 15);
+        if (m0 + r < M) out.put4(m0 + r, n0 + c, N, *reinterpret_cast<const float4 *>(sh + r * kPitch + c), vec);
     }
 }
 
@@ -325,7 +372,7 @@ cudaError_t gemm(int M, int N, int K, const TA *A, long long lda, const TB *B, l
     dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, nz);
     if (grid.y > 65535) return cudaErrorInvalidValue;
     gemm_kernel<KG, AK, BK, TA, TB><<<grid, 64 * KG, 0, st>>>(M, N, K, kpart, A, lda, vec_ok(A, lda), B, ldb,
-                                                              vec_ok(B, ldb), nz > 1 ? part : nullptr, ep);
+                                                              vec_ok(B, ldb), nz > 1 ? part : nullptr, ep, ep.vec_ok());
     if (nz > 1)
         reduce_kernel<<<(unsigned)(((long long)M * N + 255) / 256), 256, 0, st>>>(M, N, nz, part, ep);
     return cudaGetLastError();
