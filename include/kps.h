@@ -225,7 +225,10 @@ typedef struct kps_batch kps_batch;
 
 /* Multi-game kernels (kps_batch_shape.kernel):
  *   KPS_BATCH_TMEM    tensor-memory scan, 32-column tiles, 1-8 warps (every
- *                     storage type; FP64 runs its vector-register variant);
+ *                     storage type; FP64 runs its vector-register variant,
+ *                     and only where the FP64 kernel does not take the
+ *                     batch: two-card hands, few hands in ties across its
+ *                     boxes.  FP64 launch shapes mean that variant);
  *   KPS_BATCH_STAGED  FP32, BF16 or FP16 storage (FP32 arithmetic): 4 warps
  *                     per CTA scan chunks of a game's hand order in 16-hand
  *                     boxes staged by cp.async, with per-box hand records
@@ -438,7 +441,7 @@ kps_status kps_solver_strategy(kps_solver *solver, void *x, void *y, void *strea
  * best responses.  Asynchronous on `stream`. */
 kps_status kps_solver_exploitability(kps_solver *solver, double *expl, double *br1, double *br2, void *stream);
 /* The same quantity estimated cheaply for stopping tests: averages and
- * products in FP32 (tensor-memory kernels), best-response sums in FP64.
+ * products in FP32 (batched FP32 kernels), best-response sums in FP64.
  * Differs from kps_solver_exploitability by the FP32 rounding of the
  * products (about 1e-6 of the values); confirm a stop with the FP64 call. */
 kps_status kps_solver_exploitability_estimate(kps_solver *solver, double *expl, void *stream);

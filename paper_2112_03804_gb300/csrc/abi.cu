@@ -360,8 +360,8 @@ kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t
         const double *lout = dir == 0 ? h.lam1.data() : h.lam2.data();
         std::string why;
         kps::TmaParams *p = kps::tma_create(h, lin, lout, dir == 0 ? h.n[0] : h.n[1], dir == 0 ? h.n[1] : h.n[0],
-                                            g->dev.fcol[dir], g->dev.scol[dir], g->dev.fcoef_f[dir],
-                                            g->dev.scoef_f[dir], g->fcol[dir].data(), g->scol[dir].data(), &why);
+                                            g->fcol[dir].data(), g->scol[dir].data(), g->fcoef[dir].data(),
+                                            g->scoef[dir].data(), &why);
         g->tma[dir].reset(p);
         g->tma_state[dir] = p ? 1 : -1;
     }

@@ -184,12 +184,11 @@ struct TmaParams;
 struct HostGame;
 
 // Builds the parameter block for one direction (lam_in / lam_out: library
-// order; fcol, scol, fcoef, scoef: the device tables of that direction;
-// hfcol / hscol: their host copies).  Returns nullptr with *why set when
+// order; hfcol, hscol, fcoef, scoef: the host columns and payoffs of that
+// direction).  Returns nullptr with *why set when
 // the game cannot take this path.
 TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam_out, int n_out, int n_in,
-                      const int *fcol, const int *scol, const float *fcoef, const float *scoef,
-                      const int *hfcol, const int *hscol, std::string *why);
+                      const int *hfcol, const int *hscol, const double *fcoef, const double *scoef, std::string *why);
 void tma_destroy(TmaParams *p);
 // One product: out (device, [batch][n_out][hs]) from vin ([batch][n_in][hs]),
 // both 16-byte aligned.

@@ -92,6 +92,15 @@ namespace kps {
 constexpr int kTmaMaxExtra = 2;    // boxes of a chunk past the 256 tensor-memory columns
 constexpr int kMaxNw = 8;          // warps (chunks) of a CTA: 4, or 8 for few CTAs
 
+// An item, with all that a CTA needs to begin: one load instead of a chain of
+// two (128 FP32 vectors of the river game, 172 CTAs).
+struct alignas(32) TmaItem {
+    int sigma, sigma2;             // output sequence, and the fold-only sequence of its pair or -1
+    int rf, rs;                    // its fold / showdown input sequence or -1
+    float F, S, F2;                // their payoffs (0 without), the pair's fold payoff
+    int pad;
+};
+
 // Kernel arguments (__grid_constant__).
 struct alignas(128) TmaArgs {
     CUtensorMap tin;               // input  [batch][n_in][H], box 16 x 1 x 32, rows of a box swizzled (64 or 32 bytes)
@@ -100,9 +109,7 @@ struct alignas(128) TmaArgs {
     int stall_test;                // test hook: warp 0's first box expects 16 bytes that never come
     int bchunk[kMaxNw + 1];        // warp k scans boxes [bchunk[k], bchunk[k+1])
     int nitems;
-    const int2 *items;             // output sequence, and the fold-only sequence of its pair or -1
-    const int *fcol, *scol;        // per output sequence: its fold / showdown input sequence or -1
-    const float *fcoef, *scoef;    // and the payoffs
+    const TmaItem *items;
     const unsigned char *rscan;    // [nbox][kScanBlock]
     const TmaFinRec *rfin;         // [nbox * 8]
     unsigned int *err;             // set to 1 when a wait gives up
@@ -780,13 +787,13 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(cons
     c.lane = threadIdx.x & 31;
     c.warp = threadIdx.x >> 5;
     c.bb = blockIdx.x / P.nitems;
-    const int2 item = P.items[blockIdx.x - c.bb * P.nitems];
-    c.sigma = item.x;
-    c.sigma2 = item.y;
-    c.rf = P.fcol[c.sigma];
-    c.rs = P.scol[c.sigma];
-    c.F = c.rf >= 0 ? P.fcoef[c.sigma] : 0.f;
-    c.S = c.rs >= 0 ? P.scoef[c.sigma] : 0.f;
+    const TmaItem item = P.items[blockIdx.x - c.bb * P.nitems];
+    c.sigma = item.sigma;
+    c.sigma2 = item.sigma2;
+    c.rf = item.rf;
+    c.rs = item.rs;
+    c.F = item.F;
+    c.S = item.S;
     c.b0 = P.bchunk[c.warp];
     c.nb = P.bchunk[c.warp + 1] - c.b0;
     c.ok = true;
@@ -803,7 +810,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(cons
     else if (kind == kKindF) Cw = tma_scan<T, kKindF, K2, NW>(P, c);
     else Cw = tma_scan<T, kKindS, K2, NW>(P, c);
     if (NW == 4 && c.sigma2 >= 0) {   // eight warps: items are not paired
-        c.F = P.fcoef[c.sigma2];
+        c.F = item.F2;
         tma_finish<T, K2, NW, true>(P, c, Cw, c.S);
     } else {
         tma_finish<T, K2, NW, false>(P, c, Cw, kind == kKindS ? c.S : 1.f);
@@ -904,8 +911,13 @@ static std::string tma_prepare(const HostGame &h, const double *lam_in, const do
 // Items after the records: first the pairs (a fold-only sequence goes with the
 // first showdown-only one of its input row) and what is left alone, then every
 // sequence alone.
-std::string tma_items(int n_out, const int *hfcol, const int *hscol, TmaParams &p) {
-    std::vector<int2> items;
+std::string tma_items(int n_out, const int *hfcol, const int *hscol, const double *fcoef, const double *scoef,
+                      TmaParams &p) {
+    std::vector<TmaItem> items;
+    auto add = [&](int r, int q) {
+        items.push_back(TmaItem{r, q, hfcol[r], hscol[r], hfcol[r] >= 0 ? (float)fcoef[r] : 0.f,
+                                hscol[r] >= 0 ? (float)scoef[r] : 0.f, q >= 0 ? (float)fcoef[q] : 0.f, 0});
+    };
     std::vector<int> fold_of;   // by input row: its first fold-only sequence, -1 once taken
     std::vector<int> mate(n_out, -1);
     std::vector<char> taken(n_out, 0);
@@ -922,13 +934,13 @@ std::string tma_items(int n_out, const int *hfcol, const int *hscol, TmaParams &
         if (mate[r] >= 0) taken[mate[r]] = 1;
     }
     for (int r = 0; r < n_out; ++r)
-        if (!taken[r]) items.push_back(make_int2(r, mate[r]));
+        if (!taken[r]) add(r, mate[r]);
     p.npaired = (int)items.size();
     p.nsingle = n_out;
-    for (int r = 0; r < n_out; ++r) items.push_back(make_int2(r, -1));
-    p.o_items = (p.host.size() + 15) / 16 * 16;
-    p.host.resize(p.o_items + sizeof(int2) * items.size());
-    if (!items.empty()) std::memcpy(p.host.data() + p.o_items, items.data(), sizeof(int2) * items.size());
+    for (int r = 0; r < n_out; ++r) add(r, -1);
+    p.o_items = (p.host.size() + 31) / 32 * 32;
+    p.host.resize(p.o_items + sizeof(TmaItem) * items.size());
+    if (!items.empty()) std::memcpy(p.host.data() + p.o_items, items.data(), sizeof(TmaItem) * items.size());
     return "";
 }
 
@@ -937,8 +949,7 @@ std::string tma_items(int n_out, const int *hfcol, const int *hscol, TmaParams &
 namespace kps {
 
 TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam_out, int n_out, int n_in,
-                      const int *fcol, const int *scol, const float *fcoef, const float *scoef,
-                      const int *hfcol, const int *hscol, std::string *why) {
+                      const int *hfcol, const int *hscol, const double *fcoef, const double *scoef, std::string *why) {
     TmaParams *p = new (std::nothrow) TmaParams();
     if (!p) {
         *why = "host allocation";
@@ -947,7 +958,7 @@ TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam
     std::string w;
     try {
         w = tma_prepare(h, lam_in, lam_out, *p);
-        if (w.empty()) w = tma_items(n_out, hfcol, hscol, *p);
+        if (w.empty()) w = tma_items(n_out, hfcol, hscol, fcoef, scoef, *p);
     } catch (const std::bad_alloc &) {
         w = "host allocation";
     }
@@ -960,10 +971,6 @@ TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam
     }
     p->a.n_out = n_out;
     p->a.n_in = n_in;
-    p->a.fcol = fcol;
-    p->a.scol = scol;
-    p->a.fcoef = fcoef;
-    p->a.scoef = scoef;
     p->a.err = nullptr;
     return p;
 }
@@ -1020,7 +1027,7 @@ cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *v
     const int nw = p.eight && single <= sms ? 8 : 4;
     const bool pair = nw == 4 && (paired + slots - 1) / slots < (single + slots - 1) / slots;
     const unsigned char *items = static_cast<const unsigned char *>(p.dev) + p.o_items;
-    A.items = reinterpret_cast<const int2 *>(items) + (pair ? 0 : p.npaired);
+    A.items = reinterpret_cast<const TmaItem *>(items) + (pair ? 0 : p.npaired);
     A.nitems = pair ? p.npaired : p.nsingle;
     A.extra = nw == 4 ? p.extra4 : 0;
     for (int k = 0; k <= nw; ++k) A.bchunk[k] = nw == 4 ? p.chunk4[k] : p.chunk8[k];
