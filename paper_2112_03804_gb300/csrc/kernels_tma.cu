@@ -634,7 +634,7 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
 // table, whose rest is one more staging slot.  (Copied by the lanes, with
 // cp.async, a 1024-vector FP32 launch takes 6 % longer.)  A warp whose scan gave
 // up finishes nothing: a copy into its ring may still be in flight.
-template <typename T, int K2, int NW, bool PAIR>
+template <typename T, int K2, int NW, bool PAIR, bool SCALED>
 __device__ __forceinline__ void tma_finish(const TmaArgs &P, Ctx &c, float Cw, float scale) {
     if (!c.ok) return;
     constexpr int BB = Box<T>::kBytes;
@@ -691,12 +691,18 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, Ctx &c, float Cw, f
             for (int i = 0; i < 16; ++i) r[i] = xp[i * 32 + lane];
         }
     };
-    int nst = 0;   // boxes staged
+    int nst = 0, next = 0;   // boxes staged, the next one's slot
     auto put = [&](int m, int sigma, const float2 *o) {
-        const int sl = nst % nbuf;
+        const int sl = next;
+        next = sl + 1 == nbuf ? 0 : sl + 1;
         unsigned char *buf = PAIR && sl == nring ? xst : ring + qbytes + sl * BB;
+        // (a group per box: before a slot's second use all but the newest
+        // nbuf - 1 have been read)
         if (nst >= nbuf) {
-            if (lane == 0) bulk_wait_read_n(nbuf - 1);
+            if (lane == 0) {
+                if (nbuf == 3) bulk_wait_read<2>();
+                else bulk_wait_read_n(nbuf - 1);
+            }
             __syncwarp();
         }
         ++nst;
@@ -740,7 +746,7 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, Ctx &c, float Cw, f
                 nq = add2(nq, make_float2(*reinterpret_cast<const float *>(qb + r.ob1),
                                           *reinterpret_cast<const float *>(qb + r.ob2)));
             const float2 lo = make_float2(r.lout1, r.lout2);
-            o[i / 2] = mul2(mul2(S2, lo), add2(add2(make_float2(pc[i], pc[i + 1]), make_float2(Cw, Cw)), nq));
+            o[i / 2] = mul2(SCALED ? mul2(S2, lo) : lo, add2(add2(make_float2(pc[i], pc[i + 1]), make_float2(Cw, Cw)), nq));
             if (PAIR) {
                 float2 np = make_float2(*reinterpret_cast<const float *>(fb + r.oa1),
                                         *reinterpret_cast<const float *>(fb + r.oa2));
@@ -811,9 +817,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(cons
     else Cw = tma_scan<T, kKindS, K2, NW>(P, c);
     if (NW == 4 && c.sigma2 >= 0) {   // eight warps: items are not paired
         c.F = item.F2;
-        tma_finish<T, K2, NW, true>(P, c, Cw, c.S);
+        tma_finish<T, K2, NW, true, true>(P, c, Cw, c.S);
+    } else if (kind == kKindS) {
+        tma_finish<T, K2, NW, false, true>(P, c, Cw, c.S);
     } else {
-        tma_finish<T, K2, NW, false>(P, c, Cw, kind == kKindS ? c.S : 1.f);
+        tma_finish<T, K2, NW, false, false>(P, c, Cw, 1.f);
     }
     if (!c.ok && c.lane == 0) atomicExch(P.err, 1u);
     tm_fence_before();
