@@ -57,10 +57,11 @@
 // row's boxes once more (L2) for the b[h] of K_F.  A third of a game's items
 // go (43 sequences of the 1081-hand river game: 29 items), with their scans
 // and table traffic: 1024 FP32 vectors 134 -> 124 us, 250 vectors of the
-// 247-sequence tree 185 -> 168 us (single against paired items, same build).
+// 247-sequence tree 185 -> 168 us (single against paired items, same build;
+// 121 and 163 us since the finishing pass counts its staging slots).
 //
 // 16-bit storage (1000 BF16 vectors of the river game: 284 us on the
-// tensor-memory kernel, 119 us here) differs in the boxes alone.  Both storage
+// tensor-memory kernel, 118 us here) differs in the boxes alone.  Both storage
 // types are bound by the scan's and the finishing pass's short dependent
 // steps at eight resident warps per SM, not by memory (floor 55 / 27 us).
 //
