@@ -101,21 +101,44 @@ __device__ __forceinline__ Where locate(const SolverGame *games, const int *bloc
 // Regret matching of one node: b[a] = R+[a] / sum, uniform if the sum is
 // at most the noise floor theta.  The quotients share the rounded reciprocal of
 // the sum; one correction by the remainder rounds each as the division does
-// (Markstein 1990; away from the ends of the exponent range, where the division
-// itself is taken), in three instructions an action.
+// (Markstein 1990), in three instructions an action, as long as the remainder is
+// exact and the quotient normal.  Both hold when every positive R is at least
+// kLeast and the sum is below kMost (the remainder's last bit is then above the
+// smallest subnormal, the quotient above kLeast / kMost); a node with a smaller
+// regret or a larger sum takes the division (without the lower bound, one FP32
+// quotient in four of regrets below 2^-126 rounded the other way).
+template <typename C> struct QuotientRange;
+template <> struct QuotientRange<float> {
+    static constexpr float kMost = 0x1p44f;
+    static constexpr uint32_t kLeast = (127u - 80u) << 23;                       // 2^-80
+    __device__ static uint32_t lead(float p) { return __float_as_uint(p); }
+};
+template <> struct QuotientRange<double> {
+    static constexpr double kMost = 0x1p100;
+    static constexpr uint32_t kLeast = (1023u - 900u) << 20;                     // 2^-900
+    __device__ static uint32_t lead(double p) {
+        return (uint32_t)__double2hiint(p) | (__double2loint(p) != 0 ? 1u : 0u);
+    }
+};
 template <int M, typename C>
 __device__ __forceinline__ void regret_match(const C *r, int na, C *b, C theta) {
+    using Range = QuotientRange<C>;
     // positive parts (RM+ regrets are never negative; DCFR's may be)
     C sum = C(0);
+    uint32_t least = ~0u;   // leading word of the smallest positive part, less one (0 wraps to the top)
 #pragma unroll
     for (int a = 0; a < M; ++a)
-        if (a < na) sum += r[a] > C(0) ? r[a] : C(0);
+        if (a < na) {
+            const C p = r[a] > C(0) ? r[a] : C(0);
+            sum += p;
+            least = min(least, Range::lead(p) - 1u);
+        }
     const C one = C(1) / (sum > theta ? sum : C(na));   // 1 / na when uniform
     if (!(sum > theta)) {
 #pragma unroll
         for (int a = 0; a < M; ++a)
             if (a < na) b[a] = one;
-    } else if (sum > C(1e-30) && sum < C(1e30)) {
+    } else if (least >= Range::kLeast && sum < Range::kMost) {
 #pragma unroll
         for (int a = 0; a < M; ++a)
             if (a < na) {
