@@ -98,7 +98,7 @@ __host__ __device__ inline size_t am_hdr_off(int nc) { return am_state_off(kTmaW
 inline size_t am_smem_bytes(int nc) { return am_hdr_off(nc) + 16 + 2 * kTmaWarps * 32 * 4; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// 16 bytes from global memory; the bytes past `src_bytes` (0 or 16) are zero
+// 16 bytes from global memory; the bytes past `src_bytes` (0 to 16) are zero
 __device__ __forceinline__ void cp16(uint32_t dst, const void *src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
@@ -195,6 +195,13 @@ template <> struct Store<__half> {
     }
 };
 
+// Bytes of a 16-byte chunk that hold hands when `left` hands of the row remain
+// from its first (none when it is all padding).
+template <typename T>
+__device__ __forceinline__ uint32_t hand_bytes(int left) {
+    return (uint32_t)(max(0, min(left, Store<T>::kPer)) * (int)sizeof(T));
+}
+
 // One work item, one warp: scan of the warp's chunk, combination of the
 // four chunks (two CTA barriers), finishing pass.  A split item has at most
 // 16 output sequences: lanes 16-31 take the same sequences as lanes 0-15 over
@@ -229,7 +236,6 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
     const T *vin = static_cast<const T *>(P.vin) + G.in_off;
     const T *pa = vin + (size_t)(rf >= 0 ? rf : 0) * hs;
     const T *pb = vin + (size_t)(rs >= 0 ? rs : 0) * hs;
-    const uint32_t na = rf >= 0 ? 16u : 0u, nbytes_b = rs >= 0 ? 16u : 0u;
     unsigned char *ring = sm + am_ring_off(warp);
     const uint32_t ring_s = smem_u32(ring);
     unsigned char *rring = sm + am_rec_off(warp);
@@ -252,8 +258,9 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
             for (int q = 0; q < NQ; ++q) {
                 const int h0 = x + Store<T>::kPer * q;
                 const bool in = real && h0 < hs;   // hs is a multiple of 8: a chunk is all in or all out
-                cp16(dst + 512u * q, in ? pa + h0 : pa, in ? na : 0u);
-                cp16(dst + 2048u + 512u * q, in ? pb + h0 : pb, in ? nbytes_b : 0u);
+                const uint32_t nb_in = hand_bytes<T>(G.H - h0);   // padding hands hold anything: zeros
+                cp16(dst + 512u * q, in ? pa + h0 : pa, in && rf >= 0 ? nb_in : 0u);
+                cp16(dst + 2048u + 512u * q, in ? pb + h0 : pb, in && rs >= 0 ? nb_in : 0u);
             }
             // the record block of each half's box (zeros for a zero-filled box)
             if (lane < kScanBlock / 16) {
@@ -507,7 +514,8 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
                 if (x + Store<T>::kPer * q < hs)
-                    cp16(ring_s + yb + (uint32_t)((m & 1) * 2048) + 512u * q, pb + x + Store<T>::kPer * q, 16u);
+                    cp16(ring_s + yb + (uint32_t)((m & 1) * 2048) + 512u * q, pb + x + Store<T>::kPer * q,
+                         hand_bytes<T>(G.H - x - Store<T>::kPer * q));
         }
         cp_commit();
     };
