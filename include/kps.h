@@ -225,24 +225,27 @@ typedef struct kps_batch kps_batch;
 
 /* Multi-game kernels (kps_batch_shape.kernel):
  *   KPS_BATCH_TMEM    tensor-memory scan, 32-column tiles, 1-8 warps (every
- *                     storage type; FP64 runs its vector-register variant,
- *                     and only where the FP64 kernel does not take the
- *                     batch: two-card hands, few hands in ties across its
- *                     boxes.  FP64 launch shapes mean that variant);
+ *                     storage type; FP64 runs its vector-register variant);
  *   KPS_BATCH_STAGED  FP32, BF16 or FP16 storage (FP32 arithmetic): 4 warps
  *                     per CTA scan chunks of a game's hand order in 16-hand
  *                     boxes staged by cp.async, with per-box hand records
  *                     (games whose chunks fit 24 boxes and that have few
  *                     hands in tie groups of more than 4; the others run
- *                     on the tensor-memory kernel in a second launch). */
+ *                     on the tensor-memory kernel in a second launch);
+ *   KPS_BATCH_F64     FP64, two-card hands, few hands in ties across its
+ *                     boxes: six warps per CTA, one CTA per item of 8 to 32
+ *                     columns.  FP64 products run it on the batches it takes
+ *                     unless kps_batch_shape_set chose KPS_BATCH_TMEM or
+ *                     kps_batch_tune found that faster. */
 #define KPS_BATCH_TMEM 0
 #define KPS_BATCH_STAGED 1
+#define KPS_BATCH_F64 2
 
 typedef struct {
     int32_t warps;        /* warps per CTA                                  */
     int32_t grid;         /* CTAs of the persistent launch                  */
     int32_t schedule;     /* 0 atomic ticket counter, 1 static stride       */
-    int32_t kernel;       /* KPS_BATCH_TMEM or KPS_BATCH_STAGED             */
+    int32_t kernel;       /* KPS_BATCH_*                                    */
     double ms_per_pair;   /* tuned time of one A and one A^T launch, or 0   */
 } kps_batch_shape;
 
@@ -266,7 +269,9 @@ kps_status kps_batch_shape_get(kps_batch *batch, kps_dtype dt, kps_batch_shape *
 /* Sets the launch shape for `dt` (ms_per_pair ignored).  Errors: KPS_EINVAL
  * (out of range), KPS_ENOTSUP (warp count the games do not fit; the staged
  * kernel for FP64, with other than 4 warps, more than 2
- * CTAs per SM, or for games it does not take). */
+ * CTAs per SM, or for games it does not take; the FP64 kernel for another
+ * dtype, for games it does not take, or with other numbers than
+ * kps_batch_shape_get reports for it). */
 kps_status kps_batch_shape_set(kps_batch *batch, kps_dtype dt, const kps_batch_shape *shape);
 
 /* Splits items 0..n-1 (games, in order) into `parts` contiguous ranges

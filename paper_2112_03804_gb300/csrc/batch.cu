@@ -13,7 +13,6 @@
 
 #include <algorithm>
 #include <new>
-#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <string>
@@ -214,14 +213,9 @@ kps_status build_table(kps_batch *b, int dir, bool f64, int nw, const std::vecto
     std::memcpy(host.data() + o_in, in_off.data(), 8 * (size_t)ng);
     std::memcpy(host.data() + o_out, out_off.data(), 8 * (size_t)ng);
     BatchTable tb;
-    cudaError_t e = cudaMalloc(&tb.blob, total);
-    if (e != cudaSuccess) return fail(KPS_ENOMEM, "batch launch table");
-    e = cudaMemcpyAsync(tb.blob, host.data(), total, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) {
-        cudaFree(tb.blob);
-        return cuda_fail(e, "uploading the batch launch table");
-    }
+    const cudaError_t e = kps::upload_table(&tb.blob, host.data(), total, stream);
+    if (e == cudaErrorMemoryAllocation) return fail(KPS_ENOMEM, "batch launch table");
+    if (e != cudaSuccess) return cuda_fail(e, "uploading the batch launch table");
     unsigned char *bl = static_cast<unsigned char *>(tb.blob);
     tb.m.games = reinterpret_cast<const kps::FastParams *>(bl + o_fp);
     tb.m.tile_start = reinterpret_cast<const long long *>(bl + o_ts);
@@ -268,6 +262,18 @@ kps_status batch_rest_table(kps_batch *b, int dir, cudaStream_t stream, const Ba
     return KPS_OK;
 }
 
+namespace {
+// The FP64 kernel's launch (plans built): one CTA per item, the longer direction's count.
+BatchShape f64_shape(const kps_batch *b) {
+    BatchShape s;
+    s.kernel = KPS_BATCH_F64;
+    s.nw = kps::kF64Warps;
+    s.grid = std::max(kps::f64_items(b->f64[0]), kps::f64_items(b->f64[1]));
+    s.schedule = 1;
+    return s;
+}
+}  // namespace
+
 // The launch shape used for `dt` when the batch has not been tuned.
 kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, BatchShape *out) {
     auto it = b->shape.find((int)dt);
@@ -282,13 +288,20 @@ kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, 
         maxH = std::max(maxH, g->host.H);
         maxnc = std::max(maxnc, g->host.ncards + 1);
     }
-    if (dt == KPS_F64) {
+    bool decided = true;   // false: the plan may still be built by a later call
+    if (dt == KPS_F64 && batch_f64_ready(b, stream)) {
+        s = f64_shape(b);
+        b->shape[(int)dt] = s;
+        *out = s;
+        return KPS_OK;
+    } else if (dt == KPS_F64) {
+        decided = b->f64_state != 0;
         if (maxnc > 64) return fail(KPS_ENOTSUP, "card count too large for the FP64 batch kernel");
         s.nw = 8;
         while (s.nw > 1 && kps::vec_smem_bytes(storage, maxnc, s.nw) > (size_t)kps::max_dyn_smem()) --s.nw;
         s.nw = std::max(1, std::min(s.nw, (maxH + kps::kTile - 1) / kps::kTile));
         s.per_sm = std::max(1, kps::vec_multi_ctas_per_sm(storage, b->k, maxnc, s.nw));
-    } else if (dt != KPS_F64 && batch_staged_ready(b, stream)) {
+    } else if (batch_staged_ready(b, stream)) {
         s.kernel = KPS_BATCH_STAGED;
         s.nw = 4;
         s.per_sm = std::min(kps::am_ctas_per_sm(b->am[0]), kps::am_ctas_per_sm(b->am[1]));
@@ -308,15 +321,13 @@ kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, 
     }
     s.grid = sm_count() * s.per_sm;
     s.schedule = 0;
-    b->shape[(int)dt] = s;
+    if (decided) b->shape[(int)dt] = s;
     *out = s;
     return KPS_OK;
 }
 
 bool batch_f64_ready(kps_batch *b, cudaStream_t stream) {
     if (b->f64_state != 0) return b->f64_state == 1;
-    if (const char *force = std::getenv("KPS_KERNEL"))
-        if (std::strcmp(force, "f64") != 0) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
     if (e != cudaSuccess) cudaGetLastError();
@@ -359,15 +370,15 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
     if (ci < co + out_bytes && co < ci + in_bytes) return fail(KPS_EINVAL, "input and output overlap");
     if (((reinterpret_cast<uintptr_t>(vin) | reinterpret_cast<uintptr_t>(vout)) & 15) != 0)
         return fail(KPS_EINVAL, "batch vectors must be 16-byte aligned");
-    if (dt == KPS_F64 && batch_f64_ready(b, stream)) {
+    BatchShape s;
+    kps_status st = batch_default_shape(b, dt, stream, &s);
+    if (st != KPS_OK) return st;
+    if (s.kernel == KPS_BATCH_F64) {
         const cudaError_t e =
             kps::launch_f64_scan(b->f64[dir], static_cast<const double *>(vin), static_cast<double *>(vout), 1, stream);
         if (e != cudaSuccess) return cuda_fail(e, "launching the FP64 batched payoff scan");
         return KPS_OK;
     }
-    BatchShape s;
-    kps_status st = batch_default_shape(b, dt, stream, &s);
-    if (st != KPS_OK) return st;
     if (s.kernel == KPS_BATCH_STAGED) {
         cudaError_t e = cudaSuccess;
         kps::AmPlan *am = plain && b->am_plain[0] && b->am_plain[1] ? b->am_plain[dir] : b->am[dir];
@@ -516,6 +527,7 @@ kps_status kps_batch_tune(kps_batch *b, kps_dtype dt, void *stream_ptr, kps_batc
                 cands.push_back(s);
             }
     }
+    if (dt == KPS_F64 && batch_f64_ready(b, stream)) cands.push_back(f64_shape(b));
     if (cands.empty()) return fail(KPS_ENOTSUP, "no launch shape fits this batch");
     const size_t es = dtype_size(dt);
     void *vin = nullptr, *vout = nullptr;
@@ -610,8 +622,17 @@ kps_status kps_batch_shape_set(kps_batch *b, kps_dtype dt, const kps_batch_shape
     if (st != KPS_OK) return st;
     if (shape->schedule != 0 && shape->schedule != 1) return fail(KPS_EINVAL, "schedule must be 0 or 1");
     if (shape->grid < 1) return fail(KPS_EINVAL, "grid must be >= 1");
-    if (shape->kernel != KPS_BATCH_TMEM && shape->kernel != KPS_BATCH_STAGED)
-        return fail(KPS_EINVAL, "kernel must be KPS_BATCH_TMEM or KPS_BATCH_STAGED");
+    if (shape->kernel != KPS_BATCH_TMEM && shape->kernel != KPS_BATCH_STAGED && shape->kernel != KPS_BATCH_F64)
+        return fail(KPS_EINVAL, "kernel must be KPS_BATCH_TMEM, KPS_BATCH_STAGED or KPS_BATCH_F64");
+    if (shape->kernel == KPS_BATCH_F64) {
+        if (dt != KPS_F64) return fail(KPS_ENOTSUP, "the FP64 kernel takes FP64 vectors");
+        if (!batch_f64_ready(b, nullptr)) return fail(KPS_ENOTSUP, "a game of the batch does not fit the FP64 kernel");
+        const BatchShape s = f64_shape(b);
+        if (shape->warps != s.nw || shape->grid != s.grid || shape->schedule != s.schedule)
+            return fail(KPS_ENOTSUP, "the FP64 kernel runs 6 warps per CTA and one CTA per item");
+        b->shape[(int)dt] = s;
+        return KPS_OK;
+    }
     if (shape->kernel == KPS_BATCH_STAGED) {
         if (dt == KPS_F64) return fail(KPS_ENOTSUP, "the staged kernel takes FP32, BF16 or FP16 vectors");
         if (shape->warps != 4) return fail(KPS_ENOTSUP, "the staged kernel runs 4 warps per CTA");

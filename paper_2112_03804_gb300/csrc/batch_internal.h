@@ -18,7 +18,7 @@ struct BatchShape {
     int per_sm = 1;     // CTAs per SM
     int grid = 0;       // CTAs of the persistent launch
     int schedule = 0;   // 0 ticket counter, 1 static stride
-    int kernel = 0;     // KPS_BATCH_TMEM or KPS_BATCH_STAGED
+    int kernel = 0;     // KPS_BATCH_*
     double ms = 0.0;    // tuned time of one A and one A^T launch (0 = untuned)
 };
 

@@ -200,7 +200,7 @@ cudaError_t tma_take_error(bool *set);
 // FP64 path (kernels_f64.cu) for two-card games with few ties: one game and
 // many vectors, or (multi) many games with one vector each.  Builds and uploads
 // the plan (synchronises `stream`); nullptr with *why set when a game does not
-// fit.  batch: vectors of a single game, 1 for many games.
+// fit.
 struct F64GameDesc {
     const HostGame *h;
     const double *lam_in, *lam_out;   // host, library order
@@ -213,6 +213,9 @@ struct F64GameDesc {
 struct F64Plan;
 F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why);
 void f64_destroy(F64Plan *p);
+constexpr int kF64Warps = 6;          // warps of a CTA
+int f64_items(const F64Plan *p);      // CTAs of a launch over many games
+// batch: vectors of a single game, 1 for many games.
 cudaError_t launch_f64_scan(F64Plan *p, const double *vin, double *vout, int batch, cudaStream_t stream);
 
 // Staged multi-game path (FP32, BF16 or FP16 storage, kStore*; FP32

@@ -48,7 +48,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kBox = 8;                    // hands per box
-constexpr int kNW = 6;                     // warps per CTA
+constexpr int kNW = kF64Warps;             // warps per CTA
 constexpr int kNS = 2;                     // ring slots
 constexpr int kParts = 4;                  // most parts of a chunk
 constexpr int kRow = 2048;                 // bytes of one row's box (32 lanes x 64)
@@ -533,6 +533,8 @@ void f64_destroy(F64Plan *p) {
     if (p->blob) cudaFree(p->blob);
     delete p;
 }
+
+int f64_items(const F64Plan *p) { return p->nitems; }
 
 cudaError_t launch_f64_scan(F64Plan *p, const double *vin, double *vout, int batch, cudaStream_t stream) {
     Args a = p->a;

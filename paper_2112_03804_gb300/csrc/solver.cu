@@ -845,7 +845,6 @@ kps_status kps_solver_create(kps_batch *b, kps_dtype dt, kps_solver **out) {
     // launch tables of the products the solver uses, built before any capture
     for (kps_dtype d : {dt, KPS_F64}) {
         BatchShape sh;
-        if (d == KPS_F64 && batch_f64_ready(b, nullptr)) continue;
         kps_status st = batch_default_shape(b, d, nullptr, &sh);
         for (int dir = 0; dir < 2 && st == KPS_OK && sh.kernel == KPS_BATCH_TMEM; ++dir) {
             const BatchTable *t = nullptr;

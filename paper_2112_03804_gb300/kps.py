@@ -412,7 +412,7 @@ class TechniqueB:
 
 
 STATIC_SCRATCH_FLOATS = 4194304
-BATCH_TMEM, BATCH_STAGED = 0, 1
+BATCH_TMEM, BATCH_STAGED, BATCH_F64 = 0, 1, 2
 KERNEL_NAMES = {1: "tma", 2: "tmem", 3: "vec", 4: "fast", 5: "general", 6: "f64"}
 
 
@@ -471,7 +471,8 @@ class Batch:
         return sh.as_dict()
 
     def set_shape(self, dtype: int, warps: int, grid: int, schedule: int, kernel: int = 0):
-        """kernel: BATCH_TMEM (0) or BATCH_STAGED (1, FP32, 4 warps)."""
+        """kernel: BATCH_TMEM (0), BATCH_STAGED (1; FP32, BF16, FP16; 4 warps)
+        or BATCH_F64 (2; FP64; warps, grid and schedule as shape() reports)."""
         sh = BatchShape(warps, grid, schedule, kernel, 0.0)
         _check(lib().kps_batch_shape_set(self._h, dtype, C.byref(sh)))
 
