@@ -120,7 +120,7 @@ kps_status upload(kps_game *g, cudaStream_t stream) {
         put(o_sd[d], g->scoef[d].data(), 8 * r);
     }
     void *blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, off);
+    cudaError_t e = kps::device_malloc(&blob, off);
     if (e != cudaSuccess) return fail(KPS_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     e = cudaMemcpyAsync(blob, hostblob.data(), off, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -304,7 +304,7 @@ kps_status matvec_fast(kps_game *g, int dir, const kps::ScanParams &sp, int stor
             if (g->scratch) cudaFree(g->scratch);
             g->scratch = nullptr;
             g->scratch_bytes = 0;
-            cudaError_t e = cudaMalloc(&g->scratch, need);
+            cudaError_t e = kps::device_malloc(&g->scratch, need);
             if (e != cudaSuccess) return fail(KPS_ENOMEM, "partial-result buffer");
             g->scratch_bytes = need;
         }
@@ -363,12 +363,15 @@ kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t
                                             g->fcol[dir].data(), g->scol[dir].data(), g->fcoef[dir].data(),
                                             g->scoef[dir].data(), &why);
         g->tma[dir].reset(p);
-        g->tma_state[dir] = p ? 1 : -1;
+        g->tma_state[dir] = p ? 1 : why == "host allocation" ? 0 : -1;   // no memory: a later call tries again
     }
     if (g->tma_state[dir] != 1) return KPS_OK;
+    cudaError_t e = kps::tma_upload(g->tma[dir].get(), stream);
+    if (e == cudaErrorMemoryAllocation) return KPS_OK;   // the tensor-memory kernel needs less
     *taken = true;
+    if (e != cudaSuccess) return cuda_fail(e, "uploading the tables of the TMA-staged payoff scan");
     g->last_kernel[dir] = KPS_KERNEL_TMA;
-    cudaError_t e = kps::launch_tma_scan(g->tma[dir].get(), storage, vin, vout, batch, stream);
+    e = kps::launch_tma_scan(g->tma[dir].get(), storage, vin, vout, batch, stream);
     if (e != cudaSuccess) return cuda_fail(e, "launching the TMA-staged payoff scan");
     return KPS_OK;
 }
@@ -401,18 +404,17 @@ kps_status matvec_f64(kps_game *g, int dir, const void *vin, void *vout, int32_t
     if (g->f64_state[dir] == 0) {
         // the plan is uploaded with a synchronisation, which a capturing stream
         // cannot do: the other FP64 kernel's tables may be there already
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        cudaError_t e = cudaStreamIsCapturing(stream, &cap);
-        if (e != cudaSuccess) cudaGetLastError();
-        if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return KPS_OK;
+        if (kps::capturing(stream) || !kps::memory_for(g->f64_need[dir])) return KPS_OK;
         std::string why;
+        size_t need = 1;
         kps::F64Plan *p = nullptr;
         try {
-            p = kps::f64_create({f64_desc(g, dir)}, false, stream, &why);
+            p = kps::f64_create({f64_desc(g, dir)}, false, stream, &why, &need);
         } catch (const std::bad_alloc &) {
         }
         g->f64[dir].reset(p);
-        g->f64_state[dir] = p ? 1 : -1;
+        g->f64_state[dir] = p ? 1 : need > 0 ? 0 : -1;   // no memory: a later call tries again
+        g->f64_need[dir] = need;
     }
     if (g->f64_state[dir] != 1) return KPS_OK;
     *taken = true;
@@ -519,7 +521,7 @@ kps_status matvec_host(kps_game *g, int dir, const void *vin, void *vout, int32_
         if (g->stage_in) cudaFree(g->stage_in);
         g->stage_in = nullptr;
         g->stage_in_bytes = 0;
-        e = cudaMalloc(&g->stage_in, in_bytes);
+        e = kps::device_malloc(&g->stage_in, in_bytes);
         if (e != cudaSuccess) return fail(KPS_ENOMEM, "staging buffer");
         g->stage_in_bytes = in_bytes;
     }
@@ -527,7 +529,7 @@ kps_status matvec_host(kps_game *g, int dir, const void *vin, void *vout, int32_
         if (g->stage_out) cudaFree(g->stage_out);
         g->stage_out = nullptr;
         g->stage_out_bytes = 0;
-        e = cudaMalloc(&g->stage_out, out_bytes);
+        e = kps::device_malloc(&g->stage_out, out_bytes);
         if (e != cudaSuccess) return fail(KPS_ENOMEM, "staging buffer");
         g->stage_out_bytes = out_bytes;
     }

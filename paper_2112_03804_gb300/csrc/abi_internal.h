@@ -81,6 +81,7 @@ struct kps_game {
     };
     std::unique_ptr<kps::F64Plan, F64Del> f64[2];
     int f64_state[2] = {0, 0};
+    size_t f64_need[2] = {0, 0};      // bytes a plan could not get (state 0)
     // kernel of the last product per direction (KPS_KERNEL_* of kps.h)
     int last_kernel[2] = {0, 0};
 };

@@ -85,13 +85,17 @@ std::vector<kps::AmGameDesc> am_descs(const kps_batch *b, int dir) {
 
 bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
     if (b->am_state != 0) return b->am_state == 1;
+    if (kps::capturing(stream) || !kps::memory_for(b->am_need)) return false;
     b->am_state = -1;
     const int ng = (int)b->games.size();
     for (int dir = 0; dir < 2; ++dir) {
         const std::vector<kps::AmGameDesc> d = am_descs(b, dir);
         std::string why;
         std::vector<char> taken;
-        b->am[dir] = kps::am_create(d, 2 * sm_count(), false, stream, &taken, &why);
+        size_t need = 0;
+        b->am[dir] = kps::am_create(d, 2 * sm_count(), false, stream, &taken, &why, &need);
+        if (need > 0) b->am_state = 0;   // no memory: a later call tries again
+        b->am_need = need;
         bool ok = b->am[dir] != nullptr && kps::am_ctas_per_sm(b->am[dir]) >= 1;
         if (ok && dir == 1) ok = b->am_rest.size() == taken.size();
         for (int i = 0; ok && i < ng; ++i) {
@@ -141,7 +145,8 @@ bool batch_plain_ready(kps_batch *b, cudaStream_t stream) {
         std::string why;
         std::vector<char> taken;
         kps::am_destroy(b->am_plain[dir]);
-        b->am_plain[dir] = kps::am_create(am_descs(b, dir), 2 * sm_count(), true, stream, &taken, &why);
+        size_t need = 0;
+        b->am_plain[dir] = kps::am_create(am_descs(b, dir), 2 * sm_count(), true, stream, &taken, &why, &need);
     }
     return b->am_plain[0] && b->am_plain[1];
 }
@@ -288,20 +293,26 @@ kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, 
         maxH = std::max(maxH, g->host.H);
         maxnc = std::max(maxnc, g->host.ncards + 1);
     }
-    bool decided = true;   // false: the plan may still be built by a later call
     if (dt == KPS_F64 && batch_f64_ready(b, stream)) {
         s = f64_shape(b);
         b->shape[(int)dt] = s;
         *out = s;
         return KPS_OK;
-    } else if (dt == KPS_F64) {
-        decided = b->f64_state != 0;
+    }
+    const bool staged = dt != KPS_F64 && batch_staged_ready(b, stream);
+    // a plan that may still be built by a later call: a shape for the time being
+    const bool decided = dt == KPS_F64 ? b->f64_state != 0 : b->am_state != 0;
+    if (!decided && b->interim.count((int)dt)) {
+        *out = b->interim[(int)dt];
+        return KPS_OK;
+    }
+    if (dt == KPS_F64) {
         if (maxnc > 64) return fail(KPS_ENOTSUP, "card count too large for the FP64 batch kernel");
         s.nw = 8;
         while (s.nw > 1 && kps::vec_smem_bytes(storage, maxnc, s.nw) > (size_t)kps::max_dyn_smem()) --s.nw;
         s.nw = std::max(1, std::min(s.nw, (maxH + kps::kTile - 1) / kps::kTile));
         s.per_sm = std::max(1, kps::vec_multi_ctas_per_sm(storage, b->k, maxnc, s.nw));
-    } else if (batch_staged_ready(b, stream)) {
+    } else if (staged) {
         s.kernel = KPS_BATCH_STAGED;
         s.nw = 4;
         s.per_sm = std::min(kps::am_ctas_per_sm(b->am[0]), kps::am_ctas_per_sm(b->am[1]));
@@ -321,20 +332,17 @@ kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, 
     }
     s.grid = sm_count() * s.per_sm;
     s.schedule = 0;
-    if (decided) b->shape[(int)dt] = s;
+    (decided ? b->shape : b->interim)[(int)dt] = s;
     *out = s;
     return KPS_OK;
 }
 
 bool batch_f64_ready(kps_batch *b, cudaStream_t stream) {
     if (b->f64_state != 0) return b->f64_state == 1;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
-    if (e != cudaSuccess) cudaGetLastError();
-    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-    b->f64_state = -1;
+    if (kps::capturing(stream) || !kps::memory_for(b->f64_need)) return false;
     for (int dir = 0; dir < 2; ++dir) {
         std::string why;
+        size_t need = 1;
         try {
             std::vector<kps::F64GameDesc> d;
             for (size_t i = 0; i < b->games.size(); ++i) {
@@ -342,12 +350,14 @@ bool batch_f64_ready(kps_batch *b, cudaStream_t stream) {
                 d.back().in_off = b->off[dir == 0 ? 1 : 0][i];
                 d.back().out_off = b->off[dir == 0 ? 0 : 1][i];
             }
-            b->f64[dir] = kps::f64_create(d, true, stream, &why);
+            b->f64[dir] = kps::f64_create(d, true, stream, &why, &need);
         } catch (const std::bad_alloc &) {
         }
         if (!b->f64[dir]) {
             kps::f64_destroy(b->f64[0]);
             b->f64[0] = nullptr;
+            b->f64_state = need > 0 ? 0 : -1;   // no memory: a later call tries again
+            b->f64_need = need;
             return false;
         }
     }
@@ -447,7 +457,7 @@ kps_status kps_batch_create(kps_game *const *games, int32_t n, kps_batch **out) 
         for (int p = 0; p < 2; ++p) b->off[p][i + 1] = b->off[p][i] + (long long)g->host.n[p] * g->host.hs;
     }
     cudaGetDevice(&b->device);
-    cudaError_t e = cudaMalloc(&b->ticket, 256);
+    cudaError_t e = kps::device_malloc(&b->ticket, 256);
     if (e != cudaSuccess) { delete b; return fail(KPS_ENOMEM, "ticket counter"); }
     *out = b;
     return KPS_OK;
@@ -532,8 +542,8 @@ kps_status kps_batch_tune(kps_batch *b, kps_dtype dt, void *stream_ptr, kps_batc
     const size_t es = dtype_size(dt);
     void *vin = nullptr, *vout = nullptr;
     const size_t nin = std::max(b->off[0].back(), b->off[1].back());
-    cudaError_t e = cudaMalloc(&vin, nin * es);
-    if (e == cudaSuccess) e = cudaMalloc(&vout, nin * es);
+    cudaError_t e = kps::device_malloc(&vin, nin * es);
+    if (e == cudaSuccess) e = kps::device_malloc(&vout, nin * es);
     if (e != cudaSuccess) {
         cudaFree(vin);
         return fail(KPS_ENOMEM, "tuning buffers");

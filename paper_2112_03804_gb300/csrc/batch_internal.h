@@ -38,16 +38,19 @@ struct kps_batch {
     int *ticket = nullptr;           // tile ticket counter (device)
     std::map<std::tuple<int, bool, int>, kps_abi::BatchTable> tables;
     std::map<int, kps_abi::BatchShape> shape;   // per dtype
+    std::map<int, kps_abi::BatchShape> interim; // per dtype, while a plan is not to be had (no memory, capture)
     void *warm = nullptr;            // warm-start feature tables (warm.cu)
     kps::AmPlan *am[2] = {nullptr, nullptr};   // staged FP32 kernel, per direction
     kps::AmPlan *am_plain[2] = {nullptr, nullptr};   // the same with plain rows (the solver's)
-    int am_state = 0;                // 0 not tried, 1 built, -1 it takes no game
+    int am_state = 0;                // 0 not tried or no memory, 1 built, -1 it takes no game
+    size_t am_need = 0;              // bytes a plan could not get (state 0)
     std::vector<char> am_rest;       // per game: 1 when the staged kernel leaves it to the tensor-memory one
     int am_nrest = 0;
     int rest_nw = 0;                 // warps of the tensor-memory launch over those games
     std::map<int, kps_abi::BatchTable> rest_tables;   // per direction
     kps::F64Plan *f64[2] = {nullptr, nullptr};        // FP64 kernel, per direction
-    int f64_state = 0;               // 0 not tried, 1 built, -1 a game does not fit
+    int f64_state = 0;               // 0 not tried or no memory, 1 built, -1 a game does not fit
+    size_t f64_need = 0;             // as am_need
 };
 
 namespace kps_abi {

@@ -457,6 +457,33 @@ cudaError_t ensure_dyn_smem(const void *fn, size_t smem) {
     return cudaSuccess;
 }
 
+cudaError_t device_malloc(void **p, size_t bytes) {
+    // test hook (KPS_TEST_FAIL_ALLOC=n): allocations of n bytes and more find no memory
+    const char *t = std::getenv("KPS_TEST_FAIL_ALLOC");
+    if (t && (long long)bytes >= std::atoll(t)) bytes = (size_t)1 << 60;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+
+bool memory_for(size_t need) {
+    size_t room = 0, total = 0;
+    if (need == 0) return true;
+    if (cudaMemGetInfo(&room, &total) == cudaSuccess) return room >= need;
+    cudaGetLastError();
+    return false;
+}
+
+bool capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 cudaError_t upload_table(void **dev, const void *src, size_t bytes, cudaStream_t stream) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(stream, &cap);
@@ -470,7 +497,7 @@ cudaError_t upload_table(void **dev, const void *src, size_t bytes, cudaStream_t
     }
     void *p = nullptr;
     if (e == cudaSuccess) {
-        e = cudaMalloc(&p, bytes);
+        e = device_malloc(&p, bytes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
         if (own) cudaStreamDestroy(stream);

@@ -43,6 +43,22 @@ int max_dyn_smem();
 // on the current device (set once per kernel, device and size; thread safe).
 cudaError_t ensure_dyn_smem(const void *fn, size_t smem);
 
+// cudaMalloc, without the error that a failed one leaves in the runtime: a call
+// that goes on without the memory must not find it behind its own launch.
+cudaError_t device_malloc(void **p, size_t bytes);
+template <typename T>
+cudaError_t device_malloc(T **p, size_t bytes) {
+    void *v = nullptr;
+    const cudaError_t e = device_malloc(&v, bytes);
+    *p = static_cast<T *>(v);
+    return e;
+}
+// Is there device memory for a plan that could not be allocated before?
+// (need: its bytes, 0 when none was missing)
+bool memory_for(size_t need);
+// Is `stream` capturing (or not to be asked, because another one is)?
+bool capturing(cudaStream_t stream);
+
 // New device memory in *dev with a copy of the host bytes, there when the call
 // returns.  On a capturing stream the copy goes through a stream of its own (a
 // table is not a part of the graph, and a captured product may be the first
@@ -190,7 +206,9 @@ struct HostGame;
 TmaParams *tma_create(const HostGame &h, const double *lam_in, const double *lam_out, int n_out, int n_in,
                       const int *hfcol, const int *hscol, const double *fcoef, const double *scoef, std::string *why);
 void tma_destroy(TmaParams *p);
-// One product: out (device, [batch][n_out][hs]) from vin ([batch][n_in][hs]),
+// Copies the record tables to the device on the first call.
+cudaError_t tma_upload(TmaParams *p, cudaStream_t stream);
+// One product (tables uploaded): out (device, [batch][n_out][hs]) from vin ([batch][n_in][hs]),
 // both 16-byte aligned.
 cudaError_t launch_tma_scan(TmaParams *p, int storage, const void *vin, void *vout, int batch, cudaStream_t stream);
 // Reads and clears the flag the TMA-staged kernel sets when a bounded wait
@@ -200,7 +218,8 @@ cudaError_t tma_take_error(bool *set);
 // FP64 path (kernels_f64.cu) for two-card games with few ties: one game and
 // many vectors, or (multi) many games with one vector each.  Builds and uploads
 // the plan (synchronises `stream`); nullptr with *why set when a game does not
-// fit.
+// fit, or, with *need set to the bytes of the plan, when it was not to be had
+// just now.
 struct F64GameDesc {
     const HostGame *h;
     const double *lam_in, *lam_out;   // host, library order
@@ -211,7 +230,8 @@ struct F64GameDesc {
     long long in_off, out_off;        // element offsets in the batch vectors
 };
 struct F64Plan;
-F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why);
+F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why,
+                    size_t *need);
 void f64_destroy(F64Plan *p);
 constexpr int kF64Warps = 6;          // warps of a CTA
 int f64_items(const F64Plan *p);      // CTAs of a launch over many games
@@ -240,8 +260,9 @@ struct AmPlan;
 // 32 rows, every row scanned with its own payoffs (the solver's products, whose
 // roundings must not depend on how rows are grouped: a regret within rounding
 // of the matching floor decides a strategy entry).
+// *need as for f64_create.
 AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                  std::vector<char> *taken, std::string *why);
+                  std::vector<char> *taken, std::string *why, size_t *need);
 void am_destroy(AmPlan *p);
 int am_ctas_per_sm(const AmPlan *p);
 int am_grid_cap(const AmPlan *p);

@@ -640,7 +640,7 @@ struct AmPlan {
 
 namespace {
 AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                   std::vector<char> *taken, std::string *why) {
+                   std::vector<char> *taken, std::string *why, size_t *need) {
     if (games.empty() || grid_cap < 1) {
         *why = "no games";
         return nullptr;
@@ -658,13 +658,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
             *why = "games with different hand sizes";
             return nullptr;
         }
-        std::string w;
-        try {
-            w = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, true, &rec[i]);
-        } catch (const std::bad_alloc &) {
-            *why = "host allocation";
-            return nullptr;
-        }
+        std::string w = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, true, &rec[i]);
         if (w.empty() && rec[i].hs % 8 != 0) w = "hand stride not a multiple of 8";
         if (!w.empty()) {
             // left to another kernel
@@ -787,17 +781,14 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
     const size_t total = o_rec + rbytes;
     std::vector<unsigned char> host(total, 0);
     std::vector<AmGame> g(ng);
-    AmPlan *p = new (std::nothrow) AmPlan();
-    if (!p) {
-        *why = "host allocation";
-        return nullptr;
-    }
-    cudaError_t e = cudaMalloc(&p->blob, total);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&p->scratch, (size_t)grid_cap * kTmaWarps * kMaxExtra * kTmaBox * 32 * sizeof(float));
+    const size_t scratch = (size_t)grid_cap * kTmaWarps * kMaxExtra * kTmaBox * 32 * sizeof(float);
+    AmPlan *p = new AmPlan();
+    cudaError_t e = device_malloc(&p->blob, total);
+    if (e == cudaSuccess) e = device_malloc(&p->scratch, scratch);
     if (e != cudaSuccess) {
         if (p->blob) cudaFree(p->blob);
         delete p;
+        *need = total + scratch;
         *why = "device memory for the launch tables";
         return nullptr;
     }
@@ -840,6 +831,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         cudaFree(p->blob);
         cudaFree(p->scratch);
         delete p;
+        *need = total + scratch;
         *why = "uploading the launch tables";
         return nullptr;
     }
@@ -855,10 +847,12 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
 }  // namespace
 
 AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                  std::vector<char> *taken, std::string *why) {
+                  std::vector<char> *taken, std::string *why, size_t *need) {
+    *need = 0;
     try {
-        return build_plan(games, grid_cap, plain, stream, taken, why);
+        return build_plan(games, grid_cap, plain, stream, taken, why, need);
     } catch (const std::bad_alloc &) {
+        *need = 1;
         *why = "host allocation";
         return nullptr;
     }

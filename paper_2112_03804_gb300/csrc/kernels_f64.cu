@@ -361,7 +361,9 @@ struct F64Plan {
     int nunit = 0, nother = 0;     // one game: rows by kind
 };
 
-F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why) {
+F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStream_t stream, std::string *why,
+                    size_t *need) {
+    *need = 0;
     const int ng = (int)games.size();
     std::vector<std::vector<unsigned char>> rec(ng);
     std::vector<size_t> ties_at(ng);
@@ -474,12 +476,13 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         build(least, &items);
     }
     F64Plan *p = new (std::nothrow) F64Plan();
-    if (!p) { *why = "host allocation"; return nullptr; }
+    if (!p) { *why = "host allocation"; *need = 1; return nullptr; }
     const size_t o_items = al(sizeof(Game) * ng), o_rows = o_items + al(sizeof(int4) * items.size()),
                  o_rec = o_rows + al(sizeof(int2) * nrows), total = o_rec + rbytes;
-    cudaError_t e = cudaMalloc(&p->blob, total);
+    cudaError_t e = device_malloc(&p->blob, total);
     if (e != cudaSuccess) {
         delete p;
+        *need = total;
         *why = "device memory for the launch tables";
         return nullptr;
     }
@@ -514,6 +517,7 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
         f64_destroy(p);
+        *need = total;
         *why = "uploading the launch tables";
         return nullptr;
     }

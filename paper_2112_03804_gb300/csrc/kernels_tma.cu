@@ -998,20 +998,23 @@ void tma_destroy(TmaParams *p) {
     delete p;
 }
 
-cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *vout, int batch, cudaStream_t stream) {
+cudaError_t tma_upload(TmaParams *pp, cudaStream_t stream) {
     TmaParams &p = *pp;
+    if (p.dev) return cudaSuccess;
+    cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p.a.err), g_tma_err);
+    if (e != cudaSuccess) return e;
+    e = upload_table(&p.dev, p.host.data(), p.host.size(), stream);
+    if (e != cudaSuccess) return e;
+    p.a.rscan = static_cast<const unsigned char *>(p.dev);
+    p.a.rfin = reinterpret_cast<const TmaFinRec *>(static_cast<const unsigned char *>(p.dev) +
+                                                   (size_t)p.a.nbox * kScanBlock);
+    cudaGetDevice(&p.device);
+    return cudaSuccess;
+}
+
+cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *vout, int batch, cudaStream_t stream) {
+    const TmaParams &p = *pp;
     cudaError_t e;
-    if (!p.dev) {
-        // the record tables go to the device on the first product
-        e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p.a.err), g_tma_err);
-        if (e != cudaSuccess) return e;
-        e = upload_table(&p.dev, p.host.data(), p.host.size(), stream);
-        if (e != cudaSuccess) return e;
-        p.a.rscan = static_cast<const unsigned char *>(p.dev);
-        p.a.rfin = reinterpret_cast<const TmaFinRec *>(static_cast<const unsigned char *>(p.dev) +
-                                                       (size_t)p.a.nbox * kScanBlock);
-        cudaGetDevice(&p.device);
-    }
     TmaArgs A = p.a;   // a copy: other threads may launch the same game's products
     A.batch = batch;
     A.nbb = (batch + 31) / 32;

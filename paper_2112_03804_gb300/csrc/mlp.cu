@@ -414,14 +414,14 @@ kps_status ensure_cap(kps_mlp *m, int rows) {
     m->H1 = m->H2 = m->Z = m->dZ = m->dH1 = m->dH2 = m->row_loss = m->part = nullptr;
     m->cap = 0;
     const size_t r = (size_t)rows;
-    cudaError_t e = cudaMalloc(&m->H1, r * m->width * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->H2, r * m->width * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->Z, r * m->dout * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->dZ, r * m->dout * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->dH1, r * m->width * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->dH2, r * m->width * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->row_loss, r * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->part, part_floats(m) * 4);
+    cudaError_t e = kps::device_malloc(&m->H1, r * m->width * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->H2, r * m->width * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->Z, r * m->dout * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->dZ, r * m->dout * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->dH1, r * m->width * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->dH2, r * m->width * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->row_loss, r * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->part, part_floats(m) * 4);
     if (e != cudaSuccess) return fail(KPS_ENOMEM, "network activations");
     m->cap = rows;
     return KPS_OK;
@@ -525,12 +525,12 @@ kps_status kps_mlp_create(int32_t din, int32_t width, int32_t dout, uint64_t see
         std::normal_distribution<float> nd(0.f, std::sqrt(2.f / fan[l]));
         for (long long i = m->off[2 * l]; i < m->off[2 * l + 1]; ++i) host[i] = nd(rng);
     }
-    cudaError_t e = cudaMalloc(&m->p, n * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->g, n * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->m, n * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->v, n * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&m->ph, n * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&m->wsum, 4);
+    cudaError_t e = kps::device_malloc(&m->p, n * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->g, n * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->m, n * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->v, n * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->ph, n * 2);
+    if (e == cudaSuccess) e = kps::device_malloc(&m->wsum, 4);
     if (e != cudaSuccess) {
         kps_mlp_destroy(m);
         return fail(KPS_ENOMEM, "network parameters");

@@ -704,7 +704,7 @@ kps_status ensure_dtab(kps_solver *s, long long last, cudaStream_t st) {
         h[3 * t + 2] = std::pow((double)t, s->gamma);
     }
     double *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(double)) != cudaSuccess) return fail(KPS_ENOMEM, "DCFR table");
+    if (kps::device_malloc(&d, h.size() * sizeof(double)) != cudaSuccess) return fail(KPS_ENOMEM, "DCFR table");
     cudaError_t e = cudaMemcpy(d, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(d);
@@ -807,7 +807,7 @@ kps_status kps_solver_create(kps_batch *b, kps_dtype dt, kps_solver **out) {
     std::memcpy(host.data() + o_gb, game_blocks.data(), 4 * (size_t)ng);
     if (!nodes.empty()) std::memcpy(host.data() + o_nd, nodes.data(), sizeof(int4) * nodes.size());
     auto alloc = [&](size_t bytes, void **p) -> bool {
-        if (cudaMalloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) return false;
+        if (kps::device_malloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) return false;
         s->allocs.push_back(*p);
         return true;
     };

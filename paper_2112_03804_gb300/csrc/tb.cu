@@ -240,7 +240,7 @@ kps_status cusparse_plan(kps_tb *tb, int batch, kps_dtype dt, const void *y, voi
         if (tb->cbuf) cudaFree(tb->cbuf);
         tb->cbuf = nullptr;
         tb->cbuf_bytes = 0;
-        cudaError_t e = cudaMalloc(&tb->cbuf, need > 0 ? need : 1);
+        cudaError_t e = kps::device_malloc(&tb->cbuf, need > 0 ? need : 1);
         if (e != cudaSuccess) return fail(KPS_ENOMEM, "cuSPARSE workspace");
         tb->cbuf_bytes = need;
     }
@@ -305,7 +305,7 @@ kps_status tb_upload(kps_tb *tb, cudaStream_t stream) {
         if (nnz) std::memcpy(host.data() + o[w][3], h.val.data(), 8 * nnz);
     }
     void *blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, off);
+    cudaError_t e = kps::device_malloc(&blob, off);
     if (e != cudaSuccess) return fail(KPS_ENOMEM, "Technique B factors");
     e = cudaMemcpyAsync(blob, host.data(), off, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -403,7 +403,7 @@ kps_status kps_tb_matvec(kps_tb *tb, const void *y, void *out, int32_t batch, kp
         if (tb->tmp) cudaFree(tb->tmp);
         tb->tmp = tb->tmp2 = nullptr;
         tb->tmp_bytes = 0;
-        if (cudaMalloc(&tb->tmp, 2 * one) != cudaSuccess) return fail(KPS_ENOMEM, "Technique B workspace");
+        if (kps::device_malloc(&tb->tmp, 2 * one) != cudaSuccess) return fail(KPS_ENOMEM, "Technique B workspace");
         tb->tmp_bytes = 2 * one;
     }
     tb->tmp2 = static_cast<char *>(tb->tmp) + one;

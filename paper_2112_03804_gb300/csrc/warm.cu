@@ -622,7 +622,7 @@ kps_status warm_tables(kps_batch *b, const WarmTables **out) {
     std::memcpy(host.data() + o_nf, node_feat.data(), 4 * node_feat.size());
     WarmTables *t = new (std::nothrow) WarmTables;
     if (!t) return fail(KPS_ENOMEM, "warm-start tables");
-    if (cudaMalloc(&t->blob, total) != cudaSuccess) {
+    if (kps::device_malloc(&t->blob, total) != cudaSuccess) {
         delete t;
         return fail(KPS_ENOMEM, "warm-start tables");
     }
@@ -720,9 +720,9 @@ kps_status kps_warm_predict(kps_batch *b, kps_mlp *m, float *beh1, float *beh2, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int ng = t->d.ngames, nn = t->d.total_nodes;
     float *Gf = nullptr, *G1 = nullptr, *N1 = nullptr;
-    cudaError_t e = cudaMalloc(&Gf, (size_t)2 * ng * kOffNode * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&G1, (size_t)2 * ng * kWidth * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&N1, (size_t)std::max(nn, 1) * kWidth * 4);
+    cudaError_t e = kps::device_malloc(&Gf, (size_t)2 * ng * kOffNode * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&G1, (size_t)2 * ng * kWidth * 4);
+    if (e == cudaSuccess) e = kps::device_malloc(&N1, (size_t)std::max(nn, 1) * kWidth * 4);
     if (e != cudaSuccess) {
         cudaFree(Gf);
         cudaFree(G1);
