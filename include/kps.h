@@ -28,6 +28,11 @@
  *   the most recent failure of the calling thread.
  * Streams: `stream` is a cudaStream_t passed as void* (NULL = the legacy
  *   default stream).  GPU calls are asynchronous on that stream.
+ * Threads: products of one game from device vectors (kps_matvec_A / _AT) may be
+ *   called by several threads at once, each on its own stream, from the first
+ *   one on; only KPS_KERNEL_SCALAR with 16-bit vectors keeps partial results in
+ *   a buffer of the game, as the host-buffer products keep their staging
+ *   buffers.  Every other object belongs to one thread at a time.
  * Hand order ("library order"): hands sorted by ascending strength, ties
  *   broken by canonical index.  The canonical order is the deck minus the
  *   board in increasing card id (card id = rank*suits + suit); one-card hands

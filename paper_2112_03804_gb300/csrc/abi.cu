@@ -69,12 +69,14 @@ std::string split_rows(kps_game *g) {
 }
 
 kps_status upload(kps_game *g, cudaStream_t stream) {
-    if (g->uploaded) {
+    auto here = [&]() -> kps_status {
         int dev = -1;
         cudaGetDevice(&dev);
-        if (dev != g->device) return fail(KPS_EINVAL, "game tables live on another device");
-        return KPS_OK;
-    }
+        return dev == g->device ? KPS_OK : fail(KPS_EINVAL, "game tables live on another device");
+    };
+    if (g->uploaded) return here();
+    std::lock_guard<std::mutex> lock(g->first);
+    if (g->uploaded) return here();
     const kps::HostGame &h = g->host;
     const int H = h.H;
     // layout of the blob (8-byte aligned pieces)
@@ -150,7 +152,8 @@ kps_status upload(kps_game *g, cudaStream_t stream) {
 }
 
 kps_status tiles_for(kps_game *g, int nw, cudaStream_t stream, const kps_game::Tiles **out) {
-    auto it = g->tiles.find(nw);
+    std::lock_guard<std::mutex> lock(g->first);
+    auto it = g->tiles.find(nw);   // (an entry stays where it is)
     if (it == g->tiles.end()) {
         kps_game::Tiles t;
         std::vector<std::pair<int, int>> tl = layout_tiles(g->host, nw, t.tchunk, &t.spill);
@@ -355,23 +358,32 @@ kps_status matvec_tma(kps_game *g, int dir, const void *vin, void *vout, int32_t
     if (force && std::strcmp(force, "tma") != 0) return KPS_OK;
     if (((reinterpret_cast<uintptr_t>(vin) | reinterpret_cast<uintptr_t>(vout)) & 15) != 0) return KPS_OK;
     if (g->tma_state[dir] == 0) {
-        const kps::HostGame &h = g->host;
-        const double *lin = dir == 0 ? h.lam2.data() : h.lam1.data();
-        const double *lout = dir == 0 ? h.lam1.data() : h.lam2.data();
+        std::lock_guard<std::mutex> lock(g->first);
         std::string why;
-        kps::TmaParams *p = kps::tma_create(h, lin, lout, dir == 0 ? h.n[0] : h.n[1], dir == 0 ? h.n[1] : h.n[0],
-                                            g->fcol[dir].data(), g->scol[dir].data(), g->fcoef[dir].data(),
-                                            g->scoef[dir].data(), &why);
-        g->tma[dir].reset(p);
-        g->tma_state[dir] = p ? 1 : why == "host allocation" ? 0 : -1;   // no memory: a later call tries again
+        if (g->tma_state[dir] == 0 && !g->tma[dir]) {
+            const kps::HostGame &h = g->host;
+            const double *lin = dir == 0 ? h.lam2.data() : h.lam1.data();
+            const double *lout = dir == 0 ? h.lam1.data() : h.lam2.data();
+            g->tma[dir].reset(kps::tma_create(h, lin, lout, dir == 0 ? h.n[0] : h.n[1], dir == 0 ? h.n[1] : h.n[0],
+                                              g->fcol[dir].data(), g->scol[dir].data(), g->fcoef[dir].data(),
+                                              g->scoef[dir].data(), &why));
+            if (!g->tma[dir] && why != "host allocation") g->tma_state[dir] = -1;
+        }
+        if (g->tma_state[dir] == 0 && g->tma[dir]) {
+            const cudaError_t e = kps::tma_upload(g->tma[dir].get(), stream);
+            // no memory: the tensor-memory kernel needs less, and a later call tries again
+            if (e == cudaErrorMemoryAllocation) return KPS_OK;
+            if (e != cudaSuccess) {
+                *taken = true;
+                return cuda_fail(e, "uploading the tables of the TMA-staged payoff scan");
+            }
+            g->tma_state[dir] = 1;
+        }
     }
     if (g->tma_state[dir] != 1) return KPS_OK;
-    cudaError_t e = kps::tma_upload(g->tma[dir].get(), stream);
-    if (e == cudaErrorMemoryAllocation) return KPS_OK;   // the tensor-memory kernel needs less
     *taken = true;
-    if (e != cudaSuccess) return cuda_fail(e, "uploading the tables of the TMA-staged payoff scan");
     g->last_kernel[dir] = KPS_KERNEL_TMA;
-    e = kps::launch_tma_scan(g->tma[dir].get(), storage, vin, vout, batch, stream);
+    const cudaError_t e = kps::launch_tma_scan(g->tma[dir].get(), storage, vin, vout, batch, stream);
     if (e != cudaSuccess) return cuda_fail(e, "launching the TMA-staged payoff scan");
     return KPS_OK;
 }
@@ -404,17 +416,19 @@ kps_status matvec_f64(kps_game *g, int dir, const void *vin, void *vout, int32_t
     if (g->f64_state[dir] == 0) {
         // the plan is uploaded with a synchronisation, which a capturing stream
         // cannot do: the other FP64 kernel's tables may be there already
-        if (kps::capturing(stream) || !kps::memory_for(g->f64_need[dir])) return KPS_OK;
-        std::string why;
-        size_t need = 1;
-        kps::F64Plan *p = nullptr;
-        try {
-            p = kps::f64_create({f64_desc(g, dir)}, false, stream, &why, &need);
-        } catch (const std::bad_alloc &) {
+        if (kps::capturing(stream)) return KPS_OK;
+        std::lock_guard<std::mutex> lock(g->first);
+        if (g->f64_state[dir] == 0) {
+            if (!kps::memory_for(g->f64_need[dir])) return KPS_OK;
+            std::string why;
+            size_t need = 1;
+            try {
+                g->f64[dir].reset(kps::f64_create({f64_desc(g, dir)}, false, stream, &why, &need));
+            } catch (const std::bad_alloc &) {
+            }
+            g->f64_need[dir] = need;
+            g->f64_state[dir] = g->f64[dir] ? 1 : need > 0 ? 0 : -1;   // no memory: a later call tries again
         }
-        g->f64[dir].reset(p);
-        g->f64_state[dir] = p ? 1 : need > 0 ? 0 : -1;   // no memory: a later call tries again
-        g->f64_need[dir] = need;
     }
     if (g->f64_state[dir] != 1) return KPS_OK;
     *taken = true;

@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <atomic>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -42,7 +44,11 @@ struct kps_game {
     // per output row of each direction (0 = A, 1 = A^T): terminal pairs
     std::vector<int> fcol[2], scol[2];
     std::vector<double> fcoef[2], scoef[2];
-    bool uploaded = false;
+    // Threads may make the game's first products at the same time: `first` is held
+    // while tables and plans are built and uploaded; what a later call reads
+    // without it (uploaded, the states at 1) is set last.
+    std::mutex first;
+    std::atomic<bool> uploaded{false};
     int device = -1;
     kps_abi::DeviceTables dev;
     void *stage_in = nullptr, *stage_out = nullptr;
@@ -64,26 +70,26 @@ struct kps_game {
     };
     std::map<int, Tiles> tiles;
     // warps per CTA of the tensor-memory path (0 = not chosen yet)
-    int tmem_nw = 0;
+    std::atomic<int> tmem_nw{0};
     // FP32 partial results for half-precision outputs
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
-    // parameter blocks of the TMA-staged FP32 path per direction, built on
-    // first use (state 1), or -1 when the game cannot take that path
+    // parameter blocks of the TMA-staged path per direction, built and uploaded
+    // on first use (state 1), or -1 when the game cannot take that path
     struct TmaDel {
         void operator()(kps::TmaParams *p) const { kps::tma_destroy(p); }
     };
     std::unique_ptr<kps::TmaParams, TmaDel> tma[2];
-    int tma_state[2] = {0, 0};
+    std::atomic<int> tma_state[2] = {0, 0};
     // plans of the FP64 path per direction, as above
     struct F64Del {
         void operator()(kps::F64Plan *p) const { kps::f64_destroy(p); }
     };
     std::unique_ptr<kps::F64Plan, F64Del> f64[2];
-    int f64_state[2] = {0, 0};
+    std::atomic<int> f64_state[2] = {0, 0};
     size_t f64_need[2] = {0, 0};      // bytes a plan could not get (state 0)
     // kernel of the last product per direction (KPS_KERNEL_* of kps.h)
-    int last_kernel[2] = {0, 0};
+    std::atomic<int> last_kernel[2] = {0, 0};
 };
 
 namespace kps_abi {

@@ -1015,7 +1015,8 @@ cudaError_t tma_upload(TmaParams *pp, cudaStream_t stream) {
 cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *vout, int batch, cudaStream_t stream) {
     const TmaParams &p = *pp;
     cudaError_t e;
-    TmaArgs A = p.a;   // a copy: other threads may launch the same game's products
+    TmaArgs A = p.a;   // a copy: other threads may launch the same game's products (the first ones under
+                       // its lock until the tables are there)
     A.batch = batch;
     A.nbb = (batch + 31) / 32;
     // test hook (KPS_TEST_STALL_WAIT=1): one barrier per CTA never completes,
