@@ -81,7 +81,6 @@ struct AmArgs {
     const AmGame *games;
     const int4 *items;             // (game, first row, split, last row + 1)
     int nitems, nc, schedule;
-    int unit;                      // showdown-only rows are scanned with S = 1
     const void *vin;               // element type: the kernel's storage type
     void *vout;
     float *scratch;                // [grid][4 warps][kMaxExtra][16][32]
@@ -208,11 +207,16 @@ __device__ __forceinline__ uint32_t hand_bytes(int left) {
 // the second half of the warp's chunk (eight sub-chunks in all), and the half
 // with fewer boxes runs zero-filled boxes to the other's count, so that the
 // warp's tensor-memory operations stay uniform.
-template <typename T, int K2>
+// PAIRS: the rows are pairs and what is left alone, showdown-only rows scanned
+// with S = 1.  TIES: a game of the batch lists ties of more than 4 hands.  A plan
+// without them runs code without them (184 to 205 registers instead of 240): 512
+// uneven games with single rows and no long ties 168 -> 158 us, 256 river games in
+// pairs 64.6 -> 62.
+template <typename T, int K2, bool PAIRS, bool TIES>
 __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int row0, int row1, int split,
                                         unsigned char *sm, uint32_t tmem, float *xs) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nc = P.nc, hs = G.hs;
+    const int nc = P.nc, hs = G.hs, H = G.H;
     const int half = split ? lane >> 4 : 0, col = split ? lane & 15 : lane;
     const int sub = split ? 2 * warp + half : warp;   // this lane's (sub-)chunk
     const int b0 = split ? G.bchunk8[sub] : G.bchunk[warp];
@@ -221,21 +225,23 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
     const int nbh0 = __shfl_sync(kFull, nbl, 0), nbh1 = __shfl_sync(kFull, nbl, 16);
     const int nb = split ? max(nbh0, nbh1) : nbl;   // the warp's box count
     const bool act = row0 + col < row1;
-    const int2 sq = act ? G.rows[row0 + col] : make_int2(0, -1);
+    // without pairs a row is the sequence of its number
+    const int2 sq = !act ? make_int2(0, -1) : PAIRS ? G.rows[row0 + col] : make_int2(row0 + col, -1);
     const int sigma = sq.x;
     const int rf = act ? G.fcol[sigma] : -1, rs = act ? G.scol[sigma] : -1;
     const float F = rf >= 0 ? G.fcoef[sigma] : 0.f;
     // a showdown-only row is scanned with S = 1 and finished with its payoff;
     // Fm: the payoff of its fold-only mate
-    const bool unit = P.unit && rf < 0 && rs >= 0;
+    const bool unit = PAIRS && rf < 0 && rs >= 0;
     const float S = unit ? 1.f : rs >= 0 ? G.scoef[sigma] : 0.f;
     const float So = unit ? G.scoef[sigma] : 1.f, Fm = sq.y >= 0 ? G.fcoef[sq.y] : 0.f;
-    const bool pairs = __any_sync(kFull, sq.y >= 0);
+    const bool pairs = PAIRS && __any_sync(kFull, sq.y >= 0);
     const float S2 = 2.f * S;
     constexpr int NQ = 16 / Store<T>::kPer;   // 16-byte chunks per 16-hand row segment
     const T *vin = static_cast<const T *>(P.vin) + G.in_off;
     const T *pa = vin + (size_t)(rf >= 0 ? rf : 0) * hs;
     const T *pb = vin + (size_t)(rs >= 0 ? rs : 0) * hs;
+    const uint32_t na = rf >= 0 ? 16u : 0u, nbytes_b = rs >= 0 ? 16u : 0u;
     unsigned char *ring = sm + am_ring_off(warp);
     const uint32_t ring_s = smem_u32(ring);
     unsigned char *rring = sm + am_rec_off(warp);
@@ -254,13 +260,22 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
             const bool real = m < nbl;   // past its half's boxes a lane copies zeros
             const int x = kTmaBox * (b0 + (real ? m : 0));
             const uint32_t dst = ring_s + (uint32_t)(sl * kSlot) + 16u * (uint32_t)lane;
+            if (x + kTmaBox <= H) {
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const int h0 = x + Store<T>::kPer * q;
-                const bool in = real && h0 < hs;   // hs is a multiple of 8: a chunk is all in or all out
-                const uint32_t nb_in = hand_bytes<T>(G.H - h0);   // padding hands hold anything: zeros
-                cp16(dst + 512u * q, in ? pa + h0 : pa, in && rf >= 0 ? nb_in : 0u);
-                cp16(dst + 2048u + 512u * q, in ? pb + h0 : pb, in && rs >= 0 ? nb_in : 0u);
+                for (int q = 0; q < NQ; ++q) {
+                    const int h0 = x + Store<T>::kPer * q;
+                    cp16(dst + 512u * q, pa + h0, real ? na : 0u);
+                    cp16(dst + 2048u + 512u * q, pb + h0, real ? nbytes_b : 0u);
+                }
+            } else {   // the last boxes: padding hands hold anything, zeros take their place
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int h0 = x + Store<T>::kPer * q;
+                    const bool in = real && h0 < hs;   // hs is a multiple of 8: a chunk is all in or all out
+                    const uint32_t n = in ? hand_bytes<T>(H - h0) : 0u;
+                    cp16(dst + 512u * q, in ? pa + h0 : pa, min(n, na));
+                    cp16(dst + 2048u + 512u * q, in ? pb + h0 : pb, min(n, nbytes_b));
+                }
             }
             // the record block of each half's box (zeros for a zero-filled box)
             if (lane < kScanBlock / 16) {
@@ -376,7 +391,7 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
         // 1081-hand games).  The game stays on this kernel: in a launch of its own
         // on the tensor-memory kernel it cost a 256-game product 51 us more.
         const uint32_t nent = reinterpret_cast<const uint32_t *>(rsb + 256)[3];
-        if (nent && rs >= 0) {
+        if (TIES && nent && rs >= 0) {
             const TieEntry *te = G.ent + reinterpret_cast<const uint32_t *>(rsb + 256)[2];
 #pragma unroll 1
             for (uint32_t e = 0; e < nent; ++e) {
@@ -515,7 +530,7 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
             for (int q = 0; q < NQ; ++q)
                 if (x + Store<T>::kPer * q < hs)
                     cp16(ring_s + yb + (uint32_t)((m & 1) * 2048) + 512u * q, pb + x + Store<T>::kPer * q,
-                         hand_bytes<T>(G.H - x - Store<T>::kPer * q));
+                         hand_bytes<T>(H - x - Store<T>::kPer * q));
         }
         cp_commit();
     };
@@ -553,8 +568,8 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
                 q1 += *reinterpret_cast<const float *>(qb + r.ob1);
                 q2 += *reinterpret_cast<const float *>(qb + r.ob2);
             }
-            o[i] = (r.lout1 * So) * ((pc[i] + Cw) - q1);
-            o[i + 1] = (r.lout2 * So) * ((pc[i + 1] + Cw) - q2);
+            o[i] = (PAIRS ? r.lout1 * So : r.lout1) * ((pc[i] + Cw) - q1);
+            o[i + 1] = (PAIRS ? r.lout2 * So : r.lout2) * ((pc[i + 1] + Cw) - q2);
         }
         if (act && real) {
             const int x = kTmaBox * (b0 + m);
@@ -585,7 +600,7 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
     __syncwarp();
 }
 
-template <typename T, int K2>
+template <typename T, int K2, bool PAIRS, bool TIES>
 __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_constant__ AmArgs P) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int warp = threadIdx.x >> 5;
@@ -612,7 +627,7 @@ __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_consta
         }
         if (item >= P.nitems) break;
         const int4 it = P.items[item];
-        am_item<T, K2>(P, P.games[it.x], it.y, it.w, it.z, sm, tmem, xs);
+        am_item<T, K2, PAIRS, TIES>(P, P.games[it.x], it.y, it.w, it.z, sm, tmem, xs);
         // the next ticket is written only after every thread has read this one
         // (am_item ends its combination with a CTA barrier)
     }
@@ -624,10 +639,28 @@ __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_consta
 
 }  // namespace
 
-// Time (us) of an item [single rows, pairs][full, split] of a 1081-hand game,
-// {alone on its SM, two per SM}, measured on 8 to 512 river games: what
-// am_create's choice of rows and items goes by.
-constexpr double kItemTime[2][2][2] = {{{35, 52}, {25, 31}}, {{42, 66}, {31, 41}}};
+// Time (us) of an item [single rows, pairs][full, split] of a 1081-hand game in
+// FP32, {alone on its SM, two per SM}, measured on 1 to 600 river games and 20 games
+// of 247 sequences (a full item of pairs alone: 39.3 and 44.2): what am_create's
+// choice of rows and items goes by.  16-bit vectors take 0.75 to 0.8
+// of every entry, and 1128 and 1176 hands a few percent more, so the choice is the
+// same; games of some ten hands, whose items are bound by their fixed parts,
+// take single rows in full items by it too, which is the fastest there (300
+// one-card games of 47 hands 9.4 us; pairs 10.1, split items 18.4).  A choice
+// of mixed games is off by up to a tenth: 200 games of 3 to 5 board cards take
+// 83 us by it, 75 with pairs in split items; 512 take 158 (164 with pairs).
+constexpr double kItemTime[2][2][2] = {{{29.5, 45.5}, {19.5, 27.8}}, {{42, 62}, {26.5, 39.6}}};
+
+namespace {
+template <typename T>
+auto pick(int k, bool pairs, bool ties) {
+    if (k == 1)
+        return pairs ? (ties ? async_multi_kernel<T, 1, true, true> : async_multi_kernel<T, 1, true, false>)
+                     : (ties ? async_multi_kernel<T, 1, false, true> : async_multi_kernel<T, 1, false, false>);
+    return pairs ? (ties ? async_multi_kernel<T, 2, true, true> : async_multi_kernel<T, 2, true, false>)
+                 : (ties ? async_multi_kernel<T, 2, false, true> : async_multi_kernel<T, 2, false, false>);
+}
+}  // namespace
 
 struct AmPlan {
     AmArgs a{};
@@ -635,6 +668,7 @@ struct AmPlan {
     float *scratch = nullptr;
     int grid_cap = 0;              // CTAs the scratch area holds
     int k = 2;
+    bool pairs = false, ties = false;   // the kernel's variant
     int device = -1;
 };
 
@@ -674,11 +708,9 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
     if (ntaken == 0) return nullptr;
     // Rows and items of every game: pairs or single sequences, items of 32 rows
     // (a tail of at most 16 as a split item) or split items alone.  Pairs leave
-    // fewer items, split items half as long a scan: one A product of 512 river
-    // games takes 128 us with pairs in full items, 148 without pairs, of 100 games
-    // 33 us with single rows in split items, 52 in full ones, 43 with pairs; of
-    // the 241 games of a turn endgame (19 sequences, 13 rows) 37 us with pairs, 44
-    // without.
+    // fewer items, split items half as long a scan: one A product of 600 river
+    // games takes 132 us with pairs in full items, 164 without pairs, of
+    // 100 games 28 us with single rows in split items, 46 in full ones, 40 with pairs.
     std::vector<char> can_split(ng, 0);
     std::vector<std::array<int, 2 * kTmaWarps + 1>> sub(ng);
     std::vector<std::vector<int2>> paired(ng), single(ng);
@@ -837,7 +869,8 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
     }
     p->a.games = reinterpret_cast<const AmGame *>(dev + o_games);
     p->a.items = reinterpret_cast<const int4 *>(dev + o_items);
-    p->a.unit = plain ? 0 : 1;
+    p->pairs = rows == &paired;
+    for (int i = 0; i < ng; ++i) p->ties = p->ties || ((*taken)[i] && rec[i].bytes.size() > rec[i].entries_at);
     p->a.nitems = (int)nitems;
     p->a.nc = nc;
     p->k = k;
@@ -895,13 +928,11 @@ cudaError_t launch_async_multi(AmPlan *p, int storage, const void *vin, void *vo
     a.schedule = schedule;
     if (a.nitems == 0) return cudaSuccess;
     const size_t smem = am_launch_smem(a.nc);
-    void (*fn)(AmArgs);
+    void (*fn)(AmArgs) = nullptr;
     switch (storage) {
-        case kStoreF32: fn = p->k == 1 ? async_multi_kernel<float, 1> : async_multi_kernel<float, 2>; break;
-        case kStoreBF16:
-            fn = p->k == 1 ? async_multi_kernel<__nv_bfloat16, 1> : async_multi_kernel<__nv_bfloat16, 2>;
-            break;
-        case kStoreF16: fn = p->k == 1 ? async_multi_kernel<__half, 1> : async_multi_kernel<__half, 2>; break;
+        case kStoreF32: fn = pick<float>(p->k, p->pairs, p->ties); break;
+        case kStoreBF16: fn = pick<__nv_bfloat16>(p->k, p->pairs, p->ties); break;
+        case kStoreF16: fn = pick<__half>(p->k, p->pairs, p->ties); break;
         default: return cudaErrorInvalidValue;
     }
     cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void *>(fn), smem);
