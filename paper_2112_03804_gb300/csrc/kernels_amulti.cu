@@ -392,14 +392,30 @@ __device__ __forceinline__ void am_item(const AmArgs &P, const AmGame &G, int ro
         // on the tensor-memory kernel it cost a 256-game product 51 us more.
         const uint32_t nent = reinterpret_cast<const uint32_t *>(rsb + 256)[3];
         if (TIES && nent && rs >= 0) {
+            // A hand's entries follow one another: they are added up first (sixteen
+            // compares and additions a hand, not an entry), with the next two inputs
+            // and the entry after them under way: 64 games with 924 entries each
+            // 89 -> 58 us, 128 games with 810 90 -> 68.
             const TieEntry *te = G.ent + reinterpret_cast<const uint32_t *>(rsb + 256)[2];
+            const uint32_t last = nent - 1;
+            TieEntry t = te[0], t1 = te[min(1u, last)], t2 = te[min(2u, last)];
+            float y = float(pb[t.q]), y1 = float(pb[t1.q]), sum = 0.f;
 #pragma unroll 1
             for (uint32_t e = 0; e < nent; ++e) {
-                const TieEntry t = te[e];
-                const float x = S * (t.lin * float(pb[t.q]));
+                const TieEntry t3 = te[min(e + 3, last)];
+                const float y2 = float(pb[t2.q]);
+                sum = fmaf(t.lin, y, sum);
+                if (e == last || t1.i != t.i) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (i == t.i) p[i] += x;
+                    for (int i = 0; i < 16; ++i)
+                        if (i == t.i) p[i] = fmaf(S, sum, p[i]);
+                    sum = 0.f;
+                }
+                t = t1;
+                t1 = t2;
+                t2 = t3;
+                y = y1;
+                y1 = y2;
             }
         }
         // every lane has read the slot's records: refill it
