@@ -133,12 +133,18 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRingBytes = 12288;          // per warp: 3 slots of 4 KB or 6 of 2 KB (half of it for 16-bit storage)
+constexpr int kFewBoxes = 4;               // boxes up to which eight warps only add to the fixed part
+constexpr int kSmallBoxes = 24;            // boxes up to which an item is mostly fixed part (kSmall)
 constexpr int kPairMinCards = 48;          // per-card rows from which half a table holds three FP32 boxes
 constexpr int kRecRing = 6 * kScanBlock;   // per warp: one scan block per slot
 constexpr int kTmemCols = 256;             // per four warps (two CTAs of four or one of eight per SM)
 constexpr unsigned long long kWaitNs = 2000000000ull;   // give up after 2 s
 
 enum Kind { kKindF = 1, kKindS = 2, kKindFS = 3 };
+// What a launch's items are: single sequences, pairs (four warps), or single
+// sequences of a game of few boxes.  Each runs a kernel without the code of the
+// others.
+enum Form { kSingle, kPaired, kSmall };
 
 // Shared memory (from a 1 KB aligned base) with nw warps: the warps' rings,
 // their per-card tables (nc rows of 256 bytes), their overflow boxes of partial
@@ -352,8 +358,9 @@ struct Ctx {
 };
 
 // Scan and combination of one column kind; returns this warp's C.  A
-// showdown-only column is scanned with S = 1 (finishing multiplies by S).
-template <typename T, int KIND, int K2, int NW>
+// showdown-only column is scanned with S = 1 (finishing multiplies by S), but in
+// small games with its own.
+template <typename T, int KIND, int K2, int NW, Form FORM>
 __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
     constexpr bool HF = (KIND & kKindF) != 0, HS = (KIND & kKindS) != 0, FS = KIND == kKindFS;
     constexpr int NS = FS ? 3 : 6;                    // ring slots
@@ -372,7 +379,7 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
     unsigned char *lb = stb + (FS ? 8 : 4) * lane;
     float *xpart = reinterpret_cast<float *>(c.sm + extra_off(NW, warp, nc, P.extra));
     float *sums = reinterpret_cast<float *>(hdr + sums_at(NW));
-    const float F = c.F, S = FS ? c.S : 1.f, S2 = 2.f * S;
+    const float F = c.F, S = FS || FORM == kSmall ? c.S : 1.f, S2 = 2.f * S;
     const int nb = c.nb;
     const int z0 = 32 * c.bb;
     auto row = [&](uint32_t off) -> unsigned char * { return lb + (FS ? 2 * off : off); };
@@ -504,6 +511,7 @@ __device__ __forceinline__ float tma_scan(const TmaArgs &P, Ctx &c) {
                 G2 = fmaf(2.f, bb.y, gB);
                 const float2 t = fma2(make_float2(-2.f, -2.f), make_float2(cs1, cs2), make_float2(gA, gB));
                 if (HF) p[k] = fma2(S2v, t, K2 == 2 ? ww : make_float2(0.f, 0.f));
+                else if (FORM == kSmall) p[k] = K2 == 2 ? fma2(S2v, t, mul2(nS2, bb)) : mul2(S2v, t);
                 else p[k] = K2 == 2 ? fma2(nS2, bb, t) : t;   // showdown only: S = 1, w = -b
             } else {
                 p[k] = K2 == 2 ? ww : make_float2(0.f, 0.f);
@@ -784,7 +792,7 @@ __device__ __forceinline__ void tma_finish(const TmaArgs &P, Ctx &c, float Cw, f
     __syncwarp();
 }
 
-template <typename T, int K2, int NW>
+template <typename T, int K2, int NW, Form FORM>
 __global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(const __grid_constant__ TmaArgs P) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled boxes need 1 KB alignment (one KB of slack is allocated)
@@ -813,13 +821,13 @@ __global__ void __launch_bounds__(32 * NW, NW == 4 ? 2 : 1) tma_scan_kernel(cons
     c.tmem = tbase + ((uint32_t)(32 * (c.warp & 3)) << 16) + (uint32_t)(kTmemCols * (c.warp >> 2));
     const int kind = (c.rf >= 0 ? kKindF : 0) | (c.rs >= 0 ? kKindS : 0);
     float Cw;
-    if (kind == kKindFS) Cw = tma_scan<T, kKindFS, K2, NW>(P, c);
-    else if (kind == kKindF) Cw = tma_scan<T, kKindF, K2, NW>(P, c);
-    else Cw = tma_scan<T, kKindS, K2, NW>(P, c);
-    if (NW == 4 && c.sigma2 >= 0) {   // eight warps: items are not paired
+    if (kind == kKindFS) Cw = tma_scan<T, kKindFS, K2, NW, FORM>(P, c);
+    else if (kind == kKindF) Cw = tma_scan<T, kKindF, K2, NW, FORM>(P, c);
+    else Cw = tma_scan<T, kKindS, K2, NW, FORM>(P, c);
+    if (FORM == kPaired && c.sigma2 >= 0) {
         c.F = item.F2;
         tma_finish<T, K2, NW, true, true>(P, c, Cw, c.S);
-    } else if (kind == kKindS) {
+    } else if (FORM != kSmall && kind == kKindS) {
         tma_finish<T, K2, NW, false, true>(P, c, Cw, c.S);
     } else {
         tma_finish<T, K2, NW, false, false>(P, c, Cw, 1.f);
@@ -885,9 +893,11 @@ cudaError_t encode3(CUtensorMap *map, int storage, const void *base, int x, int 
 __device__ unsigned int g_tma_err;
 
 template <typename T>
-auto pick(bool one, int nw) {
-    return one ? (nw == 4 ? tma_scan_kernel<T, 1, 4> : tma_scan_kernel<T, 1, 8>)
-               : (nw == 4 ? tma_scan_kernel<T, 2, 4> : tma_scan_kernel<T, 2, 8>);
+auto pick(bool one, int nw, Form form) {
+    if (nw == 8) return one ? tma_scan_kernel<T, 1, 8, kSingle> : tma_scan_kernel<T, 2, 8, kSingle>;
+    if (form == kPaired) return one ? tma_scan_kernel<T, 1, 4, kPaired> : tma_scan_kernel<T, 2, 4, kPaired>;
+    if (form == kSmall) return one ? tma_scan_kernel<T, 1, 4, kSmall> : tma_scan_kernel<T, 2, 4, kSmall>;
+    return one ? tma_scan_kernel<T, 1, 4, kSingle> : tma_scan_kernel<T, 2, 4, kSingle>;
 }
 
 }  // namespace
@@ -1048,9 +1058,14 @@ cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *v
     // per SM, since a paired item alone takes longer (41 against 35 us a wave):
     // 192 vectors (0.85 / 0.57 waves) single 34.9, paired 41.0 us; 256 (1.13 /
     // 0.76) 54.0, 41.2; 384 (1.70 / 1.14) 60.4, 67.6; 512 (2.26 / 1.53) 80.6, 72.0.
+    // Games of few boxes: up to kFewBoxes four warps (5.2 -> 4.6 us for one vector
+    // of a 47-card one-card game), and up to kSmallBoxes the kernel whose finishing
+    // pass is one for every kind (its instructions are fetched once: 1000 vectors of
+    // a 6-card game 12.3 -> 11.1 us, 300 of a one-card game 6.5 -> 5.8).
     const long long single = (long long)p.nsingle * A.nbb, paired = (long long)p.npaired * A.nbb, slots = 2 * sms;
-    const int nw = p.eight && single <= sms ? 8 : 4;
+    const int nw = p.eight && A.nbox > kFewBoxes && single <= sms ? 8 : 4;
     const bool pair = nw == 4 && (paired + slots - 1) / slots < (single + slots - 1) / slots;
+    const Form form = pair ? kPaired : A.nbox <= kSmallBoxes ? kSmall : kSingle;
     const unsigned char *items = static_cast<const unsigned char *>(p.dev) + p.o_items;
     A.items = reinterpret_cast<const TmaItem *>(items) + (pair ? 0 : p.npaired);
     A.nitems = pair ? p.npaired : p.nsingle;
@@ -1065,9 +1080,9 @@ cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *v
     void (*fn)(TmaArgs) = nullptr;
     const bool one = A.k == 1;
     switch (storage) {
-        case kStoreF32: fn = pick<float>(one, nw); break;
-        case kStoreBF16: fn = pick<__nv_bfloat16>(one, nw); break;
-        case kStoreF16: fn = pick<__half>(one, nw); break;
+        case kStoreF32: fn = pick<float>(one, nw, form); break;
+        case kStoreBF16: fn = pick<__nv_bfloat16>(one, nw, form); break;
+        case kStoreF16: fn = pick<__half>(one, nw, form); break;
         default: return cudaErrorInvalidValue;
     }
     e = ensure_dyn_smem(reinterpret_cast<const void *>(fn), smem);
