@@ -125,6 +125,7 @@ struct TmaParams {
     int npaired = 0, nsingle = 0;
     int chunk4[5] = {}, chunk8[kMaxNw + 1] = {};
     bool eight = false;            // the eight-warp shape fits
+    bool alone = false;            // one CTA of the four-warp shape fills an SM
     int extra4 = 0;                // overflow boxes of the four-warp shape
     int device = -1;
 };
@@ -934,6 +935,8 @@ static std::string tma_prepare(const HostGame &h, const double *lam_in, const do
     }
     p.chunk8[2 * kTmaWarps] = r.nbox;
     p.eight = p.eight && tma_smem_bytes(kMaxNw, r.nc, 0) <= (size_t)max_dyn_smem();
+    // (an SM has the largest CTA's shared memory and its reserved 1 KB)
+    p.alone = 2 * (tma_smem_bytes(kTmaWarps, r.nc, r.extra) + 1024) > (size_t)max_dyn_smem() + 1024;
     p.extra4 = r.extra;
     p.host = std::move(r.bytes);
     return "";
@@ -1058,12 +1061,14 @@ cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *v
     // per SM, since a paired item alone takes longer (41 against 35 us a wave):
     // 192 vectors (0.85 / 0.57 waves) single 34.9, paired 41.0 us; 256 (1.13 /
     // 0.76) 54.0, 41.2; 384 (1.70 / 1.14) 60.4, 67.6; 512 (2.26 / 1.53) 80.6, 72.0.
+    // Where one CTA of four warps fills an SM's shared memory (1128 hands and up)
+    // eight warps always: 100 FP32 vectors 46.6 -> 32.5 us, 384 95.7 -> 65.2.
     // Games of few boxes: up to kFewBoxes four warps (5.2 -> 4.6 us for one vector
     // of a 47-card one-card game), and up to kSmallBoxes the kernel whose finishing
     // pass is one for every kind (its instructions are fetched once: 1000 vectors of
     // a 6-card game 12.3 -> 11.1 us, 300 of a one-card game 6.5 -> 5.8).
     const long long single = (long long)p.nsingle * A.nbb, paired = (long long)p.npaired * A.nbb, slots = 2 * sms;
-    const int nw = p.eight && A.nbox > kFewBoxes && single <= sms ? 8 : 4;
+    const int nw = p.eight && A.nbox > kFewBoxes && (single <= sms || p.alone) ? 8 : 4;
     const bool pair = nw == 4 && (paired + slots - 1) / slots < (single + slots - 1) / slots;
     const Form form = pair ? kPaired : A.nbox <= kSmallBoxes ? kSmall : kSingle;
     const unsigned char *items = static_cast<const unsigned char *>(p.dev) + p.o_items;

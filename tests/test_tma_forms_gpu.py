@@ -1,6 +1,7 @@
 """The TMA-staged kernel's forms at the sizes where the choice changes: games of
-1 to 26 boxes (four warps up to 4 boxes, the small form up to 24) and one-card
-hands, at one vector, a ragged tile and several waves, against the oracle on the rounded inputs.  Tolerances: 1e-5
+1 to 26 boxes (four warps up to 4 boxes, the small form up to 24), one-card hands,
+and 1128 hands, where eight warps take every batch, at one vector, a ragged tile
+and several waves, against the oracle on the rounded inputs.  Tolerances: 1e-5
 normwise for FP32, one output rounding (2^-8 BF16, 2^-10 FP16) for 16-bit storage.
 """
 import numpy as np
@@ -22,11 +23,13 @@ def _deck(ranks, suits, nboard, cards=2):
 
 
 SPECS = {"box1": _deck(4, 2, 2), "box3": _deck(6, 2, 2), "box5": _deck(4, 3, 0), "box7": _deck(4, 4, 1),
-         "box14": _deck(6, 4, 3), "box26": _deck(8, 4, 3), "one_card_box3": _deck(12, 4, 1, 1)}
+         "box14": _deck(6, 4, 3), "box26": _deck(8, 4, 3), "one_card_box3": _deck(12, 4, 1, 1),
+         "turn_board": lambda: synth.river_spec(seed=3, nboard=4, bet_frac=(0.5,))}
 
 
 @pytest.mark.parametrize("dt", list(TOL))
-@pytest.mark.parametrize("name,batch", [(n, b) for n in SPECS for b in (1, 33, 700)])
+@pytest.mark.parametrize("name,batch", [(n, b) for n in SPECS for b in (1, 33, 700) if n != "turn_board"] +
+                         [("turn_board", b) for b in (1, 40, 330)])
 def test_forms(name, batch, dt):
     spec = SPECS[name]()
     og, g = OracleGame(spec), kps.Game(spec)
