@@ -259,6 +259,26 @@ gemm_kernel(int M, int N, int K, int kpart, const TA *__restrict__ A, long long 
     }
 }
 
+// C = A W for few rows, one thread an output: the same sums as gemm_kernel<1>
+// (k in ascending order), which had one CTA per 64 rows walk all k with a
+// barrier every 8: a whole prediction for one game (2 rows of K = 1133 among its
+// products) 187 us with it, 125 here, bound by the round trips of 32 loads at a
+// time.  Every row reads W once more (L2): 256 games' 512 rows are the last that
+// gain (128 games 3.24 -> 3.11 ms, 300 games by tiles as before).
+constexpr int kFewRows = 512;
+__global__ void __launch_bounds__(64) few_rows_kernel(int N, int K, const float *__restrict__ A, long long lda,
+                                                      const __nv_bfloat16 *__restrict__ W, long long ldw,
+                                                      float *__restrict__ C, long long ldc) {
+    const int n = blockIdx.x * 64 + threadIdx.x;
+    if (n >= N) return;
+    const float *a = A + (long long)blockIdx.y * lda;
+    const __nv_bfloat16 *w = W + n;
+    float s = 0.f;
+#pragma unroll 32
+    for (int k = 0; k < K; ++k) s = fmaf(a[k], __bfloat162float(w[(long long)k * ldw]), s);
+    C[(long long)blockIdx.y * ldc + n] = s;
+}
+
 // The z parts of a split product added in order, then the epilogue.
 __global__ void __launch_bounds__(256) reduce_kernel(int M, int N, int nz, const float *__restrict__ part,
                                                      const Epilogue ep) {
@@ -385,6 +405,11 @@ namespace kps_abi {
 cudaError_t mlp_gemm_xw(int M, int N, int K, const float *A, long long lda, const __nv_bfloat16 *W, long long ldw,
                         float *C, long long ldc, cudaStream_t st) {
     // k in ascending order: the predictor's activations are rounded to BF16
+    if (M <= kFewRows) {
+        if (M <= 0 || N <= 0) return cudaSuccess;
+        few_rows_kernel<<<dim3((N + 63) / 64, M), 64, 0, st>>>(N, K, A, lda, W, ldw, C, ldc);
+        return cudaGetLastError();
+    }
     return gemm<1, true, false>(M, N, K, A, lda, W, ldw, Epilogue{C, ldc, nullptr, 0, nullptr, 0}, 1, nullptr, st);
 }
 
