@@ -93,7 +93,7 @@ bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
         std::string why;
         std::vector<char> taken;
         size_t need = 0;
-        b->am[dir] = kps::am_create(d, 2 * sm_count(), false, stream, &taken, &why, &need);
+        b->am[dir] = kps::am_create(d, 2 * sm_count(), stream, &taken, &why, &need);
         if (need > 0) b->am_state = 0;   // no memory: a later call tries again
         b->am_need = need;
         bool ok = b->am[dir] != nullptr && kps::am_ctas_per_sm(b->am[dir]) >= 1;
@@ -137,18 +137,6 @@ bool batch_staged_ready(kps_batch *b, cudaStream_t stream) {
     }
     b->am_state = 1;
     return true;
-}
-
-bool batch_plain_ready(kps_batch *b, cudaStream_t stream) {
-    if (!batch_staged_ready(b, stream)) return false;
-    for (int dir = 0; dir < 2 && (!b->am_plain[0] || !b->am_plain[1]); ++dir) {
-        std::string why;
-        std::vector<char> taken;
-        kps::am_destroy(b->am_plain[dir]);
-        size_t need = 0;
-        b->am_plain[dir] = kps::am_create(am_descs(b, dir), 2 * sm_count(), true, stream, &taken, &why, &need);
-    }
-    return b->am_plain[0] && b->am_plain[1];
 }
 
 namespace {
@@ -391,12 +379,12 @@ kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_
     }
     if (s.kernel == KPS_BATCH_STAGED) {
         cudaError_t e = cudaSuccess;
-        kps::AmPlan *am = plain && b->am_plain[0] && b->am_plain[1] ? b->am_plain[dir] : b->am[dir];
+        kps::AmPlan *am = b->am[dir];
         // no ticket to clear where every CTA has at most one item
-        if (kps::am_items(am) <= s.grid) s.schedule = 1;
+        if (kps::am_items(am, plain) <= s.grid) s.schedule = 1;
         if (s.schedule == 0) e = cudaMemsetAsync(b->ticket, 0, sizeof(int), stream);
         if (e != cudaSuccess) return cuda_fail(e, "clearing the work-item ticket");
-        e = kps::launch_async_multi(am, storage_of(dt), vin, vout, b->ticket, s.schedule, s.grid, stream);
+        e = kps::launch_async_multi(am, plain, storage_of(dt), vin, vout, b->ticket, s.schedule, s.grid, stream);
         if (e != cudaSuccess) return cuda_fail(e, "launching the staged batched payoff scan");
         if (b->am_nrest > 0) {
             // the games the staged kernel leaves: tensor-memory kernel, static stride
@@ -468,7 +456,6 @@ kps_status kps_batch_destroy(kps_batch *b) {
     for (auto &kv : b->tables) cudaFree(kv.second.blob);
     for (auto &kv : b->rest_tables) cudaFree(kv.second.blob);
     for (int k = 0; k < 2; ++k) kps::am_destroy(b->am[k]);
-    for (int k = 0; k < 2; ++k) kps::am_destroy(b->am_plain[k]);
     for (int k = 0; k < 2; ++k) kps::f64_destroy(b->f64[k]);
     warm_free(b);
     if (b->ticket) cudaFree(b->ticket);

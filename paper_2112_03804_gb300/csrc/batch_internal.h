@@ -40,8 +40,7 @@ struct kps_batch {
     std::map<int, kps_abi::BatchShape> shape;   // per dtype
     std::map<int, kps_abi::BatchShape> interim; // per dtype, while a plan is not to be had (no memory, capture)
     void *warm = nullptr;            // warm-start feature tables (warm.cu)
-    kps::AmPlan *am[2] = {nullptr, nullptr};   // staged FP32 kernel, per direction
-    kps::AmPlan *am_plain[2] = {nullptr, nullptr};   // the same with plain rows (the solver's)
+    kps::AmPlan *am[2] = {nullptr, nullptr};   // staged kernel (all storage types but FP64), per direction
     int am_state = 0;                // 0 not tried or no memory, 1 built, -1 it takes no game
     size_t am_need = 0;              // bytes a plan could not get (state 0)
     std::vector<char> am_rest;       // per game: 1 when the staged kernel leaves it to the tensor-memory one
@@ -61,14 +60,12 @@ kps_status batch_table(kps_batch *b, int dir, bool f64, int nw, cudaStream_t str
 kps_status batch_rest_table(kps_batch *b, int dir, cudaStream_t stream, const BatchTable **out);
 kps_status batch_default_shape(kps_batch *b, kps_dtype dt, cudaStream_t stream, BatchShape *out);
 // dir 0: out = A y per game (y player-2 layout, out player-1 layout); dir 1: A^T.
-// plain: the staged kernel's plain rows where batch_plain_ready built them.
+// plain: the staged kernel's plain rows (the solver's products).
 kps_status batch_matvec(kps_batch *b, int dir, const void *vin, void *vout, kps_dtype dt, cudaStream_t stream,
                         bool plain = false);
-// Builds the plans of plain rows (host work, synchronises `stream`); false
-// when the staged kernel does not serve this batch.
-bool batch_plain_ready(kps_batch *b, cudaStream_t stream);
 // Builds the staged kernel's plans on first use (host work, synchronises
-// `stream`); true when every game fits that kernel.
+// `stream`; not on a capturing one); true when that kernel takes games of the
+// batch (those it leaves, b->am_rest, run on the tensor-memory kernel).
 bool batch_staged_ready(kps_batch *b, cudaStream_t stream);
 // Builds the FP64 kernel's plans on first use (not on a capturing stream);
 // true when every game fits that kernel.

@@ -254,22 +254,22 @@ struct AmGameDesc {
 };
 struct AmPlan;
 // Builds and uploads the plan (synchronises `stream`) for the games this
-// path takes ((*taken)[i] = 1; the others, e.g. with a tie group longer than
-// 4 hands, get no work items); nullptr when it takes none or on a failure,
-// *why set.  Scratch for `grid_cap` CTAs.  plain: one sequence per row, items of
-// 32 rows, every row scanned with its own payoffs (the solver's products, whose
-// roundings must not depend on how rows are grouped: a regret within rounding
-// of the matching floor decides a strategy entry).
-// *need as for f64_create.
-AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                  std::vector<char> *taken, std::string *why, size_t *need);
+// path takes ((*taken)[i] = 1; the others, e.g. with more than kMaxTieEntries
+// listed ties in a chunk, get no work items); nullptr when it takes none or on a
+// failure, *why set, *need as for f64_create.  Scratch for `grid_cap` CTAs, shared
+// by both lists of items.  plain: one sequence per row, items of 32 rows, every row
+// scanned with its own payoffs (the solver's products, whose roundings must not
+// depend on how rows are grouped: a regret within rounding of the matching floor
+// decides a strategy entry); else the list that the plan found fastest.
+AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream_t stream, std::vector<char> *taken,
+                  std::string *why, size_t *need);
 void am_destroy(AmPlan *p);
 int am_ctas_per_sm(const AmPlan *p);
 int am_grid_cap(const AmPlan *p);
-int am_items(const AmPlan *p);        // work items of a launch
+int am_items(const AmPlan *p, bool plain);   // work items of a launch
 // One product over every game; ticket: a device counter cleared before the
 // launch when schedule == 0 (ticket), unused when 1 (static stride).
-cudaError_t launch_async_multi(AmPlan *p, int storage, const void *vin, void *vout, int *ticket, int schedule,
+cudaError_t launch_async_multi(AmPlan *p, bool plain, int storage, const void *vin, void *vout, int *ticket, int schedule,
                                int grid, cudaStream_t stream);
 
 }  // namespace kps

@@ -62,14 +62,13 @@ constexpr int kMaxExtra = 8;               // chunk boxes past tensor memory (sc
 
 // One game in one direction (device).
 struct alignas(16) AmGame {
-    int H, hs, nc, n_rows;
-    int nbox, pad0, pad1, pad2;
+    int H, hs, nc, nbox;
     int bchunk[kTmaWarps + 1];
     int pad3[3];
     int bchunk8[2 * kTmaWarps + 1];   // split items: each chunk cut in two at a tie-free box boundary
     int pad4[3];
     long long in_off, out_off;     // element offsets of the game's input / output vectors
-    const int2 *rows;              // [n_rows] output sequence, the fold-only sequence of its pair or -1
+    const int2 *rows;              // of pairs: output sequence, the fold-only sequence of its pair or -1
     const int *fcol, *scol;        // per output sequence: its fold / showdown input sequence or -1
     const float *fcoef, *scoef;    // and the payoffs
     const unsigned char *rscan;    // [nbox][kScanBlock]
@@ -678,19 +677,26 @@ auto pick(int k, bool pairs, bool ties) {
 }
 }  // namespace
 
+// One direction of a batch.  Two lists of items over the same records and scratch
+// area: the fastest ones (0), and plain rows (1).
 struct AmPlan {
     AmArgs a{};
-    void *blob = nullptr;          // games, items, records
+    struct {
+        const int4 *items = nullptr;
+        int n = 0;
+        bool pairs = false;
+    } list[2];
+    bool ties = false;             // a game lists ties of more than 4 hands
+    void *blob = nullptr;          // games, items, rows, records
     float *scratch = nullptr;
     int grid_cap = 0;              // CTAs the scratch area holds
     int k = 2;
-    bool pairs = false, ties = false;   // the kernel's variant
     int device = -1;
 };
 
 namespace {
-AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                   std::vector<char> *taken, std::string *why, size_t *need) {
+AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream_t stream, std::vector<char> *taken,
+                   std::string *why, size_t *need) {
     if (games.empty() || grid_cap < 1) {
         *why = "no games";
         return nullptr;
@@ -700,7 +706,6 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
     taken->assign(ng, 0);
     int nc = 0, ntaken = 0;
     size_t rbytes = 0;
-    long long nitems = 0;
     const int k = games[0].h->k;
     for (int i = 0; i < ng; ++i) {
         const AmGameDesc &d = games[i];
@@ -729,7 +734,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
     // 100 games 28 us with single rows in split items, 46 in full ones, 40 with pairs.
     std::vector<char> can_split(ng, 0);
     std::vector<std::array<int, 2 * kTmaWarps + 1>> sub(ng);
-    std::vector<std::vector<int2>> paired(ng), single(ng);
+    std::vector<std::vector<int2>> paired(ng);
     for (int i = 0; i < ng; ++i) {
         if (!(*taken)[i]) continue;
         const AmGameDesc &d = games[i];
@@ -761,10 +766,8 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
             if (c >= (int)fold_of.size()) fold_of.resize(c + 1, -1);
             if (d.hfcol[s] >= 0 && d.hscol[s] < 0) fold_of[d.hfcol[s]] = s;
         }
-        single[i].reserve(d.n_out);
         paired[i].reserve(d.n_out);
         for (int s = 0; s < d.n_out; ++s) {
-            single[i].push_back(make_int2(s, -1));
             if (d.hfcol[s] >= 0) continue;
             int2 row = make_int2(s, -1);
             if (d.hscol[s] >= 0) {
@@ -778,16 +781,16 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
             if (d.hfcol[s] >= 0 && !mated[s]) paired[i].push_back(make_int2(s, -1));
     }
     // estimated time of a layout (see kItemTime), its items in *out
-    auto layout = [&](const std::vector<std::vector<int2>> &rows, bool halves, std::vector<int4> *out) {
+    auto layout = [&](bool pairs, bool halves, std::vector<int4> *out) {
         double sum = 0.0, alone = 0.0, longest = 0.0;
         long long n_items = 0;
         for (int i = 0; i < ng; ++i) {
-            const int n = (int)rows[i].size();
+            const int n = !(*taken)[i] ? 0 : pairs ? (int)paired[i].size() : games[i].n_out;
             for (int r0 = 0; r0 < n;) {
                 const bool half = can_split[i] && (halves || n - r0 <= 16);
                 const int r1 = std::min(n, r0 + (half ? 16 : 32));
                 if (out) out->push_back(make_int4(i, r0, half ? 1 : 0, r1));
-                const double *c = kItemTime[&rows == &paired ? 1 : 0][half ? 1 : 0];
+                const double *c = kItemTime[pairs ? 1 : 0][half ? 1 : 0];
                 sum += c[1];
                 alone = std::max(alone, c[0]);
                 longest = std::max(longest, c[1]);
@@ -799,23 +802,22 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         return n_items <= grid_cap ? longest : sum / grid_cap + 0.45 * longest;
     };
     double best = 0.0;
-    const std::vector<std::vector<int2>> *rows = nullptr;
-    bool halves = false;
-    for (int v = plain ? 1 : 0; v < (plain ? 2 : 4); ++v) {
-        const auto &rv = v & 1 ? single : paired;
-        const double t = layout(rv, (v & 2) != 0, nullptr);
-        if (!rows || t < best) {
+    int choice = -1;   // bit 0: single rows, bit 1: split items alone
+    for (int v = 0; v < 4; ++v) {
+        const double t = layout((v & 1) == 0, (v & 2) != 0, nullptr);
+        if (choice < 0 || t < best) {
             best = t;
-            rows = &rv;
-            halves = (v & 2) != 0;
+            choice = v;
         }
     }
-    std::vector<int4> items;
-    layout(*rows, halves, &items);
-    nitems = (long long)items.size();
+    const bool pairs = (choice & 1) == 0, same = choice == 1;   // same: plain rows are the fastest
+    std::vector<int4> items[2];
+    layout(pairs, (choice & 2) != 0, &items[0]);
+    if (!same) layout(false, false, &items[1]);
+    const size_t nitems = items[0].size() + items[1].size();
     size_t nrows = 0;
-    for (int i = 0; i < ng; ++i) nrows += (*rows)[i].size();
-    if (nitems > 0x7fffffffLL) {
+    for (int i = 0; i < ng && pairs; ++i) nrows += paired[i].size();
+    if (std::max(items[0].size(), items[1].size()) > 0x7fffffffULL) {
         *why = "too many work items";
         return nullptr;
     }
@@ -824,7 +826,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         return nullptr;
     }
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-    const size_t o_games = 0, o_items = al(sizeof(AmGame) * ng), o_rows = o_items + al(sizeof(int4) * (size_t)nitems),
+    const size_t o_games = 0, o_items = al(sizeof(AmGame) * ng), o_rows = o_items + al(sizeof(int4) * nitems),
                  o_rec = o_rows + al(sizeof(int2) * nrows);
     const size_t total = o_rec + rbytes;
     std::vector<unsigned char> host(total, 0);
@@ -852,10 +854,11 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         x.H = r.H;
         x.hs = r.hs;
         x.nc = r.nc;
-        x.n_rows = (int)(*rows)[i].size();
-        std::memcpy(host.data() + rowo, (*rows)[i].data(), sizeof(int2) * (*rows)[i].size());
-        x.rows = reinterpret_cast<const int2 *>(dev + rowo);
-        rowo += sizeof(int2) * (*rows)[i].size();
+        if (pairs) {
+            std::memcpy(host.data() + rowo, paired[i].data(), sizeof(int2) * paired[i].size());
+            x.rows = reinterpret_cast<const int2 *>(dev + rowo);
+            rowo += sizeof(int2) * paired[i].size();
+        }
         for (int w = 0; w <= 2 * kTmaWarps; ++w) x.bchunk8[w] = sub[i][w];
         x.nbox = r.nbox;
         for (int w = 0; w <= kTmaWarps; ++w) x.bchunk[w] = r.bchunk[w];
@@ -872,7 +875,9 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         ro += al(r.bytes.size());
     }
     std::memcpy(host.data() + o_games, g.data(), sizeof(AmGame) * ng);
-    if (!items.empty()) std::memcpy(host.data() + o_items, items.data(), sizeof(int4) * items.size());
+    for (int l = 0, at = 0; l < 2; at += (int)items[l].size(), ++l)
+        if (!items[l].empty())
+            std::memcpy(host.data() + o_items + sizeof(int4) * at, items[l].data(), sizeof(int4) * items[l].size());
     e = cudaMemcpyAsync(p->blob, host.data(), total, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
@@ -884,10 +889,10 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
         return nullptr;
     }
     p->a.games = reinterpret_cast<const AmGame *>(dev + o_games);
-    p->a.items = reinterpret_cast<const int4 *>(dev + o_items);
-    p->pairs = rows == &paired;
+    p->list[0] = {reinterpret_cast<const int4 *>(dev + o_items), (int)items[0].size(), pairs};
+    if (same) p->list[1] = p->list[0];
+    else p->list[1] = {p->list[0].items + items[0].size(), (int)items[1].size(), false};
     for (int i = 0; i < ng; ++i) p->ties = p->ties || ((*taken)[i] && rec[i].bytes.size() > rec[i].entries_at);
-    p->a.nitems = (int)nitems;
     p->a.nc = nc;
     p->k = k;
     cudaGetDevice(&p->device);
@@ -895,11 +900,11 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, bool plai
 }
 }  // namespace
 
-AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, bool plain, cudaStream_t stream,
-                  std::vector<char> *taken, std::string *why, size_t *need) {
+AmPlan *am_create(const std::vector<AmGameDesc> &games, int grid_cap, cudaStream_t stream, std::vector<char> *taken,
+                  std::string *why, size_t *need) {
     *need = 0;
     try {
-        return build_plan(games, grid_cap, plain, stream, taken, why, need);
+        return build_plan(games, grid_cap, stream, taken, why, need);
     } catch (const std::bad_alloc &) {
         *need = 1;
         *why = "host allocation";
@@ -920,7 +925,7 @@ static size_t am_launch_smem(int nc) { return std::max<size_t>(am_smem_bytes(nc)
 
 int am_grid_cap(const AmPlan *p) { return p->grid_cap; }
 
-int am_items(const AmPlan *p) { return p->a.nitems; }
+int am_items(const AmPlan *p, bool plain) { return p->list[plain ? 1 : 0].n; }
 
 int am_ctas_per_sm(const AmPlan *p) {
     const size_t smem = am_launch_smem(p->a.nc);
@@ -932,11 +937,14 @@ int am_ctas_per_sm(const AmPlan *p) {
     return std::max(0, std::min(2, by_smem));
 }
 
-cudaError_t launch_async_multi(AmPlan *p, int storage, const void *vin, void *vout, int *ticket, int schedule,
-                               int grid, cudaStream_t stream) {
+cudaError_t launch_async_multi(AmPlan *p, bool plain, int storage, const void *vin, void *vout, int *ticket,
+                               int schedule, int grid, cudaStream_t stream) {
     // the scratch area holds the chunk boxes past tensor memory of grid_cap CTAs
     if (grid <= 0 || grid > p->grid_cap) return cudaErrorInvalidValue;
     AmArgs a = p->a;
+    const auto &l = p->list[plain ? 1 : 0];
+    a.items = l.items;
+    a.nitems = l.n;
     a.vin = vin;
     a.vout = vout;
     a.scratch = p->scratch;
@@ -946,9 +954,9 @@ cudaError_t launch_async_multi(AmPlan *p, int storage, const void *vin, void *vo
     const size_t smem = am_launch_smem(a.nc);
     void (*fn)(AmArgs) = nullptr;
     switch (storage) {
-        case kStoreF32: fn = pick<float>(p->k, p->pairs, p->ties); break;
-        case kStoreBF16: fn = pick<__nv_bfloat16>(p->k, p->pairs, p->ties); break;
-        case kStoreF16: fn = pick<__half>(p->k, p->pairs, p->ties); break;
+        case kStoreF32: fn = pick<float>(p->k, l.pairs, p->ties); break;
+        case kStoreBF16: fn = pick<__nv_bfloat16>(p->k, l.pairs, p->ties); break;
+        case kStoreF16: fn = pick<__half>(p->k, l.pairs, p->ties); break;
         default: return cudaErrorInvalidValue;
     }
     cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void *>(fn), smem);

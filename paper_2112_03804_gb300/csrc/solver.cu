@@ -852,7 +852,6 @@ kps_status kps_solver_create(kps_batch *b, kps_dtype dt, kps_solver **out) {
         }
         if (st != KPS_OK) { free_solver(s); return st; }
     }
-    if (dt != KPS_F64) batch_plain_ready(b, nullptr);
     // one iteration outside any capture sets every kernel attribute; then start over
     kps_status st = kps_solver_reset(s, nullptr, nullptr, nullptr);
     if (st == KPS_OK) st = one_iteration(s, nullptr);

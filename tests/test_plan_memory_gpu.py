@@ -97,3 +97,27 @@ def test_solver(monkeypatch):
     t.status()
     # FP32 rounding of the products, amplified by 17 iterations
     assert abs(float(e - f)) <= 1e-4 and abs(float(e - ref)) <= 1e-2 * float(ref)
+
+
+def test_solver_shares_the_batch_plans():
+    """A solver's products (plain rows) run on the batch's own plans: creating
+    one takes its state's memory, not a second set of records and scratch areas
+    (20 MB each)."""
+    def make():
+        b = kps.Batch([kps.Game(synth.river_spec(seed=3))])
+        x = torch.zeros(int(b.offsets(1)[-1]), device="cuda")
+        b.matvec_A(x, torch.zeros(int(b.offsets(0)[-1]), device="cuda"))
+        torch.cuda.synchronize()
+        return b
+
+    keep = kps.Solver(make(), kps.F32)          # loads every kernel
+    keep.step(2)
+    torch.cuda.synchronize()
+    b = make()
+    before, _ = torch.cuda.mem_get_info()
+    s = kps.Solver(b, kps.F32)
+    torch.cuda.synchronize()
+    after, _ = torch.cuda.mem_get_info()
+    assert before - after < 16 << 20
+    s.step(2)
+    s.status()
