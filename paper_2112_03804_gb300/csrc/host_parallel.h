@@ -1,0 +1,43 @@
+// Host work on many games by a few threads.
+#pragma once
+
+#include <algorithm>
+#include <atomic>
+#include <new>
+#include <thread>
+#include <vector>
+
+namespace kps {
+
+// fn(i) for every i in [0, n), on up to 8 threads, one for every 32768 hands (a
+// thread costs about as much as the records of 5000 hands, and its first
+// allocations as much again); the calling thread is one of them.  fn throws nothing but bad_alloc, which is passed on when all have
+// ended.  Every i is independent of the others, so results do not depend on the
+// threads.
+template <typename F>
+void parallel_for(int n, long long hands, F fn) {
+    const int threads =
+        std::max(1, (int)std::min<long long>({8, std::thread::hardware_concurrency(), n, hands / 32768}));
+    std::atomic<int> next{0};
+    std::atomic<bool> failed{false};
+    auto work = [&]() {
+        for (int i; !failed && (i = next.fetch_add(1)) < n;) {
+            try {
+                fn(i);
+            } catch (...) {
+                failed = true;
+            }
+        }
+    };
+    std::vector<std::thread> others;
+    try {
+        others.reserve(threads - 1);
+        for (int k = 1; k < threads; ++k) others.emplace_back(work);
+    } catch (...) {   // as many as there are
+    }
+    work();
+    for (std::thread &t : others) t.join();
+    if (failed) throw std::bad_alloc();
+}
+
+}  // namespace kps

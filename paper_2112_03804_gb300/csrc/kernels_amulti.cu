@@ -34,6 +34,7 @@
 // hardware), no atomics on results: bit-reproducible.
 #include "kernels.h"
 #include "game.h"
+#include "host_parallel.h"
 #include "scan_records.h"
 
 #include <cuda_bf16.h>
@@ -707,18 +708,24 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
     int nc = 0, ntaken = 0;
     size_t rbytes = 0;
     const int k = games[0].h->k;
-    for (int i = 0; i < ng; ++i) {
-        const AmGameDesc &d = games[i];
-        if (d.h->k != k) {
+    for (int i = 0; i < ng; ++i)
+        if (games[i].h->k != k) {
             *why = "games with different hand sizes";
             return nullptr;
         }
-        std::string w = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, true, &rec[i]);
-        if (w.empty() && rec[i].hs % 8 != 0) w = "hand stride not a multiple of 8";
-        if (!w.empty()) {
+    std::vector<std::string> refused(ng);
+    long long hands = 0;
+    for (int i = 0; i < ng; ++i) hands += games[i].h->H;
+    parallel_for(ng, hands, [&](int i) {
+        const AmGameDesc &d = games[i];
+        refused[i] = build_scan_records(*d.h, d.lam_in, d.lam_out, kMaxExtra, true, &rec[i]);
+        if (refused[i].empty() && rec[i].hs % 8 != 0) refused[i] = "hand stride not a multiple of 8";
+        if (!refused[i].empty()) rec[i] = ScanRecords();
+    });
+    for (int i = 0; i < ng; ++i) {
+        if (!refused[i].empty()) {
             // left to another kernel
-            if (why->empty()) *why = "game " + std::to_string(i) + ": " + w;
-            rec[i] = ScanRecords();
+            if (why->empty()) *why = "game " + std::to_string(i) + ": " + refused[i];
             continue;
         }
         (*taken)[i] = 1;
@@ -735,8 +742,8 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
     std::vector<char> can_split(ng, 0);
     std::vector<std::array<int, 2 * kTmaWarps + 1>> sub(ng);
     std::vector<std::vector<int2>> paired(ng);
-    for (int i = 0; i < ng; ++i) {
-        if (!(*taken)[i]) continue;
+    parallel_for(ng, hands, [&](int i) {
+        if (!(*taken)[i]) return;
         const AmGameDesc &d = games[i];
         const ScanRecords &r = rec[i];
         // sub-chunks of split items: each chunk cut at the tie-free box
@@ -779,7 +786,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
         }
         for (int s = 0; s < d.n_out; ++s)
             if (d.hfcol[s] >= 0 && !mated[s]) paired[i].push_back(make_int2(s, -1));
-    }
+    });
     // estimated time of a layout (see kItemTime), its items in *out
     auto layout = [&](bool pairs, bool halves, std::vector<int4> *out) {
         double sum = 0.0, alone = 0.0, longest = 0.0;
@@ -831,6 +838,14 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
     const size_t total = o_rec + rbytes;
     std::vector<unsigned char> host(total, 0);
     std::vector<AmGame> g(ng);
+    std::vector<size_t> rec_at(ng), rows_at(ng);
+    for (size_t i = 0, ro = o_rec, rowo = o_rows; i < (size_t)ng; ++i) {
+        rec_at[i] = ro;
+        rows_at[i] = rowo;
+        if (!(*taken)[i]) continue;
+        ro += al(rec[i].bytes.size());
+        if (pairs) rowo += sizeof(int2) * paired[i].size();
+    }
     const size_t scratch = (size_t)grid_cap * kTmaWarps * kMaxExtra * kTmaBox * 32 * sizeof(float);
     AmPlan *p = new AmPlan();
     cudaError_t e = device_malloc(&p->blob, total);
@@ -844,20 +859,19 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
     }
     p->grid_cap = grid_cap;
     unsigned char *dev = static_cast<unsigned char *>(p->blob);
-    size_t ro = o_rec, rowo = o_rows;
-    for (int i = 0; i < ng; ++i) {
+    parallel_for(ng, hands, [&](int i) {
         const AmGameDesc &d = games[i];
         const ScanRecords &r = rec[i];
         AmGame &x = g[i];
         std::memset(&x, 0, sizeof(x));
-        if (!(*taken)[i]) continue;
+        if (!(*taken)[i]) return;
+        const size_t ro = rec_at[i];
         x.H = r.H;
         x.hs = r.hs;
         x.nc = r.nc;
         if (pairs) {
-            std::memcpy(host.data() + rowo, paired[i].data(), sizeof(int2) * paired[i].size());
-            x.rows = reinterpret_cast<const int2 *>(dev + rowo);
-            rowo += sizeof(int2) * paired[i].size();
+            std::memcpy(host.data() + rows_at[i], paired[i].data(), sizeof(int2) * paired[i].size());
+            x.rows = reinterpret_cast<const int2 *>(dev + rows_at[i]);
         }
         for (int w = 0; w <= 2 * kTmaWarps; ++w) x.bchunk8[w] = sub[i][w];
         x.nbox = r.nbox;
@@ -872,8 +886,7 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
         x.rscan = dev + ro;
         x.rfin = reinterpret_cast<const TmaFinRec *>(dev + ro + (size_t)r.nbox * kScanBlock);
         x.ent = reinterpret_cast<const TieEntry *>(dev + ro + r.entries_at);
-        ro += al(r.bytes.size());
-    }
+    });
     std::memcpy(host.data() + o_games, g.data(), sizeof(AmGame) * ng);
     for (int l = 0, at = 0; l < 2; at += (int)items[l].size(), ++l)
         if (!items[l].empty())

@@ -32,6 +32,7 @@
 // chunks may cut tie groups.  No atomics: results are bit-reproducible.
 #include "kernels.h"
 #include "game.h"
+#include "host_parallel.h"
 
 #include <cuda_runtime.h>
 
@@ -379,8 +380,6 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
                     size_t *need) {
     *need = 0;
     const int ng = (int)games.size();
-    std::vector<std::vector<unsigned char>> rec(ng);
-    std::vector<size_t> ties_at(ng);
     std::vector<std::vector<int2>> rows(ng);
     std::vector<Game> g(ng);
     std::vector<int4> items;
@@ -388,16 +387,30 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
     int nc = 0, dev = 0, sms = 1;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     size_t rbytes = 0, nrows = 0;
+    long long hands = 0;
     for (int i = 0; i < ng; ++i) {
+        nc = std::max(nc, games[i].h->ncards + 1);
+        hands += games[i].h->H;
+    }
+    std::vector<std::vector<RecBox>> rec(ng);
+    std::vector<std::vector<Tie>> listed(ng);
+    std::vector<std::string> refused(ng);
+    std::atomic<bool> fits{true};
+    parallel_for(ng, hands, [&](int i) {
         const F64GameDesc &d = games[i];
         const HostGame &h = *d.h;
-        if (h.k != 2) { *why = "one-card hands"; return nullptr; }
-        if (h.hs % kBox != 0) { *why = "hand stride"; return nullptr; }
-        nc = std::max(nc, h.ncards + 1);
+        auto refuse = [&](const char *w) {
+            refused[i] = w;
+            fits = false;
+        };
+        if (!fits) return;   // another game is refused: so is the batch
+        if (h.k != 2) return refuse("one-card hands");
+        if (h.hs % kBox != 0) return refuse("hand stride");
         const int nbox = h.hs / kBox;
-        std::vector<RecBox> rb(nbox);
-        std::memset(rb.data(), 0, sizeof(RecBox) * nbox);
-        std::vector<Tie> ties;
+        std::vector<RecBox> &rb = rec[i];
+        rb.resize(nbox);     // (zeros)
+        std::vector<Tie> &ties = listed[i];
+        ties.reserve(h.H / 4);
         auto card = [&](int x, int j) { return h.hand_slots[2 * x + j]; };
         auto share = [&](int x, int y) {
             return card(x, 0) == card(y, 0) || card(x, 0) == card(y, 1) || card(x, 1) == card(y, 0) ||
@@ -434,18 +447,13 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
             rb[b].count = n;
         }
         // on average at most two corrections a hand
-        if (ties.size() > 2 * (size_t)h.H) { *why = "many tied hands"; return nullptr; }
-        rec[i].resize(sizeof(RecBox) * nbox + sizeof(Tie) * ties.size());
-        std::memcpy(rec[i].data(), rb.data(), sizeof(RecBox) * nbox);
-        ties_at[i] = sizeof(RecBox) * nbox;
-        if (!ties.empty()) std::memcpy(rec[i].data() + ties_at[i], ties.data(), sizeof(Tie) * ties.size());
-        rbytes += al(rec[i].size());
+        if (ties.size() > 2 * (size_t)h.H) return refuse("many tied hands");
         // rows: showdown-only sequences with the fold-only one of their input row, then the others
         std::vector<int> fold_of;
         std::vector<char> mated(d.n_out, 0);
         for (int s = 0; s < d.n_out; ++s) {
             const int c = std::max(d.hfcol[s], d.hscol[s]);
-            if (c < 0) { *why = "an output sequence without terminals"; return nullptr; }
+            if (c < 0) return refuse("an output sequence without terminals");
             if (c >= (int)fold_of.size()) fold_of.resize(c + 1, -1);
             if (d.hscol[s] < 0) fold_of[d.hfcol[s]] = s;
         }
@@ -460,6 +468,13 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         for (int s = 0; s < d.n_out; ++s)
             if (d.hfcol[s] >= 0 && !mated[s]) rows[i].push_back(make_int2(s, -1));
         g[i].nrows = (int)rows[i].size();
+    });
+    for (int i = 0; i < ng; ++i) {
+        if (!refused[i].empty()) {
+            *why = refused[i];
+            return nullptr;
+        }
+        rbytes += al(sizeof(RecBox) * rec[i].size() + sizeof(Tie) * listed[i].size());
         nrows += rows[i].size();
     }
     if (smem_bytes(nc) > (size_t)max_dyn_smem()) { *why = "shared memory"; return nullptr; }
@@ -499,10 +514,17 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         }
         build(least, &items);
     }
-    F64Plan *p = new (std::nothrow) F64Plan();
-    if (!p) { *why = "host allocation"; *need = 1; return nullptr; }
     const size_t o_items = al(sizeof(Game) * ng), o_rows = o_items + al(sizeof(int4) * items.size()),
                  o_rec = o_rows + al(sizeof(int2) * nrows), total = o_rec + rbytes;
+    std::vector<unsigned char> host(total, 0);
+    std::vector<size_t> rec_at(ng), rows_at(ng);
+    for (size_t i = 0, ro = o_rec, rowo = o_rows; i < (size_t)ng; ++i) {
+        rec_at[i] = ro;
+        rows_at[i] = rowo;
+        ro += al(sizeof(RecBox) * rec[i].size() + sizeof(Tie) * listed[i].size());
+        rowo += sizeof(int2) * rows[i].size();
+    }
+    F64Plan *p = new F64Plan();
     cudaError_t e = device_malloc(&p->blob, total);
     if (e != cudaSuccess) {
         delete p;
@@ -511,9 +533,7 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         return nullptr;
     }
     unsigned char *b = static_cast<unsigned char *>(p->blob);
-    std::vector<unsigned char> host(total, 0);
-    size_t ro = o_rec, rowo = o_rows;
-    for (int i = 0; i < ng; ++i) {
+    parallel_for(ng, hands, [&](int i) {
         const F64GameDesc &d = games[i];
         Game &x = g[i];
         x.H = d.h->H;
@@ -527,14 +547,14 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         x.scol = d.scol;
         x.fcoef = d.fcoef;
         x.scoef = d.scoef;
-        if (!rows[i].empty()) std::memcpy(host.data() + rowo, rows[i].data(), sizeof(int2) * rows[i].size());
-        x.rows = reinterpret_cast<const int2 *>(b + rowo);
-        rowo += sizeof(int2) * rows[i].size();
-        std::memcpy(host.data() + ro, rec[i].data(), rec[i].size());
-        x.rec = reinterpret_cast<const RecBox *>(b + ro);
-        x.ties = reinterpret_cast<const Tie *>(b + ro + ties_at[i]);
-        ro += al(rec[i].size());
-    }
+        if (!rows[i].empty()) std::memcpy(host.data() + rows_at[i], rows[i].data(), sizeof(int2) * rows[i].size());
+        x.rows = reinterpret_cast<const int2 *>(b + rows_at[i]);
+        const size_t ties_at = rec_at[i] + sizeof(RecBox) * rec[i].size();
+        std::memcpy(host.data() + rec_at[i], rec[i].data(), sizeof(RecBox) * rec[i].size());
+        if (!listed[i].empty()) std::memcpy(host.data() + ties_at, listed[i].data(), sizeof(Tie) * listed[i].size());
+        x.rec = reinterpret_cast<const RecBox *>(b + rec_at[i]);
+        x.ties = reinterpret_cast<const Tie *>(b + ties_at);
+    });
     std::memcpy(host.data(), g.data(), sizeof(Game) * ng);
     if (!items.empty()) std::memcpy(host.data() + o_items, items.data(), sizeof(int4) * items.size());
     e = cudaMemcpyAsync(p->blob, host.data(), total, cudaMemcpyHostToDevice, stream);
