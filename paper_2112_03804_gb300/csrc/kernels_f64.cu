@@ -363,6 +363,7 @@ struct F64Plan {
     int nitems = 0;                // many games
     int nunit = 0, nother = 0;     // one game: rows by kind
     int nbox = 0;                  // and its boxes
+    int sms = 1;                   // of the device
 };
 
 namespace {
@@ -412,10 +413,9 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         std::vector<Tie> &ties = listed[i];
         ties.reserve(h.H / 4);
         auto card = [&](int x, int j) { return h.hand_slots[2 * x + j]; };
-        auto share = [&](int x, int y) {
-            return card(x, 0) == card(y, 0) || card(x, 0) == card(y, 1) || card(x, 1) == card(y, 0) ||
-                   card(x, 1) == card(y, 1);
-        };
+        // the hands' cards as bits (a deck has at most 63)
+        std::vector<uint64_t> cards(h.H);
+        for (int x = 0; x < h.H; ++x) cards[x] = 1ull << card(x, 0) | 1ull << card(x, 1);
         for (int b = 0; b < nbox; ++b) {
             for (int k = 0; k < kBox / 2; ++k) {
                 Rec &r = rb[b].r[k];
@@ -438,7 +438,7 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
             uint32_t n = 0;
             for (int x = kBox * b; x < std::min(h.H, kBox * b + kBox); ++x)
                 for (int q = h.group_lo[x]; q <= h.group_hi[x]; ++q)
-                    if (q != x && !share(x, q)) {
+                    if (q != x && (cards[x] & cards[q]) == 0) {
                         const Tie t{x - kBox * b, q, q > x ? d.lam_in[q] : -d.lam_in[q]};
                         if (n < kInline) rb[b].t[n] = t;
                         else ties.push_back(t);
@@ -568,6 +568,7 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
     p->a.games = reinterpret_cast<const Game *>(b);
     p->a.items = multi ? reinterpret_cast<const int4 *>(b + o_items) : nullptr;
     p->a.nc = nc;
+    p->sms = sms;
     p->nitems = (int)items.size();
     if (!multi) {
         p->nunit = g[0].nunit;
@@ -592,10 +593,7 @@ cudaError_t launch_f64_scan(F64Plan *p, const double *vin, double *vout, int bat
     a.batch = batch;
     long long n = p->nitems;
     if (!a.items) {
-        int dev = 0, sms = 1;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
+        const int sms = p->sms;
         const long long cu = (long long)p->nunit * batch, co = (long long)p->nother * batch;
         if (std::max(cu, co) > 0x7fffffe0LL) return cudaErrorInvalidValue;
         // the parts whose waves of items are shortest: 60 vectors of the river

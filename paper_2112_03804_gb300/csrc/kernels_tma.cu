@@ -127,6 +127,7 @@ struct TmaParams {
     bool eight = false;            // the eight-warp shape fits
     bool alone = false;            // one CTA of the four-warp shape fills an SM
     int extra4 = 0;                // overflow boxes of the four-warp shape
+    int sms = 1;                   // of the device
     int device = -1;
 };
 
@@ -1028,12 +1029,16 @@ cudaError_t tma_upload(TmaParams *pp, cudaStream_t stream) {
     if (p.dev) return cudaSuccess;
     cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p.a.err), g_tma_err);
     if (e != cudaSuccess) return e;
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     e = upload_table(&p.dev, p.host.data(), p.host.size(), stream);
     if (e != cudaSuccess) return e;
     p.a.rscan = static_cast<const unsigned char *>(p.dev);
     p.a.rfin = reinterpret_cast<const TmaFinRec *>(static_cast<const unsigned char *>(p.dev) +
                                                    (size_t)p.a.nbox * kScanBlock);
-    cudaGetDevice(&p.device);
+    p.device = dev;
     return cudaSuccess;
 }
 
@@ -1051,10 +1056,7 @@ cudaError_t launch_tma_scan(TmaParams *pp, int storage, const void *vin, void *v
     e = encode3(&A.tin, storage, vin, A.H, A.n_in, batch, A.hs);
     if (e == cudaSuccess) e = encode3(&A.tout, storage, vout, A.hs, A.n_out, batch, A.hs);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 1;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
+    const int sms = p.sms;
     // Shape.  Eight warps (half as long a scan per warp) while every single item
     // has an SM to itself: 1 FP32 vector 26.6 -> 20.5 us, 96 vectors 28.8 ->
     // 22.6 us.  Else four warps, and pairs where they save a wave of two CTAs

@@ -58,12 +58,11 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
         if (hand >= H || j >= h.k) return (uint32_t)h.ncards * 128u;
         return (uint32_t)card(hand, j) * 128u;
     };
-    auto share = [&](int x, int y) {   // any card of hand y in hand x
-        for (int j = 0; j < h.k; ++j)
-            for (int l = 0; l < h.k; ++l)
-                if (card(x, j) == card(y, l)) return true;
-        return false;
-    };
+    // the hands' cards as bits (at most 63 cards)
+    std::vector<uint64_t> cards(H);
+    for (int i = 0; i < H; ++i)
+        for (int j = 0; j < h.k; ++j) cards[i] |= 1ull << card(i, j);
+    auto share = [&](int x, int y) { return (cards[x] & cards[y]) != 0; };
     std::vector<TieEntry> entries;
     size_t chunk_first = 0;
     for (int bx = 0; bx < nbox; ++bx) {
