@@ -765,27 +765,12 @@ AmPlan *build_plan(const std::vector<AmGameDesc> &games, int grid_cap, cudaStrea
             can_split[i] = can_split[i] && mid - lo <= 16 && hi - mid <= 16;
         }
         sub[i][2 * kTmaWarps] = r.nbox;
-        // fold_of[c]: the fold-only sequence that reads input row c
-        std::vector<char> mated(d.n_out, 0);
-        std::vector<int> fold_of;
-        for (int s = 0; s < d.n_out; ++s) {
-            const int c = std::max(d.hfcol[s], d.hscol[s]);
-            if (c >= (int)fold_of.size()) fold_of.resize(c + 1, -1);
-            if (d.hfcol[s] >= 0 && d.hscol[s] < 0) fold_of[d.hfcol[s]] = s;
-        }
+        const std::vector<int> mate = fold_mates(d.n_out, d.hfcol, d.hscol);
         paired[i].reserve(d.n_out);
-        for (int s = 0; s < d.n_out; ++s) {
-            if (d.hfcol[s] >= 0) continue;
-            int2 row = make_int2(s, -1);
-            if (d.hscol[s] >= 0) {
-                row.y = fold_of[d.hscol[s]];
-                if (row.y >= 0 && mated[row.y]) row.y = -1;
-                if (row.y >= 0) mated[row.y] = 1;
-            }
-            paired[i].push_back(row);
-        }
         for (int s = 0; s < d.n_out; ++s)
-            if (d.hfcol[s] >= 0 && !mated[s]) paired[i].push_back(make_int2(s, -1));
+            if (d.hfcol[s] < 0) paired[i].push_back(make_int2(s, mate[s]));
+        for (int s = 0; s < d.n_out; ++s)
+            if (d.hfcol[s] >= 0 && mate[s] != kMate) paired[i].push_back(make_int2(s, -1));
     });
     // estimated time of a layout (see kItemTime), its items in *out
     auto layout = [&](bool pairs, bool halves, std::vector<int4> *out) {

@@ -33,6 +33,7 @@
 #include "kernels.h"
 #include "game.h"
 #include "host_parallel.h"
+#include "scan_records.h"
 
 #include <cuda_runtime.h>
 
@@ -449,24 +450,14 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         // on average at most two corrections a hand
         if (ties.size() > 2 * (size_t)h.H) return refuse("many tied hands");
         // rows: showdown-only sequences with the fold-only one of their input row, then the others
-        std::vector<int> fold_of;
-        std::vector<char> mated(d.n_out, 0);
-        for (int s = 0; s < d.n_out; ++s) {
-            const int c = std::max(d.hfcol[s], d.hscol[s]);
-            if (c < 0) return refuse("an output sequence without terminals");
-            if (c >= (int)fold_of.size()) fold_of.resize(c + 1, -1);
-            if (d.hscol[s] < 0) fold_of[d.hfcol[s]] = s;
-        }
-        for (int s = 0; s < d.n_out; ++s) {
-            if (d.hfcol[s] >= 0) continue;
-            int f = fold_of[d.hscol[s]];
-            if (f >= 0 && mated[f]) f = -1;
-            if (f >= 0) mated[f] = 1;
-            rows[i].push_back(make_int2(s, f));
-        }
+        for (int s = 0; s < d.n_out; ++s)
+            if (d.hfcol[s] < 0 && d.hscol[s] < 0) return refuse("an output sequence without terminals");
+        const std::vector<int> mate = fold_mates(d.n_out, d.hfcol, d.hscol);
+        for (int s = 0; s < d.n_out; ++s)
+            if (d.hfcol[s] < 0) rows[i].push_back(make_int2(s, mate[s]));
         g[i].nunit = (int)rows[i].size();
         for (int s = 0; s < d.n_out; ++s)
-            if (d.hfcol[s] >= 0 && !mated[s]) rows[i].push_back(make_int2(s, -1));
+            if (d.hfcol[s] >= 0 && mate[s] != kMate) rows[i].push_back(make_int2(s, -1));
         g[i].nrows = (int)rows[i].size();
     });
     for (int i = 0; i < ng; ++i) {

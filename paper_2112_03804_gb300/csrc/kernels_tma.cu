@@ -943,8 +943,7 @@ static std::string tma_prepare(const HostGame &h, const double *lam_in, const do
     return "";
 }
 
-// Items after the records: first the pairs (a fold-only sequence goes with the
-// first showdown-only one of its input row) and what is left alone, then every
+// Items after the records: first the pairs and what is left alone, then every
 // sequence alone.
 std::string tma_items(int n_out, const int *hfcol, const int *hscol, const double *fcoef, const double *scoef,
                       TmaParams &p) {
@@ -953,23 +952,12 @@ std::string tma_items(int n_out, const int *hfcol, const int *hscol, const doubl
         items.push_back(TmaItem{r, q, hfcol[r], hscol[r], hfcol[r] >= 0 ? (float)fcoef[r] : 0.f,
                                 hscol[r] >= 0 ? (float)scoef[r] : 0.f, q >= 0 ? (float)fcoef[q] : 0.f, 0});
     };
-    std::vector<int> fold_of;   // by input row: its first fold-only sequence, -1 once taken
-    std::vector<int> mate(n_out, -1);
-    std::vector<char> taken(n_out, 0);
-    for (int r = 0; r < n_out; ++r) {
-        if (hfcol[r] < 0 && hscol[r] < 0) return "an output sequence without terminals";
-        if (hscol[r] >= 0 || p.a.nc < kPairMinCards) continue;
-        if (hfcol[r] >= (int)fold_of.size()) fold_of.resize(hfcol[r] + 1, -1);
-        if (fold_of[hfcol[r]] < 0) fold_of[hfcol[r]] = r;
-    }
-    for (int r = 0; r < n_out; ++r) {
-        if (hfcol[r] >= 0 || hscol[r] >= (int)fold_of.size()) continue;
-        mate[r] = fold_of[hscol[r]];
-        fold_of[hscol[r]] = -1;
-        if (mate[r] >= 0) taken[mate[r]] = 1;
-    }
     for (int r = 0; r < n_out; ++r)
-        if (!taken[r]) add(r, mate[r]);
+        if (hfcol[r] < 0 && hscol[r] < 0) return "an output sequence without terminals";
+    std::vector<int> mate(n_out, -1);
+    if (p.a.nc >= kPairMinCards) mate = fold_mates(n_out, hfcol, hscol);
+    for (int r = 0; r < n_out; ++r)
+        if (mate[r] != kMate) add(r, mate[r]);
     p.npaired = (int)items.size();
     p.nsingle = n_out;
     for (int r = 0; r < n_out; ++r) add(r, -1);

@@ -7,6 +7,24 @@
 
 namespace kps {
 
+std::vector<int> fold_mates(int n_out, const int *hfcol, const int *hscol) {
+    std::vector<int> mate(n_out, -1), fold_of;   // by input row: its first fold-only sequence, -1 once taken
+    for (int s = 0; s < n_out; ++s) {
+        if (hfcol[s] < 0 || hscol[s] >= 0) continue;
+        if (hfcol[s] >= (int)fold_of.size()) fold_of.resize(hfcol[s] + 1, -1);
+        if (fold_of[hfcol[s]] < 0) fold_of[hfcol[s]] = s;
+    }
+    for (int s = 0; s < n_out; ++s) {
+        if (hfcol[s] >= 0 || hscol[s] < 0 || hscol[s] >= (int)fold_of.size()) continue;
+        const int f = fold_of[hscol[s]];
+        if (f < 0) continue;
+        mate[s] = f;
+        mate[f] = kMate;
+        fold_of[hscol[s]] = -1;
+    }
+    return mate;
+}
+
 std::string build_scan_records(const HostGame &h, const double *lam_in, const double *lam_out, int max_extra,
                                bool long_ties, ScanRecords *out) {
     ScanRecords &R = *out;

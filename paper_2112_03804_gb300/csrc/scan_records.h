@@ -62,6 +62,15 @@ struct ScanRecords {
     std::vector<unsigned char> bytes;
 };
 
+// Pairs of output sequences with one input row: where a player answers a bet by a
+// fold or a call, both answers read the bet's row, one as a fold-only and one as
+// a showdown-only sequence (hfcol, hscol: a sequence's fold / showdown input row or
+// -1).  Returns for every sequence the fold-only one of its pair (a showdown-only
+// sequence takes the first fold-only one of its row that is not taken), kMate
+// for a fold-only sequence that is in one, and -1 for one left alone.
+constexpr int kMate = -2;
+std::vector<int> fold_mates(int n_out, const int *hfcol, const int *hscol);
+
 // Empty string on success, else why the game does not fit these kernels
 // (tie group over 4 hands or, with long_ties, more than kMaxTieEntries pairs in a
 // chunk; more than 64 card rows; a chunk longer than 16 + max_extra boxes).
