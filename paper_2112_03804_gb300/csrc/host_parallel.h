@@ -16,8 +16,9 @@ namespace kps {
 // threads.
 template <typename F>
 void parallel_for(int n, long long hands, F fn) {
-    const int threads =
-        std::max(1, (int)std::min<long long>({8, std::thread::hardware_concurrency(), n, hands / 32768}));
+    int threads = (int)std::min<long long>({8, n, hands / 32768});
+    // (asking for the number of cores takes 15 us: one game's plan does not)
+    if (threads > 1) threads = std::min(threads, (int)std::thread::hardware_concurrency());
     std::atomic<int> next{0};
     std::atomic<bool> failed{false};
     auto work = [&]() {
@@ -31,7 +32,7 @@ void parallel_for(int n, long long hands, F fn) {
     };
     std::vector<std::thread> others;
     try {
-        others.reserve(threads - 1);
+        if (threads > 1) others.reserve(threads - 1);
         for (int k = 1; k < threads; ++k) others.emplace_back(work);
     } catch (...) {   // as many as there are
     }

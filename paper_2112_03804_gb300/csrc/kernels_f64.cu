@@ -414,9 +414,8 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
         std::vector<Tie> &ties = listed[i];
         ties.reserve(h.H / 4);
         auto card = [&](int x, int j) { return h.hand_slots[2 * x + j]; };
-        // the hands' cards as bits (a deck has at most 63)
-        std::vector<uint64_t> cards(h.H);
-        for (int x = 0; x < h.H; ++x) cards[x] = 1ull << card(x, 0) | 1ull << card(x, 1);
+        // a hand's cards as bits (a deck has at most 63)
+        auto cards = [&](int x) { return 1ull << card(x, 0) | 1ull << card(x, 1); };
         for (int b = 0; b < nbox; ++b) {
             for (int k = 0; k < kBox / 2; ++k) {
                 Rec &r = rb[b].r[k];
@@ -439,7 +438,7 @@ F64Plan *f64_create(const std::vector<F64GameDesc> &games, bool multi, cudaStrea
             uint32_t n = 0;
             for (int x = kBox * b; x < std::min(h.H, kBox * b + kBox); ++x)
                 for (int q = h.group_lo[x]; q <= h.group_hi[x]; ++q)
-                    if (q != x && (cards[x] & cards[q]) == 0) {
+                    if (q != x && (cards(x) & cards(q)) == 0) {
                         const Tie t{x - kBox * b, q, q > x ? d.lam_in[q] : -d.lam_in[q]};
                         if (n < kInline) rb[b].t[n] = t;
                         else ties.push_back(t);

@@ -76,11 +76,9 @@ std::string build_scan_records(const HostGame &h, const double *lam_in, const do
         if (hand >= H || j >= h.k) return (uint32_t)h.ncards * 128u;
         return (uint32_t)card(hand, j) * 128u;
     };
-    // the hands' cards as bits (at most 63 cards)
-    std::vector<uint64_t> cards(H);
-    for (int i = 0; i < H; ++i)
-        for (int j = 0; j < h.k; ++j) cards[i] |= 1ull << card(i, j);
-    auto share = [&](int x, int y) { return (cards[x] & cards[y]) != 0; };
+    // a hand's cards as bits (at most 63 cards)
+    auto cards = [&](int x) { return 1ull << card(x, 0) | (h.k == 2 ? 1ull << card(x, 1) : 0); };
+    auto share = [&](int x, int y) { return (cards(x) & cards(y)) != 0; };
     std::vector<TieEntry> entries;
     size_t chunk_first = 0;
     for (int bx = 0; bx < nbox; ++bx) {
