@@ -657,15 +657,16 @@ __global__ void __launch_bounds__(128, 2) async_multi_kernel(const __grid_consta
 
 // Time (us) of an item [single rows, pairs][full, split] of a 1081-hand game in
 // FP32, {alone on its SM, two per SM}, measured on 1 to 600 river games and 20 games
-// of 247 sequences (a full item of pairs alone: 39.3 and 44.2): what am_create's
-// choice of rows and items goes by.  16-bit vectors take 0.75 to 0.8
+// of 247 sequences (a full item of pairs alone: 39.3 and 44.2; two per SM 62 where
+// every row is a pair, less in uneven games): what am_create's choice of rows and
+// items goes by.  16-bit vectors take 0.75 to 0.8
 // of every entry, and 1128 and 1176 hands a few percent more, so the choice is the
 // same; games of some ten hands, whose items are bound by their fixed parts,
 // take single rows in full items by it too, which is the fastest there (300
-// one-card games of 47 hands 9.4 us; pairs 10.1, split items 18.4).  A choice
-// of mixed games is off by up to a tenth: 200 games of 3 to 5 board cards take
-// 83 us by it, 75 with pairs in split items; 512 take 158 (164 with pairs).
-constexpr double kItemTime[2][2][2] = {{{29.5, 45.5}, {19.5, 27.8}}, {{42, 62}, {26.5, 39.6}}};
+// one-card games of 47 hands 9.4 us; pairs 10.1, split items 18.4).  Uneven games (3 to
+// 5 board cards): 200 games take 81 us by it (75 with pairs in split items), 512
+// 155 (161 with pairs), 1500 404 and 4096 1055 with pairs (406 and 1077 without).
+constexpr double kItemTime[2][2][2] = {{{29.5, 45.5}, {19.5, 27.8}}, {{42, 60}, {26.5, 39.6}}};
 
 namespace {
 template <typename T>
