@@ -14,8 +14,8 @@
 // and the pipe must never wait: six warps per SM, each with its own per-card
 // table.  The kernel it replaces (kernels_vec.cu, still taken where this one
 // does not apply) had three warps per SM and several times the instructions:
-// 100 vectors of the 1081-hand river game 436 -> 215 us, one product of 64 such
-// games 514 -> 132 us.
+// 100 vectors of the 1081-hand river game 432 -> 214 us, one product of 64 such
+// games 514 -> 122 us.
 //
 // Organisation.  A CTA = one item: up to 32 columns (row, vector) of one game
 // and one kind, lane = column; or up to 16 (8) columns, their two (four) groups

@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(256, 1) predict_kernel(const PredictArgs a) {
     // forward (no search), and consecutive rows mostly share game and node: their
     // part of layer 1 is formed once.  The rows of the next tile are looked up
     // while the tensor cores run layer 2.  4.15 M queries of 128 games: 4.82 ms
-    // with a search and four gathered parts per row, 3.24 ms now.
+    // with a search and four gathered parts per row, 3.20 ms now.
     const long long ntiles = (a.nq + kPR - 1) / kPR;
     const long long t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
     int game = tid < kPR && t0 < t1 ? decode(a.d, min(t0 * kPR + tid, a.nq - 1)).game : 0;   // of this thread's row
